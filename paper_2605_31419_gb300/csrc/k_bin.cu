@@ -10,8 +10,8 @@
 //  3. each pair is placed in its tile's segment (shared-memory atomics on the block's places, or
 //     global atomic cursors) as the 64-bit key (float bits of the depth key << 32 | face id),
 //     unique within a tile;
-//  4. each segment is sorted by that key (bitonic networks: one warp in registers up to 64 pairs,
-//     one warp in shared memory up to 512, one CTA beyond), and written out as the pair list:
+//  4. each segment is sorted by that key (one warp's registers up to 512 pairs, one CTA beyond: runs
+//     of 128 sorted in registers, then merged in shared memory), and written out as the pair list:
 //     key (global tile id << 32 | depth bits) and face id, ascending depth with ties in ascending
 //     face id -- the order a stable sort of the (view, face)-ordered pairs by (tile, depth) gives.
 // Every kernel reads the pair count from the device, so nothing here synchronises the host.
@@ -303,9 +303,9 @@ __global__ void __launch_bounds__(BIN_T) k_bin_place(MatArgs a) {
   }
 }
 
-// Step 4.  Bitonic networks in the form whose every compare-exchange moves the smaller key to the
-// lower index (each merge starts by comparing mirrored positions), so that the positions past a
-// segment's end can stand for +infinity without being stored: a pair with one of them never moves.
+// Step 4.  In registers, bitonic networks in the form whose every compare-exchange moves the smaller key to
+// the lower index (each merge starts by comparing mirrored positions); positions past a segment's end
+// hold +infinity and stay behind its keys.
 struct SortOut {
   const unsigned long long* seg;
   unsigned long long* keys;
@@ -324,11 +324,87 @@ __device__ __forceinline__ void put_pair(const SortOut& o, long long t, long lon
   o.vals[pos] = (uint32_t)k;
 }
 
-constexpr int WARP_SORT_MAX = 512;  // pairs a warp sorts in its shared memory (32 KB per block)
+constexpr int WARP_SORT_MAX = 512;  // pairs a warp sorts in its registers (16 per lane)
 constexpr int SORT_WARPS_PER_BLOCK = 8;
 
-// One warp per tile: up to 32 pairs in registers, up to WARP_SORT_MAX in shared memory; longer
-// segments are listed for the CTA-wide kernel.
+// Keep the smaller (lower) or the larger key of a compare-exchange with a lane that keeps the other.
+__device__ __forceinline__ unsigned long long keep_key(unsigned long long x, unsigned long long y, bool lower) {
+  return (y < x) == lower ? y : x;
+}
+__device__ __forceinline__ void cmp_exchange(unsigned long long& a, unsigned long long& b) {
+  const bool sw = b < a;
+  const unsigned long long lo = sw ? b : a, hi = sw ? a : b;
+  a = lo;
+  b = hi;
+}
+
+// Sort a warp's 32 * K keys, K per lane, so that position lane * K + r holds the ascending order.
+// Exchanges at distances below K stay in the lane's registers, the others are lane shuffles: of the
+// 36 steps of 256 keys 21 need no shuffle, and nothing touches shared memory or divides an index.
+template <int K>
+__device__ __forceinline__ void warp_sort(unsigned long long (&x)[K], int lane) {
+#pragma unroll
+  for (int k = 2; k <= K; k <<= 1) {  // within the lane
+#pragma unroll
+    for (int r = 0; r < K; ++r)
+      if ((r & (k >> 1)) == 0) cmp_exchange(x[r], x[r ^ (k - 1)]);
+#pragma unroll
+    for (int j = k >> 2; j > 0; j >>= 1)
+#pragma unroll
+      for (int r = 0; r < K; ++r)
+        if ((r & j) == 0) cmp_exchange(x[r], x[r ^ j]);
+  }
+#pragma unroll 1
+  for (int kl = 2; kl <= 32; kl <<= 1) {  // merges of kl lanes' keys
+    {  // mirrored positions: lane ^ (kl - 1), register K - 1 - r
+      const bool lower = (lane & (kl >> 1)) == 0;
+#pragma unroll
+      for (int r = 0; r < K / 2; ++r) {
+        const unsigned long long y0 = __shfl_xor_sync(0xffffffffu, x[K - 1 - r], kl - 1);
+        const unsigned long long y1 = __shfl_xor_sync(0xffffffffu, x[r], kl - 1);
+        x[r] = keep_key(x[r], y0, lower);
+        x[K - 1 - r] = keep_key(x[K - 1 - r], y1, lower);
+      }
+    }
+#pragma unroll 1
+    for (int j = kl >> 2; j > 0; j >>= 1) {
+      const bool lower = (lane & j) == 0;
+#pragma unroll
+      for (int r = 0; r < K; ++r) x[r] = keep_key(x[r], __shfl_xor_sync(0xffffffffu, x[r], j), lower);
+    }
+#pragma unroll
+    for (int j = K >> 1; j > 0; j >>= 1)
+#pragma unroll
+      for (int r = 0; r < K; ++r)
+        if ((r & j) == 0) cmp_exchange(x[r], x[r ^ j]);
+  }
+}
+
+// Place of position p in a shared-memory key buffer: lanes that write 4, 8 or 16 consecutive keys
+// each, and lanes that read consecutive ones, both hit distinct banks.
+__device__ __forceinline__ int key_place(int p) { return p ^ ((p >> 4) & 15); }
+
+// Sort a segment of 64 < n <= 32 * K pairs in the warp's registers; the sorted keys go through the
+// warp's shared buffer so that the writes to memory are coalesced.
+template <int K>
+__device__ __forceinline__ void sort_segment(const SortOut& o, long long t, long long start, int n, int lane,
+                                             unsigned long long* buf) {
+  unsigned long long x[K];
+#pragma unroll
+  for (int r = 0; r < K; ++r) x[r] = r * 32 + lane < n ? o.seg[start + r * 32 + lane] : ~0ull;
+  warp_sort<K>(x, lane);
+#pragma unroll
+  for (int r = 0; r < K; ++r) buf[key_place(lane * K + r)] = x[r];
+  __syncwarp();
+#pragma unroll
+  for (int r = 0; r < K; ++r)
+    if (r * 32 + lane < n) put_pair(o, t, start + r * 32 + lane, buf[key_place(r * 32 + lane)]);
+}
+
+// One warp per tile, its keys in registers; segments longer than WARP_SORT_MAX are listed for the
+// CTA-wide kernel.  Issue-bound (about 6 warp instructions a key at 512 keys, 4.5 at 128).  Lists of
+// more than 64 pairs in shared memory, with an integer division per exchange, took 161 us where this
+// takes 73 (12 views of a 1M-face map, 127 pairs a tile) and 35 where it takes 9 (mesh, 561k pixels).
 __global__ void __launch_bounds__(32 * SORT_WARPS_PER_BLOCK) k_tile_sort(SortOut o) {
   __shared__ unsigned long long sbuf[SORT_WARPS_PER_BLOCK][WARP_SORT_MAX];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -415,72 +491,113 @@ __global__ void __launch_bounds__(32 * SORT_WARPS_PER_BLOCK) k_tile_sort(SortOut
     }
     return;
   }
-  unsigned long long* s = sbuf[warp];
-  for (int i = lane; i < n; i += 32) s[i] = o.seg[start + i];
-  __syncwarp();
-  int P = 64;
-  while (P < n) P <<= 1;
-  for (int k = 2; k <= P; k <<= 1) {
-    for (int j = k >> 1; j > 0; j >>= 1) {
-      for (int q = lane; q < P / 2; q += 32) {
-        const int blk = q / j, off = q - blk * j;
-        const int i = blk * 2 * j + off;
-        // the merge's first step pairs mirrored positions of its block of k, then half-cleaners
-        const int l = (j == (k >> 1)) ? (i / k) * k + k - 1 - (i % k) : i + j;
-        if (l < n) {
-          const unsigned long long u = s[i], v = s[l];
-          if (v < u) {
-            s[i] = v;
-            s[l] = u;
-          }
-        }
-      }
-      __syncwarp();
-    }
-  }
-  for (int i = lane; i < n; i += 32) put_pair(o, t, start + i, s[i]);
+  if (n <= 128) sort_segment<4>(o, t, start, n, lane, sbuf[warp]);
+  else if (n <= 256) sort_segment<8>(o, t, start, n, lane, sbuf[warp]);
+  else sort_segment<16>(o, t, start, n, lane, sbuf[warp]);
 }
 
-constexpr int LARGE_T = 1024;
-constexpr int LARGE_SMEM_ITEMS = 16384;  // 128 KB of keys
+constexpr int LARGE_T = 256;
+constexpr int LARGE_ITEMS = 4096;  // keys sorted in shared memory at a time, in two buffers (64 KB)
+constexpr int LARGE_RUN = 128;     // keys a warp sorts in registers (4 per lane) before the merges
+constexpr int LARGE_VT = 8;        // consecutive outputs a thread merges
 
-// The listed long segments, one CTA each (grid-stride over the list): in shared memory up to
-// LARGE_SMEM_ITEMS pairs, else in place in the segment buffer.
-__global__ void __launch_bounds__(LARGE_T) k_tile_sort_large(SortOut o, unsigned long long* seg) {
-  extern __shared__ __align__(16) unsigned long long lbuf[];
-  const unsigned nl = min(*o.n_large, (unsigned)o.n_tiles);
-  for (unsigned w = blockIdx.x; w < nl; w += gridDim.x) {
-    const long long t = o.large[w];
-    const uint2 rg = o.ranges[t];  // already cut to the capacity
-    const long long start = rg.x;
-    const long long end = rg.y;
-    const long long n = end - start;
-    const bool in_smem = n <= LARGE_SMEM_ITEMS;
-    unsigned long long* s = in_smem ? lbuf : seg + start;
-    if (in_smem)
-      for (long long i = threadIdx.x; i < n; i += LARGE_T) s[i] = seg[start + i];
-    __syncthreads();
-    long long P = 1;
-    while (P < n) P <<= 1;
-    for (long long k = 2; k <= P; k <<= 1) {
-      for (long long j = k >> 1; j > 0; j >>= 1) {
-        for (long long q = threadIdx.x; q < P / 2; q += LARGE_T) {
-          const long long blk = q / j, off = q - blk * j;
-          const long long i = blk * 2 * j + off;
-          const long long l = (j == (k >> 1)) ? (i / k) * k + k - 1 - (i % k) : i + j;
-          if (l < n) {
-            const unsigned long long u = s[i], v = s[l];
-            if (v < u) {
-              s[i] = v;
-              s[l] = u;
-            }
-          }
-        }
-        __syncthreads();
+// One merge level of a block's n keys: sorted runs of w keys (w a power of two, the last one shorter)
+// become runs of 2w.  A thread finds where its LARGE_VT consecutive outputs start in the two runs by
+// bisection along their diagonal (merge path) and merges serially: 0.7 warp instructions a key.
+template <typename I, typename Buf>  // I: the type of a position
+__device__ __forceinline__ void merge_level(const Buf& src, const Buf& dst, I n, I w) {
+  for (I o = (I)threadIdx.x * LARGE_VT; o < n; o += LARGE_T * LARGE_VT) {
+    const I base = o & ~(2 * w - 1), d = o - base;
+    const I la = min(w, n - base), lb = max((I)0, min(w, n - base - w));
+    I lo = max((I)0, d - lb), hi = min(d, la);
+    while (lo < hi) {
+      const I mid = (lo + hi) >> 1;
+      if (src.get(base + mid) < src.get(base + w + d - 1 - mid)) lo = mid + 1;
+      else hi = mid;
+    }
+    I i = lo, j = d - lo;
+    unsigned long long ka = i < la ? src.get(base + i) : ~0ull, kb = j < lb ? src.get(base + w + j) : ~0ull;
+#pragma unroll
+    for (int v = 0; v < LARGE_VT; ++v) {
+      if (o + v >= n) break;
+      const bool a = ka < kb;  // keys are unique, and below ~0 while any is left
+      dst.put(o + v, a ? ka : kb);
+      if (a) {
+        ++i;
+        ka = i < la ? src.get(base + i) : ~0ull;
+      } else {
+        ++j;
+        kb = j < lb ? src.get(base + w + j) : ~0ull;
       }
     }
-    for (long long i = threadIdx.x; i < n; i += LARGE_T) put_pair(o, t, start + i, s[i]);
-    __syncthreads();
+  }
+}
+
+struct SharedKeys {
+  unsigned long long* p;
+  __device__ __forceinline__ unsigned long long get(int i) const { return p[key_place(i)]; }
+  __device__ __forceinline__ void put(int i, unsigned long long k) const { p[key_place(i)] = k; }
+};
+struct GlobalKeys {
+  unsigned long long* p;
+  __device__ __forceinline__ unsigned long long get(long long i) const { return p[i]; }
+  __device__ __forceinline__ void put(long long i, unsigned long long k) const { p[i] = k; }
+};
+
+// The listed long segments, one CTA each (grid-stride over the list).  LARGE_ITEMS keys at a time are
+// sorted in shared memory; a longer segment's sorted parts are then merged in global memory, between
+// the segment buffer and the segment's place in the output.  (A bitonic network over the whole
+// segment in shared memory took 574 us of a 9-view render of 2M faces where this takes 85, 120 us of a
+// 12-view window of 1M faces where this takes 21.)
+__global__ void __launch_bounds__(LARGE_T) k_tile_sort_large(SortOut o, unsigned long long* seg) {
+  extern __shared__ __align__(16) unsigned long long lbuf[];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const unsigned nl = min(*o.n_large, (unsigned)o.n_tiles);
+  for (unsigned e = blockIdx.x; e < nl; e += gridDim.x) {
+    const long long t = o.large[e];
+    const uint2 rg = o.ranges[t];  // already cut to the capacity
+    const long long start = rg.x;
+    const long long len = (long long)rg.y - start;
+    for (long long c0 = 0; c0 < len; c0 += LARGE_ITEMS) {
+      const int n = (int)min((long long)LARGE_ITEMS, len - c0);
+      SharedKeys cur{lbuf}, nxt{lbuf + LARGE_ITEMS};
+      for (int r0 = warp * LARGE_RUN; r0 < n; r0 += (LARGE_T / 32) * LARGE_RUN) {
+        unsigned long long x[4];
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          x[r] = r0 + r * 32 + lane < n ? seg[start + c0 + r0 + r * 32 + lane] : ~0ull;
+        warp_sort<4>(x, lane);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          if (r0 + lane * 4 + r < n) cur.put(r0 + lane * 4 + r, x[r]);
+      }
+      __syncthreads();
+      for (int w = LARGE_RUN; w < n; w <<= 1) {
+        merge_level(cur, nxt, n, w);
+        __syncthreads();
+        const SharedKeys sw = cur;
+        cur = nxt;
+        nxt = sw;
+      }
+      if (len <= LARGE_ITEMS) {
+        for (int i = threadIdx.x; i < n; i += LARGE_T) put_pair(o, t, start + i, cur.get(i));
+      } else {
+        for (int i = threadIdx.x; i < n; i += LARGE_T) seg[start + c0 + i] = cur.get(i);
+      }
+      __syncthreads();
+    }
+    if (len > LARGE_ITEMS) {
+      GlobalKeys src{seg + start}, dst{o.keys + start};
+      for (long long w = LARGE_ITEMS; w < len; w <<= 1) {
+        merge_level(src, dst, len, w);
+        __syncthreads();
+        const GlobalKeys sw = src;
+        src = dst;
+        dst = sw;
+      }
+      for (long long i = threadIdx.x; i < len; i += LARGE_T) put_pair(o, t, start + i, src.get(i));
+      __syncthreads();
+    }
   }
 }
 
@@ -533,8 +650,9 @@ cudaError_t ts_launch_bin(const TsPlanImpl* p, const TsWs& w, cudaStream_t s) {
              p->bin_blocks > 0 ? w.tmat : nullptr, p->bin_blocks, &w.hdr->n_pairs};
   k_tile_sort<<<(unsigned)((p->n_tiles + SORT_WARPS_PER_BLOCK - 1) / SORT_WARPS_PER_BLOCK), 32 * SORT_WARPS_PER_BLOCK,
                 0, s>>>(so);
-  e = ts_smem_limit((const void*)k_tile_sort_large, (int)(LARGE_SMEM_ITEMS * sizeof(unsigned long long)));
+  constexpr int large_smem = 2 * LARGE_ITEMS * (int)sizeof(unsigned long long);
+  e = ts_smem_limit((const void*)k_tile_sort_large, large_smem);
   if (e != cudaSuccess) return e;
-  k_tile_sort_large<<<(unsigned)ts_sm_count(), LARGE_T, LARGE_SMEM_ITEMS * sizeof(unsigned long long), s>>>(so, w.keys[1]);
+  k_tile_sort_large<<<3u * (unsigned)ts_sm_count(), LARGE_T, large_smem, s>>>(so, w.keys[1]);  // 3 fit on an SM
   return cudaGetLastError();
 }
