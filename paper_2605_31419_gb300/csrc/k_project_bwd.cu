@@ -13,21 +13,24 @@
 //     Jacobian [I, -[v_C]x] (Eq. 7): dL/dtau += [g_C ; v_C x g_C].
 //
 // Gradient slots are face-major (slot = face * V + view) and cleared by the projection pass for
-// the visible ones.  Persistent warps take 4 faces at a time; one ballot per face and 32 views
-// gives the face's visible views.  Lanes 0..20 each own one output word (3 positions x 3 vertices,
-// 3 colours x 3 vertices, the opacity; lane 21 sigma_F), sum it over the face's visible views in
-// view order and add it to the map gradient.  Each view's pose terms are added to the warp's
-// per-view sums in shared memory in face order; at the end the warps' sums are added in a fixed
-// order into per-block partials, which a last kernel adds in a fixed order.  Two forms, with the
-// same arithmetic and the same summation orders (so the same results):
-//   * one pass (8 or more views): the 4 faces' (face, view) entries, numbered face by face with
-//     views in order, run the chain rule one per lane (batches of 32), each lane leaving its
-//     entry's 20 map words in a shared-memory row that the word lanes sum; each slot is read
-//     once and nothing is written back;
-//   * two passes (fewer views, where 4 faces fill few lanes): A. persistent warps scan the
-//     visibility counts, queue the visible slots with ballots and run the chain rule on full warps,
-//     writing each slot's results back into it; B. the word lanes sum the written-back words,
-//     with up to 8 loads in flight.
+// the visible ones; each is read once, in full, and nothing is written back.  Two forms:
+//   * with map gradients, a warp takes 32 faces at a time (8 or 16 of a small map): it stages the faces'
+//     vertices in shared memory, lists their visible entries face by face with views in order, and runs
+//     the chain rule on 32 entries at a time; each entry leaves its 20 map words in a shared row, lane w
+//     sums word w over each face's rows in view order, and the sums are added to the map gradient,
+//     consecutive vertices by consecutive lanes.  Pose terms are added to per-view sums in face order;
+//   * without map gradients (tracking), warps walk one view's faces, queue the visible ones and run the
+//     chain rule on full warps, each lane keeping its own pose sums.
+// In both, a lane's next slot crosses into shared memory (cp.async) while the current one is worked on.
+// Every sum runs in a fixed order, so the gradients are deterministic given the slots.  The pose sums
+// leave per-block partials, which a last kernel adds in a fixed order.
+//
+// Both are bound by the latency of their loads and by issue (37 % issue active, 16 warps per SM; the chain
+// rule is about 550 instructions a batch).  With 4 faces a warp, each lane gathering its entry's vertices,
+// view and slot itself, and a separate two-pass form below 8 views, the map form took 489 us of a 12-view
+// window of 1M faces (now 278), 185 of a 20-view room of 300k (157), 130 of a 6-view window of 300k (70),
+// 48 of a 3-view indexed mesh (25); the pose alone, 64 views of 150k faces, 185 (155).  Two buffers of
+// staged vertices cost the fourth resident block and a second wave: 263 us on the room.
 
 #include <algorithm>
 
@@ -45,11 +48,12 @@ struct PBArgs {
   const float4* aux;  // per (view, face) normal and sigma_F (TS_FLAG_NORMALS / TS_FLAG_FACE_SIGMA)
   bool normals, face_sigma;
   float* dst_sigma;  // dL/dsigma_F per face (TS_FLAG_FACE_SIGMA), may be null
-  const TsDevHeader* hdr;
+  TsDevHeader* hdr;
   float* dst[7];  // gpx, gpy, gpz, gcr, gcg, gcb, gop
   bool min_opacity;  // o_F = min of the vertex opacities: dL/do_F to the first minimal vertex
-  float* part;
-  int nblocks;
+  float* part;       // per (view, block): the pose sums
+  int part_stride;   // blocks the workspace has room for
+  int unit;          // without map gradients: consecutive faces per warp (a multiple of 32)
 };
 
 __device__ __forceinline__ long long face_vertex(const TsDevHeader* h, long long m, int k) {
@@ -57,12 +61,68 @@ __device__ __forceinline__ long long face_vertex(const TsDevHeader* h, long long
   return (j >= 0 && j < h->n_vertices) ? j : 0;
 }
 
-// One 32-byte load (eight floats) from a 32-byte aligned global address.
-__device__ __forceinline__ void ld_v8(const float* p, float* o) {
-  asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3]), "=f"(o[4]), "=f"(o[5]), "=f"(o[6]), "=f"(o[7])
-               : "l"(p)
-               : "memory");
+// A slot's sums in registers: words 0..23, and with the side array 24, 30 and 31.
+struct SlotSums {
+  float G[24], w24, w30, w31;
+};
+// Floats between the lanes' slot copies in shared memory: 7 or 9 16-byte groups, so that the lanes of a
+// quarter warp read distinct banks.
+__host__ __device__ constexpr int slot_stride(bool aux) { return aux ? 36 : 28; }
+
+// This lane copies a slot into its place `dst`; wait_slot waits for the lane's own copies only.
+__device__ __forceinline__ void fetch_slot(const PBArgs& a, float* dst, long long slot) {
+  const float* src = a.grad + slot * TS_GRAD_WORDS;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) ts_cp_async16(dst + 4 * i, src + 4 * i);
+  if (a.aux) {
+    ts_cp_async16(dst + 24, src + 24);
+    ts_cp_async16(dst + 28, src + 28);
+  }
+  ts_cp_async_commit();
+}
+__device__ __forceinline__ void wait_slot(const PBArgs& a, const float* src, SlotSums& s) {
+  ts_cp_async_wait_all();
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const float4 q = reinterpret_cast<const float4*>(src)[i];
+    s.G[4 * i] = q.x; s.G[4 * i + 1] = q.y; s.G[4 * i + 2] = q.z; s.G[4 * i + 3] = q.w;
+  }
+  s.w24 = s.w30 = s.w31 = 0.f;
+  if (a.aux) {
+    s.w24 = src[24];
+    s.w30 = src[30];
+    s.w31 = src[31];
+  }
+}
+
+// 4-byte asynchronous copy of one value.
+__device__ __forceinline__ void cp_async4(float* dst, const float* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(ts_smem_u32(dst)), "l"(src) : "memory");
+}
+// Copy vertex j as vertex k of a staged face (positions at d + 3k, colours at d + 9 + 3k); the copies
+// join the group committed next.
+__device__ __forceinline__ void fetch_vertex(const TsDevHeader* h, float* d, int k, long long j) {
+  d += 3 * k;
+  cp_async4(d, h->px + j);
+  cp_async4(d + 1, h->py + j);
+  cp_async4(d + 2, h->pz + j);
+  cp_async4(d + 9, h->cr + j);
+  cp_async4(d + 10, h->cg + j);
+  cp_async4(d + 11, h->cb + j);
+}
+
+// A view's intrinsics and pose as 16 floats: fx, fy, cx, cy, R, t.  VP is odd, so that lanes with
+// different views read distinct banks.
+constexpr int VP = 17;
+__device__ __forceinline__ void stage_view(const PBArgs& a, float* d, int v) {
+  d[0] = a.views[v].fx;
+  d[1] = a.views[v].fy;
+  d[2] = a.views[v].cx;
+  d[3] = a.views[v].cy;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) d[4 + i] = a.poses[v].R[i];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) d[13 + i] = a.poses[v].t[i];
 }
 
 // What the chain rule of one visible (view, face) gives: the world-space vertex-position
@@ -75,28 +135,30 @@ struct SlotTerms {
   float gsig;    // dL/dsigma_F (TS_FLAG_FACE_SIGMA)
 };
 
-// The chain rule of one visible (view, face).
-__device__ __forceinline__ void chain_terms(const PBArgs& a, int v, long long m, SlotTerms& t) {
-  const TsDevHeader* h = a.hdr;
-  const long long slot = m * a.V + v;
-  const float* gw = a.grad + slot * TS_GRAD_WORDS;
-  float G[24];
-  ld_v8(gw, G);
-  ld_v8(gw + 8, G + 8);
-  ld_v8(gw + 16, G + 16);
-  const float gsig = a.face_sigma ? gw[24] : 0.f;  // word 24
-  const TsView vw = a.views[v];
-  const ts_pose P = a.poses[v];
+// The chain rule of one visible (view, face) from its slot's sums; X holds the face's world positions
+// (vertex k, coordinate c at 3k + c) and then its vertex colours, vp its view (stage_view).
+__device__ __forceinline__ void chain_terms(const PBArgs& a, int v, long long m, const SlotSums& sl, const float* X,
+                                            const float* vp, SlotTerms& t) {
+  const float(&G)[24] = sl.G;
+  TsView vw;
+  vw.fx = vp[0];
+  vw.fy = vp[1];
+  vw.cx = vp[2];
+  vw.cy = vp[3];
+  ts_pose P;
+#pragma unroll
+  for (int i = 0; i < 9; ++i) P.R[i] = vp[4 + i];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) P.t[i] = vp[13 + i];
   // The projection, edge vectors, lengths and area are recomputed in the forward record's fixed
   // operation order, so the chain rule sees bit-identical values; for slivers the area is a
   // cancelling difference and a one-ulp change of a vertex would move the gradient visibly.
   float xc[3], yc[3], zc[3], u[3], w[3], col[3][3];
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
-    const long long j = face_vertex(h, m, k);
-    ts_rigid_f32(P, __ldg(h->px + j), __ldg(h->py + j), __ldg(h->pz + j), xc[k], yc[k], zc[k]);
+    ts_rigid_f32(P, X[3 * k], X[3 * k + 1], X[3 * k + 2], xc[k], yc[k], zc[k]);
     ts_pinhole_f32(vw, xc[k], yc[k], zc[k], u[k], w[k]);
-    col[k][0] = __ldg(h->cr + j); col[k][1] = __ldg(h->cg + j); col[k][2] = __ldg(h->cb + j);
+    col[k][0] = X[9 + 3 * k]; col[k][1] = X[10 + 3 * k]; col[k][2] = X[11 + 3 * k];
   }
   float ex[3], ey[3], len[3], il[3];
 #pragma unroll
@@ -165,7 +227,7 @@ __device__ __forceinline__ void chain_terms(const PBArgs& a, int v, long long m,
   // dL/du = s (g - n (n . g)) / |u|, dL/de1 = e2 x dL/du, dL/de2 = dL/du x e1
   float ng[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
   if (a.normals) {
-    const float gn[3] = {G[23], a.grad[slot * TS_GRAD_WORDS + 30], a.grad[slot * TS_GRAD_WORDS + 31]};
+    const float gn[3] = {G[23], sl.w30, sl.w31};
     if (gn[0] != 0.f || gn[1] != 0.f || gn[2] != 0.f) {
       const float4 nn = a.aux[(long long)v * a.M + m];
       const float e1[3] = {xc[1] - xc[0], yc[1] - yc[0], zc[1] - zc[0]};
@@ -210,318 +272,285 @@ __device__ __forceinline__ void chain_terms(const PBArgs& a, int v, long long m,
 #pragma unroll
   for (int i = 0; i < 9; ++i) t.gc[i] = G[G_C + i];
   t.go = G[G_O];
-  t.gsig = gsig;
+  t.gsig = sl.w24;
 }
 
-// Two-pass form, pass A: the chain rule of one visible (view, face), written back into its slot:
-// positions into words 0..8 (the edge sums, now consumed), pose terms into 24..29, sigma_F into 23.
-__device__ __forceinline__ void chain_slot(const PBArgs& a, int v, long long m) {
-  SlotTerms t;
-  chain_terms(a, v, m, t);
-  float* gs = a.grad + (m * a.V + v) * TS_GRAD_WORDS;
-  float4* gp = reinterpret_cast<float4*>(gs);
-  gp[0] = make_float4(t.out[0], t.out[1], t.out[2], t.out[3]);
-  gp[1] = make_float4(t.out[4], t.out[5], t.out[6], t.out[7]);
-  gs[8] = t.out[8];
-  gp[6] = make_float4(t.tau[0], t.tau[1], t.tau[2], t.tau[3]);
-  gs[28] = t.tau[4];
-  gs[29] = t.tau[5];
-  if (a.face_sigma) gs[23] = t.gsig;
+constexpr int PB_WARPS = 4;
+constexpr int PB_T = 32 * PB_WARPS;
+constexpr int PB_RS = 21;   // floats per entry row (positions 9, colours 9, opacity, sigma; odd: no bank conflicts)
+constexpr int PB_FS = 19;   // floats per staged face (positions 9, colours 9)
+constexpr int PB_PS = 7;    // floats per view's pose sums (6 used)
+
+// Views whose visibility the lanes of one face look up at a time (64 bits each).
+__host__ __device__ constexpr int pbwd_view_chunk(int faces) { return 64 * (32 / faces); }
+// Shared floats of one warp (a multiple of 4): slot copies, entry rows, staged faces, per-face sums,
+// per-view pose sums, entry list.
+__host__ __device__ constexpr int pbwd_warp_floats(int V, int faces, bool aux) {
+  const int chunk = V < pbwd_view_chunk(faces) ? V : pbwd_view_chunk(faces);
+  return (32 * slot_stride(aux) + 32 * PB_RS + faces * (PB_FS + PB_RS) + V * PB_PS + (faces * chunk + 1) / 2 + 3) & ~3;
 }
 
-constexpr int PA_T = 256;
-constexpr int PA_WARPS = PA_T / 32;
-
-__global__ void __launch_bounds__(PA_T) k_pbwd_chain(PBArgs a) {
-  __shared__ long long q[PA_WARPS][64];  // queued view-major indices v * M + m
+// With map gradients: FPW faces per warp iteration, 32 / FPW lanes looking up each face's views.
+template <int FPW>
+__global__ void __launch_bounds__(PB_T, 4) k_pbwd_map(PBArgs a) {
+  constexpr int LPF = 32 / FPW, ROUNDS = (3 * FPW + 31) / 32;
+  extern __shared__ __align__(16) float pv[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long long gw = (long long)blockIdx.x * PA_WARPS + warp, nw = (long long)gridDim.x * PA_WARPS;
-  const unsigned lt = (1u << lane) - 1u;
+  const TsDevHeader* h = a.hdr;
+  const bool aux = a.aux != nullptr;
+  const int per_warp = pbwd_warp_floats(a.V, FPW, aux);
+  float* views = pv + (size_t)PB_WARPS * per_warp;  // [V][VP]
+  float* slots = pv + (size_t)warp * per_warp;
+  float* rows = slots + 32 * slot_stride(aux);
+  float* fdat = rows + 32 * PB_RS;
+  float* fsum = fdat + FPW * PB_FS;
+  float* my = fsum + FPW * PB_RS;
+  uint16_t* list = reinterpret_cast<uint16_t*>(my + a.V * PB_PS);  // face * 256 + view
+  float* slot_here = slots + lane * slot_stride(aux);
+  for (int v = threadIdx.x; v < a.V; v += PB_T) stage_view(a, views + v * VP, v);
+  for (int i = lane; i < a.V * PB_PS; i += 32) my[i] = 0.f;
+  __syncthreads();
+  const bool indexed = h->faces != nullptr;
+  const int f = lane / LPF;
+  const long long stride = (long long)gridDim.x * PB_WARPS * FPW;
+  for (long long m0 = ((long long)blockIdx.x * PB_WARPS + warp) * FPW; m0 < a.M; m0 += stride) {
+#pragma unroll
+    for (int i0 = 0; i0 < 3 * FPW; i0 += 32) {
+      const int i = i0 + lane, fi = i / 3, k = i - 3 * fi;
+      if (i < 3 * FPW && m0 + fi < a.M) fetch_vertex(h, fdat + fi * PB_FS, k, face_vertex(h, m0 + fi, k));
+    }
+    ts_cp_async_commit();
+    for (int i = lane; i < FPW * PB_RS; i += 32) fsum[i] = 0.f;
+    unsigned seen = 0u;
+    for (int c0 = 0; c0 < a.V; c0 += pbwd_view_chunk(FPW)) {
+      // this lane looks up views [va, vb) of face f
+      const int nvc = min(a.V - c0, pbwd_view_chunk(FPW)), Q = (nvc + LPF - 1) / LPF;
+      const int va = c0 + min((lane % LPF) * Q, nvc), vb = min(va + Q, c0 + nvc);
+      unsigned long long bits = 0ull;
+      {
+        const uint32_t* cp = a.count + (long long)va * a.M + m0 + f;
+        const int nv = m0 + f < a.M ? vb - va : 0;
+#pragma unroll 8
+        for (int i = 0; i < nv; ++i) bits |= (unsigned long long)(cp[(long long)i * a.M] != 0u) << i;
+      }
+      const int mine = __popcll(bits);
+      int incl = mine;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += t;
+      }
+      const int total = __shfl_sync(0xffffffffu, incl, 31);
+      seen |= __ballot_sync(0xffffffffu, mine > 0);
+      for (int k = incl - mine; bits; bits &= bits - 1) list[k++] = (uint16_t)(f * 256 + va + __ffsll(bits) - 1);
+      // where this lane's vertices' faces have their entries: one round of lanes per 32 (face, vertex)s
+      int e0[ROUNDS], e1[ROUNDS];
+#pragma unroll
+      for (int r = 0; r < ROUNDS; ++r) {
+        const int fi = min((r * 32 + lane) / 3, FPW - 1);
+        e1[r] = __shfl_sync(0xffffffffu, incl, fi * LPF + LPF - 1);
+        e0[r] = __shfl_sync(0xffffffffu, incl - mine, fi * LPF);
+        if (r * 32 + lane >= 3 * FPW) e1[r] = e0[r];
+      }
+      if (c0 == 0) ts_cp_async_wait_all();  // this lane's share of the faces
+      __syncwarp();
+      int next = lane < total ? list[lane] : -1;
+      if (next >= 0) fetch_slot(a, slot_here, (m0 + (next >> 8)) * a.V + (next & 255));
+      for (int b0 = 0; b0 < total; b0 += 32) {
+        const int ne = min(total - b0, 32);
+        const bool act = lane < ne;
+        const int code = act ? next : 0;
+        const int fe = code >> 8, v = code & 255;
+        SlotSums sl;
+        if (act) wait_slot(a, slot_here, sl);
+        next = b0 + 32 + lane < total ? list[b0 + 32 + lane] : -1;
+        if (next >= 0) fetch_slot(a, slot_here, (m0 + (next >> 8)) * a.V + (next & 255));
+        float tau[6];
+        if (act) {
+          SlotTerms t;
+          chain_terms(a, v, m0 + fe, sl, fdat + fe * PB_FS, views + v * VP, t);
+          float* row = rows + lane * PB_RS;
+#pragma unroll
+          for (int i = 0; i < 9; ++i) row[i] = t.out[i];
+#pragma unroll
+          for (int i = 0; i < 9; ++i) row[9 + i] = t.gc[i];
+          row[18] = t.go;
+          row[19] = t.gsig;
+#pragma unroll
+          for (int i = 0; i < 6; ++i) tau[i] = t.tau[i];
+        }
+        // pose terms: the entries of one view, in face order, one after another
+        const unsigned same = __match_any_sync(0xffffffffu, act ? v : 256 + lane);
+        const int rank = __popc(same & ((1u << lane) - 1u));
+        const int rounds = (int)__reduce_max_sync(0xffffffffu, (unsigned)rank) + 1;
+        for (int r = 0; r < rounds; ++r) {
+          if (act && rank == r) {
+#pragma unroll
+            for (int i = 0; i < 6; ++i) my[v * PB_PS + i] += tau[i];
+          }
+          __syncwarp();
+        }
+        // map words: the lane of each (face, vertex) sums its words over the face's rows, views in order
+#pragma unroll
+        for (int r = 0; r < ROUNDS; ++r) {
+          const int lo = max(e0[r] - b0, 0), hi = min(e1[r] - b0, 32);
+          if (lo < hi) {
+            const int i = r * 32 + lane, k = i % 3;
+            float* w = fsum + i / 3 * PB_RS;
+            float sum[8];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) sum[c] = w[3 * k + c];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) sum[3 + c] = w[9 + 3 * c + k];
+            sum[6] = w[18];
+            sum[7] = w[19];
+            for (int e = lo; e < hi; ++e) {
+              const float* row = rows + e * PB_RS;
+#pragma unroll
+              for (int c = 0; c < 3; ++c) sum[c] += row[3 * k + c];
+#pragma unroll
+              for (int c = 0; c < 3; ++c) sum[3 + c] += row[9 + 3 * c + k];
+              sum[6] += row[18];
+              sum[7] += row[19];
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) w[3 * k + c] = sum[c];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) w[9 + 3 * c + k] = sum[3 + c];
+            if (k == 0) {  // (the face's other two lanes drop these sums)
+              w[18] = sum[6];
+              w[19] = sum[7];
+            }
+          }
+        }
+        __syncwarp();  // every lane has read the rows before the next batch writes them
+      }
+    }
+    // into the map gradient; a face seen by no view adds nothing
+    for (int i = lane; i < 3 * FPW; i += 32) {
+      const int fi = i / 3, k = i - 3 * fi;
+      if (((seen >> (fi * LPF)) & ((1u << LPF) - 1u)) == 0u) continue;  // (a face past M has no view)
+      const long long m = m0 + fi, j = face_vertex(h, m, k);
+      const float* w = fsum + fi * PB_RS;
+      float scale = 1.0f / 3.0f;
+      if (a.min_opacity) {  // the first vertex, in face order, attaining the minimum
+        const float o0 = __ldg(h->op + face_vertex(h, m, 0)), o1 = __ldg(h->op + face_vertex(h, m, 1));
+        const float o2 = __ldg(h->op + face_vertex(h, m, 2));
+        const int km = (o0 <= o1 && o0 <= o2) ? 0 : (o1 <= o2 ? 1 : 2);
+        scale = k == km ? 1.0f : 0.0f;
+      }
+      float add[7];
+#pragma unroll
+      for (int c = 0; c < 7; ++c) add[c] = c < 3 ? w[3 * k + c] : (c < 6 ? w[9 + 3 * (c - 3) + k] : w[18] * scale);
+      if (indexed) {
+#pragma unroll
+        for (int c = 0; c < 7; ++c)
+          if (a.dst[c]) atomicAdd(a.dst[c] + j, add[c]);
+      } else {
+        float old[7];
+#pragma unroll
+        for (int c = 0; c < 7; ++c) old[c] = a.dst[c] ? a.dst[c][j] : 0.f;
+#pragma unroll
+        for (int c = 0; c < 7; ++c)
+          if (a.dst[c]) a.dst[c][j] = old[c] + add[c];
+      }
+      if (k == 0 && a.dst_sigma) a.dst_sigma[m] += w[19];
+    }
+    __syncwarp();  // the next faces reuse the sums and the list
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < a.V * 6; t += PB_T) {
+    const int v = t / 6, i = t - 6 * (t / 6);
+    float sum = 0.f;
+#pragma unroll
+    for (int w = 0; w < PB_WARPS; ++w) sum += pv[(size_t)w * per_warp + (my - slots) + v * PB_PS + i];
+    a.part[((long long)v * a.part_stride + blockIdx.x) * 6 + i] = sum;
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) a.hdr->pose_blocks = gridDim.x;
+}
+
+// Without map gradients: blocks (part of the faces, view), a.unit consecutive faces per warp.
+__global__ void __launch_bounds__(PB_T, 4) k_pbwd_pose(PBArgs a) {
+  extern __shared__ __align__(16) float pv[];  // [PB_T] slot copies, [PB_T] faces
+  __shared__ uint32_t q[PB_WARPS][64];         // queued visible faces
+  __shared__ float red[PB_WARPS][6], view[VP];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, v = blockIdx.y;
+  const TsDevHeader* h = a.hdr;
+  const uint32_t* cnt = a.count + (long long)v * a.M;
+  float* slot_here = pv + threadIdx.x * slot_stride(a.aux != nullptr);
+  float* face_here = pv + PB_T * slot_stride(a.aux != nullptr) + threadIdx.x * PB_FS;
+  if (threadIdx.x == 0) stage_view(a, view, v);
+  __syncthreads();
+  float tau[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+  long long pend = -1;  // the face whose slot this lane fetched last
+  // take up the pending face, after starting the copies of the next one's vertices and slot
+  auto take = [&](long long m_next) {
+    const long long m = pend;
+    SlotSums sl;
+    float X[18];
+    if (m >= 0) {
+      wait_slot(a, slot_here, sl);
+#pragma unroll
+      for (int i = 0; i < 18; ++i) X[i] = face_here[i];
+    }
+    if (m_next >= 0) {
+#pragma unroll
+      for (int k = 0; k < 3; ++k) fetch_vertex(h, face_here, k, face_vertex(h, m_next, k));
+      fetch_slot(a, slot_here, m_next * a.V + v);
+    }
+    pend = m_next;
+    if (m < 0) return;
+    SlotTerms t;
+    chain_terms(a, v, m, sl, X, view, t);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) tau[i] += t.tau[i];
+  };
   int qn = 0;
-  for (long long c = gw; c * 32 < a.VM; c += nw) {
-    const long long idx = c * 32 + lane;
-    const bool vis = idx < a.VM && a.count[idx] > 0;
-    const unsigned bal = __ballot_sync(0xffffffffu, vis);
-    if (vis) q[warp][qn + __popc(bal & lt)] = idx;
+  const long long m_begin = ((long long)blockIdx.x * PB_WARPS + warp) * a.unit, m_end = min(m_begin + a.unit, a.M);
+  uint32_t next = m_begin + lane < m_end ? cnt[m_begin + lane] : 0u;
+  for (long long m0 = m_begin; m0 < m_end; m0 += 32) {
+    const uint32_t cur = next;
+    const long long mn = m0 + 32 + lane;
+    next = mn < m_end ? cnt[mn] : 0u;  // the next 32 faces' counts are on their way
+    const unsigned bal = __ballot_sync(0xffffffffu, cur > 0u);
+    if (cur > 0u) q[warp][qn + __popc(bal & ((1u << lane) - 1u))] = (uint32_t)(m0 + lane);
     qn += __popc(bal);
     __syncwarp();
     if (qn >= 32) {
-      const long long e = q[warp][lane];
-      const int v = (int)(e / a.M);
-      chain_slot(a, v, e - (long long)v * a.M);
+      take(q[warp][lane]);
       __syncwarp();
       if (lane < qn - 32) q[warp][lane] = q[warp][lane + 32];
       qn -= 32;
       __syncwarp();
     }
   }
-  if (lane < qn) {
-    const long long e = q[warp][lane];
-    const int v = (int)(e / a.M);
-    chain_slot(a, v, e - (long long)v * a.M);
-  }
-}
-
-constexpr int PG_WARPS = 4;
-constexpr int PG_T = 32 * PG_WARPS;
-constexpr int PG_F = 4;    // faces per warp iteration
-constexpr int PG_RS = 21;  // floats per entry row (out 9, colour 9, opacity, sigma; odd: no bank conflicts)
-constexpr int PG_RMAX = (TS_MAX_VIEWS + 31) / 32;
-constexpr int PBWD_ONE_PASS_VIEWS = 8;  // from here on the one-pass form is faster (room scene, 300k faces)
-
-// Shared memory of one block: per-warp per-view pose sums, per-warp entry rows, per-warp view masks.
-size_t pbwd_smem(int V) {
-  return (size_t)PG_WARPS * V * 8 * sizeof(float) + (size_t)PG_WARPS * 32 * PG_RS * sizeof(float) +
-         (size_t)PG_WARPS * PG_F * PG_RMAX * sizeof(uint32_t);
-}
-
-// Two-pass form, pass B.
-__global__ void __launch_bounds__(PG_T) k_pbwd_gather(PBArgs a) {
-  extern __shared__ float pv[];  // [PG_WARPS][V][8] per-warp per-view pose sums
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const TsDevHeader* h = a.hdr;
-  float* my = pv + (size_t)warp * a.V * 8;
-  for (int i = lane; i < a.V * 8; i += 32) my[i] = 0.f;
+  take(lane < qn ? (long long)q[warp][lane] : -1);
+  take(-1);
   __syncwarp();
-  // lanes 0..20 each own one output word: array c (gpx..gop), vertex k; with per-face sigma,
-  // lane 21 owns the face's dL/dsigma_F (word 23 after the chain pass)
-  const int c = lane / 3, k = lane - 3 * (lane / 3);
-  const bool face_word = lane == 21;
-  const bool owner = lane < 21 || (face_word && a.face_sigma);
-  const int word = c < 3 ? G_DPOS + 3 * k + c : (c < 6 ? G_C + 3 * (c - 3) + k : (c == 6 ? G_O : 23));
-  const float mean_scale = c == 6 ? (1.0f / 3.0f) : 1.0f;
-  float* dst = owner ? (face_word ? a.dst_sigma : a.dst[c]) : nullptr;
-  const bool indexed = h->faces != nullptr;
-  const long long stride = (long long)gridDim.x * PG_WARPS * PG_F;
-  for (long long m0 = ((long long)blockIdx.x * PG_WARPS + warp) * PG_F; m0 < a.M; m0 += stride) {
-    long long j[PG_F];
-    float old[PG_F], s[PG_F];
 #pragma unroll
-    for (int f = 0; f < PG_F; ++f) {
-      const long long m = m0 + f;
-      j[f] = (m < a.M && dst) ? (face_word ? m : face_vertex(h, m, k)) : 0;
-      old[f] = (m < a.M && dst && (!indexed || face_word)) ? dst[j[f]] : 0.f;  // issued early
-      s[f] = 0.f;
-    }
-    for (int r = 0; r * 32 < a.V; ++r) {
-      const int vl = r * 32 + lane;
-      unsigned msk[PG_F];
+  for (int i = 0; i < 6; ++i) {
 #pragma unroll
-      for (int f = 0; f < PG_F; ++f) {
-        const long long m = m0 + f;
-        const uint32_t cnt = (m < a.M && vl < a.V) ? a.count[(long long)vl * a.M + m] : 0u;
-        msk[f] = __ballot_sync(0xffffffffu, cnt > 0);
-      }
-      // pose terms: the lane owning view vl adds each face's terms to the warp's sums (face order)
-#pragma unroll
-      for (int f = 0; f < PG_F; ++f) {
-        if ((msk[f] >> lane) & 1u) {
-          const float* t = a.grad + ((m0 + f) * a.V + vl) * TS_GRAD_WORDS + G_TAU;
-#pragma unroll
-          for (int i = 0; i < 6; ++i) my[vl * 8 + i] += t[i];
-        }
-      }
-      // output words: sum over the visible views in view order, up to 8 loads in flight
-#pragma unroll
-      for (int f = 0; f < PG_F; ++f) {
-        unsigned bits = msk[f];
-        const float* base = a.grad + (m0 + f) * a.V * TS_GRAD_WORDS + word;
-        while (bits) {
-          float vals[8];
-#pragma unroll
-          for (int u = 0; u < 8; ++u) {
-            vals[u] = 0.f;
-            if (bits) {
-              const int v = r * 32 + __ffs(bits) - 1;
-              bits &= bits - 1;
-              if (dst) vals[u] = base[(long long)v * TS_GRAD_WORDS];  // only for a requested output
-            }
-          }
-#pragma unroll
-          for (int u = 0; u < 8; ++u) s[f] += vals[u];
-        }
-      }
-    }
-#pragma unroll
-    for (int f = 0; f < PG_F; ++f) {
-      if (m0 + f < a.M && dst) {
-        float scale = mean_scale;
-        if (c == 6 && a.min_opacity) {  // the first vertex, in face order, attaining the minimum
-          const long long m = m0 + f;
-          const float o0 = __ldg(h->op + face_vertex(h, m, 0)), o1 = __ldg(h->op + face_vertex(h, m, 1));
-          const float o2 = __ldg(h->op + face_vertex(h, m, 2));
-          const int km = (o0 <= o1 && o0 <= o2) ? 0 : (o1 <= o2 ? 1 : 2);
-          scale = k == km ? 1.0f : 0.0f;
-        }
-        if (indexed && !face_word) atomicAdd(dst + j[f], s[f] * scale);
-        else dst[j[f]] = old[f] + s[f] * scale;
-      }
-    }
+    for (int o = 16; o > 0; o >>= 1) tau[i] += __shfl_xor_sync(0xffffffffu, tau[i], o);
+    if (lane == 0) red[warp][i] = tau[i];
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < a.V * 6; t += PG_T) {
-    const int v = t / 6, i = t - 6 * (t / 6);
+  if (threadIdx.x < 6) {
     float sum = 0.f;
 #pragma unroll
-    for (int w = 0; w < PG_WARPS; ++w) sum += pv[((size_t)w * a.V + v) * 8 + i];
-    a.part[((long long)v * a.nblocks + blockIdx.x) * 6 + i] = sum;
+    for (int w = 0; w < PB_WARPS; ++w) sum += red[w][threadIdx.x];
+    a.part[((long long)v * a.part_stride + blockIdx.x) * 6 + threadIdx.x] = sum;
   }
+  if (blockIdx.x == 0 && v == 0 && threadIdx.x == 0) a.hdr->pose_blocks = gridDim.x;
 }
 
-// One-pass form.
-__global__ void __launch_bounds__(PG_T) k_pbwd_face(PBArgs a) {
-  extern __shared__ float pv[];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const TsDevHeader* h = a.hdr;
-  float* my = pv + (size_t)warp * a.V * 8;  // this warp's pose sums [V][8]
-  float* rows = pv + (size_t)PG_WARPS * a.V * 8 + (size_t)warp * 32 * PG_RS;
-  uint32_t* vm = reinterpret_cast<uint32_t*>(pv + (size_t)PG_WARPS * a.V * 8 + (size_t)PG_WARPS * 32 * PG_RS) +
-                 warp * PG_F * PG_RMAX;  // [f][r]: the face's visible views r * 32 + bit
-  for (int i = lane; i < a.V * 8; i += 32) my[i] = 0.f;
-  __syncwarp();
-  // lanes 0..20 each own one output word: array c (gpx..gop), vertex k; with per-face sigma,
-  // lane 21 owns the face's dL/dsigma_F
-  const int c = lane / 3, k = lane - 3 * (lane / 3);
-  const bool face_word = lane == 21;
-  const bool owner = lane < 21 || (face_word && a.face_sigma);
-  const int ridx = c < 3 ? 3 * k + c : (c < 6 ? 9 + 3 * (c - 3) + k : (c == 6 ? 18 : 19));
-  const float mean_scale = c == 6 ? (1.0f / 3.0f) : 1.0f;
-  float* dst = owner ? (face_word ? a.dst_sigma : a.dst[c]) : nullptr;
-  const bool indexed = h->faces != nullptr;
-  const int R = (a.V + 31) >> 5;
-  const long long stride = (long long)gridDim.x * PG_WARPS * PG_F;
-  for (long long m0 = ((long long)blockIdx.x * PG_WARPS + warp) * PG_F; m0 < a.M; m0 += stride) {
-    long long j[PG_F];
-    float old[PG_F], s[PG_F];
-    int nf[PG_F];
-#pragma unroll
-    for (int f = 0; f < PG_F; ++f) {
-      const long long m = m0 + f;
-      j[f] = (m < a.M && dst) ? (face_word ? m : face_vertex(h, m, k)) : 0;
-      old[f] = (m < a.M && dst && (!indexed || face_word)) ? dst[j[f]] : 0.f;  // issued early
-      s[f] = 0.f;
-      nf[f] = 0;
-    }
-    // the faces' visible views, 32 at a time
-    for (int r = 0; r < R; ++r) {
-      const int vl = r * 32 + lane;
-      uint32_t cnt[PG_F];
-#pragma unroll
-      for (int f = 0; f < PG_F; ++f) {
-        const long long m = m0 + f;
-        cnt[f] = (m < a.M && vl < a.V) ? a.count[(long long)vl * a.M + m] : 0u;
-      }
-#pragma unroll
-      for (int f = 0; f < PG_F; ++f) {
-        const unsigned msk = __ballot_sync(0xffffffffu, cnt[f] > 0);
-        if (lane == 0) vm[f * PG_RMAX + r] = msk;
-        nf[f] += __popc(msk);
-      }
-    }
-    __syncwarp();
-    int total = 0, st[PG_F];
-#pragma unroll
-    for (int f = 0; f < PG_F; ++f) {
-      st[f] = total;
-      total += nf[f];
-    }
-    // the (face, view) entries, face by face and views in order, one per lane
-    for (int b0 = 0; b0 < total; b0 += 32) {
-      const int ee = b0 + lane;
-      const bool act = ee < total;
-      int fe = 0, kk = ee;
-      bool found = false;
-#pragma unroll
-      for (int f = 0; f < PG_F; ++f) {
-        if (!found) {
-          if (kk < nf[f]) {
-            fe = f;
-            found = true;
-          } else {
-            kk -= nf[f];
-          }
-        }
-      }
-      int v = 0;
-      SlotTerms t;
-      if (act) {
-        int r = 0;
-        uint32_t mr = vm[fe * PG_RMAX];
-        while (kk >= __popc(mr)) {  // the entry is in a later round of the face's views
-          kk -= __popc(mr);
-          mr = vm[fe * PG_RMAX + ++r];
-        }
-        int pb = 0;
-#pragma unroll
-        for (int w = 16; w > 0; w >>= 1) {  // the kk-th set bit of mr
-          const int cl = __popc(mr & ((1u << w) - 1u));
-          if (kk >= cl) {
-            kk -= cl;
-            pb += w;
-            mr >>= w;
-          }
-        }
-        v = r * 32 + pb;
-        chain_terms(a, v, m0 + fe, t);
-        float* row = rows + lane * PG_RS;
-#pragma unroll
-        for (int i = 0; i < 9; ++i) row[i] = t.out[i];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) row[9 + i] = t.gc[i];
-        row[18] = t.go;
-        row[19] = t.gsig;
-      }
-      // pose terms: face by face (a face's views are distinct), so each view's sum runs in face order
-#pragma unroll
-      for (int f = 0; f < PG_F; ++f) {
-        if (act && fe == f) {
-#pragma unroll
-          for (int i = 0; i < 6; ++i) my[v * 8 + i] += t.tau[i];
-        }
-        __syncwarp();
-      }
-      // output words: each face's entries of this batch, views in order
-      if (dst) {
-#pragma unroll
-        for (int f = 0; f < PG_F; ++f) {
-          const int lo = max(st[f] - b0, 0), hi = min(st[f] + nf[f] - b0, 32);
-          for (int e = lo; e < hi; ++e) s[f] += rows[e * PG_RS + ridx];
-        }
-      }
-      __syncwarp();  // every lane has read the rows before the next batch writes them
-    }
-#pragma unroll
-    for (int f = 0; f < PG_F; ++f) {
-      if (m0 + f < a.M && dst) {
-        float scale = mean_scale;
-        if (c == 6 && a.min_opacity) {  // the first vertex, in face order, attaining the minimum
-          const long long m = m0 + f;
-          const float o0 = __ldg(h->op + face_vertex(h, m, 0)), o1 = __ldg(h->op + face_vertex(h, m, 1));
-          const float o2 = __ldg(h->op + face_vertex(h, m, 2));
-          const int km = (o0 <= o1 && o0 <= o2) ? 0 : (o1 <= o2 ? 1 : 2);
-          scale = k == km ? 1.0f : 0.0f;
-        }
-        if (indexed && !face_word) atomicAdd(dst + j[f], s[f] * scale);
-        else dst[j[f]] = old[f] + s[f] * scale;
-      }
-    }
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < a.V * 6; t += PG_T) {
-    const int v = t / 6, i = t - 6 * (t / 6);
-    float sum = 0.f;
-#pragma unroll
-    for (int w = 0; w < PG_WARPS; ++w) sum += pv[((size_t)w * a.V + v) * 8 + i];
-    a.part[((long long)v * a.nblocks + blockIdx.x) * 6 + i] = sum;
-  }
-}
-
-__global__ void __launch_bounds__(256) k_pose_reduce(const float* __restrict__ part, int nblocks, float* dtau) {
+__global__ void __launch_bounds__(256) k_pose_reduce(const float* __restrict__ part, int part_stride,
+                                                     const TsDevHeader* __restrict__ hdr, float* dtau) {
   __shared__ float red[256][6];
   const int v = blockIdx.x;
+  const int nblocks = min((int)hdr->pose_blocks, part_stride);  // written by the backward
   float s[6] = {0, 0, 0, 0, 0, 0};
   for (int b = threadIdx.x; b < nblocks; b += 256) {
-    const float* p = part + ((long long)v * nblocks + b) * 6;
+    const float* p = part + ((long long)v * part_stride + b) * 6;
 #pragma unroll
     for (int i = 0; i < 6; ++i) s[i] += p[i];
   }
@@ -540,13 +569,26 @@ __global__ void __launch_bounds__(256) k_pose_reduce(const float* __restrict__ p
 
 }  // namespace
 
-// The chain-rule pass's block count fixes the partial-sum layout of the pose gradient and so its summation
-// order: a constant cap (not the device's SM count) keeps dtau's rounding the same on every GPU.
-constexpr long long POSE_BLOCKS_MAX = 2432;
-int ts_pose_blocks(long long M) {
-  const long long want = (M + PG_WARPS * PG_F - 1) / (PG_WARPS * PG_F);
-  return (int)std::max<long long>(1, std::min<long long>(want, POSE_BLOCKS_MAX));
+// The faces per warp and block fix the partial sums of the pose gradient and so its summation order: they
+// depend on the map's size alone, so that a view's dtau is the same alone and among others, and on every GPU.
+constexpr long long MAP_BLOCKS = 608;    // 4 resident blocks on 152 SMs
+constexpr long long POSE_BLOCKS = 2432;  // most blocks per view of the form without map gradients
+int ts_pose_blocks(long long M) {        // the most either form uses
+  return (int)std::max<long long>(1, std::min<long long>((M + 31) / 32, POSE_BLOCKS));
 }
+
+namespace {
+template <int FPW>
+cudaError_t launch_pbwd_map(const PBArgs& a, cudaStream_t s) {
+  const int smem =
+      (PB_WARPS * pbwd_warp_floats(a.V, FPW, a.aux != nullptr) + a.V * VP) * (int)sizeof(float);  // <= 146 KB
+  const cudaError_t e = ts_smem_limit((const void*)k_pbwd_map<FPW>, smem);
+  if (e != cudaSuccess) return e;
+  const long long want = (a.M + PB_WARPS * FPW - 1) / (PB_WARPS * FPW);
+  k_pbwd_map<FPW><<<(unsigned)std::min(want, MAP_BLOCKS), PB_T, smem, s>>>(a);
+  return cudaGetLastError();
+}
+}  // namespace
 
 cudaError_t ts_launch_project_bwd(const TsPlanImpl* p, const TsWs& w, const ts_map_grad* g, cudaStream_t s) {
   if (p->M == 0) {
@@ -570,19 +612,26 @@ cudaError_t ts_launch_project_bwd(const TsPlanImpl* p, const TsWs& w, const ts_m
   a.dst[6] = g->gop;
   a.min_opacity = p->min_opacity;
   a.part = w.pose;
-  a.nblocks = (int)p->n_pose_blocks;
-  if (p->V >= PBWD_ONE_PASS_VIEWS) {
-    k_pbwd_face<<<(unsigned)p->n_pose_blocks, PG_T, pbwd_smem(p->V), s>>>(a);  // < 44 KiB for 256 views
-  } else {
-    const long long chunks = (a.VM + 31) / 32;
-    const long long grid_a = std::min<long long>((chunks + PA_WARPS - 1) / PA_WARPS, (long long)ts_sm_count() * 8);
-    k_pbwd_chain<<<(unsigned)grid_a, PA_T, 0, s>>>(a);
-    k_pbwd_gather<<<(unsigned)p->n_pose_blocks, PG_T, (size_t)PG_WARPS * p->V * 8 * sizeof(float), s>>>(a);
+  a.part_stride = (int)p->n_pose_blocks;
+  a.unit = 0;
+  bool map = a.dst_sigma != nullptr;
+  for (int c = 0; c < 7; ++c) map = map || a.dst[c] != nullptr;
+  if (!map) {
+    // faces per warp: enough that full batches dominate, once every SM has warps
+    const long long least = (p->M + PB_WARPS * POSE_BLOCKS - 1) / (PB_WARPS * POSE_BLOCKS);
+    a.unit = p->M >= (1 << 16) ? (int)std::max<long long>(512, (least + 31) / 32 * 32) : (p->M >= (1 << 14) ? 128 : 32);
+    const long long nb = (p->M + PB_WARPS * a.unit - 1) / (PB_WARPS * a.unit);
+    const int smem = PB_T * (slot_stride(a.aux != nullptr) + PB_FS) * (int)sizeof(float);  // <= 28 KB
+    k_pbwd_pose<<<dim3((unsigned)nb, (unsigned)p->V), PB_T, smem, s>>>(a);
+    return cudaGetLastError();
   }
-  return cudaGetLastError();
+  // 32 faces a warp once every warp of the grid has some, fewer of smaller maps
+  if (p->M > MAP_BLOCKS * PB_WARPS * 16) return launch_pbwd_map<32>(a, s);
+  if (p->M > MAP_BLOCKS * PB_WARPS * 8) return launch_pbwd_map<16>(a, s);
+  return launch_pbwd_map<8>(a, s);
 }
 
 cudaError_t ts_launch_pose_reduce(const TsPlanImpl* p, const TsWs& w, float* dtau, cudaStream_t s) {
-  k_pose_reduce<<<p->V, 256, 0, s>>>(w.pose, (int)p->n_pose_blocks, dtau);
+  k_pose_reduce<<<p->V, 256, 0, s>>>(w.pose, (int)p->n_pose_blocks, w.hdr, dtau);
   return cudaGetLastError();
 }

@@ -13,7 +13,7 @@
 
 #define TS_PLAN_MAGIC 0x54535031u  // "TSP1"
 #define TS_REC_WORDS 32            // 128-byte record, a multiple of 16 B for cp.async.bulk
-#define TS_GRAD_WORDS 32           // per-(view, face) gradient slot: 24 accumulators + chain outputs
+#define TS_GRAD_WORDS 32           // per-(view, face) gradient slot: 24 accumulators, 32 with the side array
 #define TS_SCAN_ITEMS 4096         // items per scan block (1024 threads x 4)
 #define TS_BIN_FACES 8192          // faces per block of the shared-memory tile counts
 #define TS_BIN_MAX_TILES 40960     // the most tiles of a view those counts hold (160 KB)
@@ -46,9 +46,8 @@ enum {
 
 // Gradient word indices: G_E[i][k] = sum_p dL/dE_i * lambda_k (edge i nearest), G_c[ch][k] =
 // sum_p dL/dc_ch * lambda_k, G_z[k] = sum_p dL/dz * lambda_k, G_o = dL/do_F, count = pixels.
-// The raster backward accumulates words 0..23; the chain-rule pass then overwrites words
-// G_DPOS.. with the face's world-space vertex-position gradients and G_TAU.. with its pose terms.
-enum { G_E = 0, G_C = 9, G_Z = 18, G_O = 21, G_CNT = 22, G_DPOS = 0, G_TAU = 24 };
+// The raster backward accumulates words 0..23; the chain-rule pass reads them.
+enum { G_E = 0, G_C = 9, G_Z = 18, G_O = 21, G_CNT = 22 };
 
 struct TsView {
   float fx, fy, cx, cy;
@@ -80,7 +79,8 @@ struct TsDevHeader {
   long long n_vertices;
   unsigned int tile_counter;  // work counter of the persistent raster launches
   unsigned int n_large;       // tiles listed for the CTA-wide pair sort
-  unsigned int pad[12];
+  unsigned int pose_blocks;   // per-view pose partials the last backward wrote
+  unsigned int pad[11];
 };
 
 struct TsPlanImpl {
@@ -222,7 +222,7 @@ cudaError_t ts_launch_pose_apply(const TsPlanImpl* p, ts_pose* poses, const floa
 cudaError_t ts_launch_pose_adam(const TsPlanImpl* p, ts_pose* poses, const float* dtau, float* state, float lr_rho,
                                 float lr_theta, float b1, float b2, float eps, cudaStream_t s);
 cudaError_t ts_launch_timeout_probe(const TsWs& w, unsigned long long limit_ns, cudaStream_t s);
-int ts_pose_blocks(long long M);                 // blocks of the projection-backward kernel
+int ts_pose_blocks(long long M);                 // most blocks of the chain-rule pass (pose partials per view)
 // Streaming multiprocessors of the current device (queried once per device; 1 if the query fails).
 int ts_sm_count();
 cudaError_t ts_launch_sum_counters(const TsWs& w, cudaStream_t s);

@@ -1,10 +1,10 @@
 """Kernels at the sizes where their splits change: tile lists around the sort's register, warp and CTA
-limits (needs a GB300)."""
+limits, and the chain rule around its faces per warp (needs a GB300)."""
 import numpy as np
 import pytest
 
-from harness import gpu_run, params_pair
-from ts_synth.scenes import Scene
+from harness import assert_grad, assert_pose_grad, gpu_run, oracle_run, params_pair
+from ts_synth.scenes import Scene, noise_targets, random_triangles_scene
 
 pytestmark = pytest.mark.gpu
 
@@ -25,3 +25,31 @@ def test_tile_sort_list_lengths(n):
     order = np.lexsort((np.arange(n), zb))
     assert np.array_equal(rast.debug("ids").cpu().numpy().view(np.uint32)[:n], order)
     assert np.array_equal(rast.debug("keys").cpu().numpy().view(np.uint64)[:n], zb[order].astype(np.uint64))
+
+
+@pytest.mark.parametrize("n_faces", [1, 7, 33, 200])
+@pytest.mark.parametrize("n_views", [1, 2, 3, 7, 8, 33])
+def test_chain_rule_views_and_faces(oracle, n_views, n_faces):
+    """The chain rule with map gradients at every number of faces a warp takes, ragged ones included,
+    and the form without map gradients, whose pose gradient sums in another order."""
+    sc = random_triangles_scene(seed=n_faces, n_faces=n_faces, W=40, H=30, f=40.0, z_lo=1.0, z_hi=2.0, side_lo=0.2,
+                                side_hi=0.5)
+    poses = np.repeat(sc.poses[:1], n_views, axis=0).copy()
+    poses[:, 9] = np.linspace(-0.6, 0.6, n_views)  # some faces leave some views
+    sc = Scene(sc.pos, sc.col, sc.opa, None, np.repeat(sc.cams[:1], n_views, axis=0), poses)
+    sc.tgt_color, sc.tgt_depth = noise_targets(3, sc.cams)
+    sc.pair_capacity = 64 * n_views * n_faces
+    p, po = params_pair(sigma=1.0)
+    r = oracle_run(oracle, sc, po)
+    g = gpu_run(sc, p, dC=r["dC_used"], dD=r["dD_used"])
+    for k in ("dpos", "dcol", "dopa"):
+        assert_grad(g[k], r[k], k)
+    assert_pose_grad(g["dtau"], r["dtau"], r["dtau_abs"])
+    # the same backward without map gradients
+    import torch
+    import paper_2605_31419_gb300 as ts
+    rast = g["rast"]
+    rast.forward(ts.Map.from_numpy(sc.pos, sc.col, sc.opa), ts.poses_tensor(sc.poses))
+    dev = lambda a: torch.as_tensor(np.asarray(a), dtype=torch.float32, device="cuda")  # noqa: E731
+    rast.backward(dev(r["dC_used"]), dev(r["dD_used"]))
+    assert_pose_grad(rast.pose_grad().cpu().numpy().astype(np.float64), r["dtau"], r["dtau_abs"])
