@@ -1,17 +1,23 @@
 // k_render.cu -- Eq. 3-4 forward blend and its adjoint, one CTA per (view, tile) at a time.
 //
-// Staging: the tile's depth-sorted face ids select 128-byte records that the CTA copies into
-// shared memory with 16-byte cp.async copies (a warp moves four records per instruction; one
-// bulk copy per record was bound by its per-request cost); two buffers alternate so the next
-// stage streams in while the current one is blended.  Each warp owns an 8 x 4 pixel sub-block of
-// the tile; per stage, a mask per record says which sub-blocks can contain one of the face's
-// covered pixel centres, and each warp walks only the set bits of its own ballot over the stage.
+// Staging: the tile's depth-sorted face ids select 128-byte records, of which the CTA copies seven of
+// the eight 16-byte groups into shared memory with cp.async (two edge vectors are subtractions of the
+// staged vertices, rounded as the projection rounds them); two buffers alternate so the next stage
+// streams in while the current one is blended.  A staged record is 28 words long, so that 8 lanes
+// reading the same group of 8 consecutive records hit distinct banks.  Each warp owns an 8 x 4 pixel
+// sub-block of the tile.
 //
-// Forward: per pixel, front to back: window (Eq. 3) from cancellation-free edge functions,
-// alpha = min(alpha_max, o_F I), skip below alpha_min, stop before the face that would take T
-// below T_min, accumulate colour, depth and opacity (Eq. 4).  Writes C + T bg, D, A = 1 - T, and
-// per pixel T_final and the list position after the last contribution, and per sorted pair and
-// warp the mask of the warp's pixels that blended the face.
+// Forward: for 32 staged faces at a time, lane = face computes which of the warp's 32 pixels its face
+// can cover (per pixel row the interval between its edges, widened: conservative); a 32 x 32 bit
+// transpose gives every pixel the faces to visit, and then lane = pixel walks its own faces front to
+// back, two per pass: window (Eq. 3) from cancellation-free edge functions, alpha = min(alpha_max,
+// o_F I), skip below alpha_min, stop before the face that would take T below T_min, accumulate colour,
+// depth and opacity (Eq. 4).  A warp's cost is its longest pixel list instead of all the faces of its
+// sub-block, each of which 5 of 32 pixels blend: issue-bound either way, the forward of 9 views of a
+// 2M-face map went from 1182 to 688 us, of 64 tracking views from 878 to 687, and the fused step from
+// 1893 to 1645 us (20-view room) and 1823 to 1441 (12-view window), images bit for bit.  The transpose of the blended bits gives, per face, the mask of the warp's pixels that
+// blended it.  Writes C + T bg, D, A = 1 - T, per pixel T_final and the list position after the last
+// contribution, and per sorted pair and warp that mask.
 //
 // Backward: per pixel, back to front from that position: recover T_n = T_{n+1} / (1 - alpha_n),
 // keep the suffix sum S of later contributions (including the background term), form
@@ -92,7 +98,6 @@ constexpr int raster_min_blocks(int threads) {
 
 // Shared state of a render CTA.
 struct RenderSmem {
-  uint16_t smask[2][128];  // per staged face, the warps (sub-blocks) that visit it
   float lred[16][2];       // fused step: the warps' loss sums
   int lmax[16];            // fused step: the warps' largest last positions
   int view;
@@ -107,12 +112,12 @@ struct FwdMasks {
 };
 
 // What a tile's forward leaves for the backward of the fused step, per pixel (thread) and for the
-// stage buffers: the last stage processed, its buffer, and whether the stage before it is still in
-// the other buffer.
+// stage buffers: the last stage processed (in buffer st & 1), and whether the stage before it is still
+// in the other buffer.
 struct TileCarry {
   float T, C0, C1, C2, D;
   int nl;
-  int st_last, b_last;
+  int st_last;
   bool prev_in;
 };
 
@@ -173,17 +178,19 @@ __device__ __forceinline__ TileGeom<TW, TH> tile_geom(const RenderArgs& a, long 
   return g;
 }
 
-// Every thread of the CTA copies 16-byte chunks of stage `st` (records [st*S, st*S + cnt) of the
-// tile's list) into buffer `b` with cp.async, eight chunks per record and, with the side array,
-// one more for the record's side entry (normal, sigma_F) after both record buffers; one commit
-// group per stage.  A warp moves four records per instruction, and no copy engine request is
-// made per record.
+// 16-byte groups of a staged record: groups 0, 1 and 3..7 of the record (group 2 holds the edge vectors
+// e1 and e2).
+constexpr int SG = 7;
+
+// Every thread of the CTA copies 16-byte groups of stage `st` (records [st*S, st*S + cnt) of the
+// tile's list) into buffer `b` with cp.async, SG groups per record and, with the side array, one more
+// for the record's side entry (normal, sigma_F) after both record buffers; one commit group per stage.
 template <bool AUX>
 __device__ __forceinline__ void issue_stage(const RenderArgs& a, float4* smrec, int b, int st, uint32_t start, int n,
                                             const float4* vbase, const float4* nbase, int nthreads) {
   const int S = a.S;
   const int cnt = min(S, n - st * S);
-  constexpr int PER = AUX ? 9 : 8;
+  constexpr int PER = AUX ? SG + 1 : SG;
   for (int i = threadIdx.x; i < cnt * PER; i += nthreads) {
     const int j = i / PER, c = i - j * PER;
     uint32_t id = __ldg(a.ids + start + (uint32_t)(st * S + j));
@@ -191,53 +198,14 @@ __device__ __forceinline__ void issue_stage(const RenderArgs& a, float4* smrec, 
       atomicOr(&a.hdr->error_bits, TS_ERRBIT_BOUNDS);
       id = 0;
     }
-    if (!AUX || c < 8) {
-      ts_cp_async16(smrec + ((size_t)b * S + j) * 8 + c, vbase + (size_t)id * 8 + c);
+    if (!AUX || c < SG) {
+      ts_cp_async16(smrec + ((size_t)b * S + j) * SG + c, vbase + (size_t)id * 8 + (c < 2 ? c : c + 1));
     } else {
-      ts_cp_async16(smrec + (size_t)2 * S * 8 + (size_t)b * S + j, nbase + id);
+      ts_cp_async16(smrec + (size_t)2 * S * SG + (size_t)b * S + j, nbase + id);
     }
   }
   ts_cp_async_commit();
 }
-
-// For each staged record, the mask of warp sub-blocks (8 x 4 pixels) that can contain one of its
-// covered pixel centres: sub-blocks inside the face's pixel box whose pixel-centre rectangle,
-// widened by 0.01 px, is not entirely outside one of the three edges.  Conservative: a pixel with
-// a positive window always keeps its sub-block's bit.
-template <int TW, int TH>
-__device__ __forceinline__ void stage_masks(const float* rb, uint16_t* smask, int cnt, int X0, int Y0) {
-  constexpr int NSBX = TW / 8;
-  for (int j = threadIdx.x; j < cnt; j += TW * TH) {
-    const float* r = rb + j * TS_REC_WORDS;
-    const uint32_t bx = __float_as_uint(r[R_BOXX]), by = __float_as_uint(r[R_BOXY]);
-    const int x0 = (int)(bx & 0xffffu) - X0, x1 = (int)(bx >> 16) - X0;
-    const int y0 = (int)(by & 0xffffu) - Y0, y1 = (int)(by >> 16) - Y0;
-    uint32_t mask = 0;
-    if (x1 >= 0 && x0 < TW && y1 >= 0 && y0 < TH) {
-      const int c0 = max(x0, 0) >> 3, c1 = min(x1, TW - 1) >> 3;
-      const int r0 = max(y0, 0) >> 2, r1 = min(y1, TH - 1) >> 2;
-      const float sgn = r[R_INVD] > 0.f ? 1.f : -1.f;
-      const float qx[3] = {r[R_U0], r[R_U1], r[R_U2]}, qy[3] = {r[R_V0], r[R_V1], r[R_V2]};
-      const float ex[3] = {r[R_E0X], r[R_E1X], r[R_E2X]}, ey[3] = {r[R_E0Y], r[R_E1Y], r[R_E2Y]};
-      for (int rr = r0; rr <= r1; ++rr) {
-        const float cy = (float)(Y0 + rr * 4) + 2.0f;  // centre of the sub-block's pixel centres
-        for (int cc = c0; cc <= c1; ++cc) {
-          const float cx = (float)(X0 + cc * 8) + 4.0f;
-          bool in = true;
-#pragma unroll
-          for (int i = 0; i < 3; ++i) {
-            const float f = sgn * (ex[i] * (cy - qy[i]) - ey[i] * (cx - qx[i])) + fabsf(ey[i]) * 3.51f +
-                            fabsf(ex[i]) * 1.51f;
-            in = in && f > 0.f;
-          }
-          if (in) mask |= 1u << (rr * NSBX + cc);
-        }
-      }
-    }
-    smask[j] = (uint16_t)mask;
-  }
-}
-
 
 // Wait for the stage issued last: each thread's copies (they always complete), then a barrier.
 __device__ __forceinline__ void wait_stage() {
@@ -245,10 +213,88 @@ __device__ __forceinline__ void wait_stage() {
   __syncthreads();
 }
 
-// Forward of one tile; seq counts the stages this CTA has staged so far (buffer seq & 1 is next).
+static_assert(R_U0 == 0 && R_V0 == 3 && R_V1 == 4 && R_E0X == 6 && R_E1X == 8 && R_E2X == 10 && R_K0 == 12 &&
+                  R_INVD == 15 && R_OF == 16 && R_C0 == 17 && R_C1 == 20 && R_C2 == 23 && R_Z0 == 26 && R_Z2 == 28 &&
+                  R_SLOT == 31,
+              "record layout assumed by the staged groups");
+
+// The edge evaluation (cross products, normalised edge functions, their minimum) from a staged
+// record's groups 0..2: u, v, e0 and k, 1 / D2.  e1 and e2 are the projection's own subtractions.
+__device__ __forceinline__ TsPix eval_edges(float4 q0, float4 q1, float4 qk, float px, float py) {
+  TsPix o;
+  o.cr0 = ts_det2(q1.z, q1.w, px - q0.x, py - q0.w);
+  o.cr1 = ts_det2(__fsub_rn(q0.z, q0.y), __fsub_rn(q1.y, q1.x), px - q0.y, py - q1.x);
+  o.cr2 = ts_det2(__fsub_rn(q0.x, q0.z), __fsub_rn(q0.w, q1.y), px - q0.z, py - q1.y);
+  const float e0 = o.cr0 * qk.x, e1 = o.cr1 * qk.y, e2 = o.cr2 * qk.z;
+  o.m = e0;
+  o.arg = 0;
+  if (e1 < o.m) { o.m = e1; o.arg = 1; }
+  if (e2 < o.m) { o.m = e2; o.arg = 2; }
+  return o;
+}
+
+// Conservative cover of one staged face in an 8 x 4 pixel block whose first pixel centre is (px, py):
+// bit 8 r + c set when pixel (c, r) can have a positive window.  Per edge, the pixels inside satisfy
+// f(c, r) = g + r a - c b > 0 (a, b the edge vector turned so that inside is positive, g the edge
+// function at the block's first centre), i.e. c lies below or above (g + r a) / b; every row's interval
+// is the intersection of its edges'.  g is widened by what moves the edge 0.01 px and by the rounding
+// of its own terms (relevant for vertices far outside the image).
+__device__ __forceinline__ unsigned block_cover(const float4* r4, float px, float py) {
+  const float4 q0 = r4[0], q1 = r4[1];
+  const float sg = r4[2].w > 0.f ? 1.f : -1.f;
+  const float u[3] = {q0.x, q0.y, q0.z}, v[3] = {q0.w, q1.x, q1.y};
+  // columns cut off at the right (hi) and at the left (lo) of each row
+  float hi[4] = {0.f, 0.f, 0.f, 0.f}, lo[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const int j = (i + 1) % 3;
+    const float a = sg * (u[j] - u[i]), b = sg * (v[j] - v[i]);
+    const float ya = a * (py - v[i]), xb = b * (px - u[i]);
+    const float g = (ya - xb) + (0.01f * (fabsf(a) + fabsf(b)) + 1e-6f * (fabsf(ya) + fabsf(xb)));
+    const float ib = ts_rcp_approx(fabsf(b));  // b = 0: infinite or NaN cuts, which cut nothing or everything
+    const bool right = b > 0.f;
+    // cut at the right: 7 - floor(t), at the left: ceil(t), t = (g + r a) / b; both -(g + r a) / |b| + a
+    // constant, rounded to nearest below with 0.499 for the floor and the ceiling
+    const float c0 = fmaf(-g, ib, right ? 7.499f : 0.499f), cs = -a * ib;
+    if (right) {
+      hi[0] = fmaxf(hi[0], c0);
+#pragma unroll
+      for (int r = 1; r < 4; ++r) hi[r] = fmaxf(hi[r], fmaf((float)r, cs, c0));
+    } else {
+      lo[0] = fmaxf(lo[0], c0);
+#pragma unroll
+      for (int r = 1; r < 4; ++r) lo[r] = fmaxf(lo[r], fmaf((float)r, cs, c0));
+    }
+  }
+  constexpr float MAGIC = 12582912.f;  // 1.5 * 2^23: adding it rounds to an integer in the low bits
+  unsigned cover = 0u;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const unsigned h = __float_as_uint(fminf(hi[r], 8.f) + MAGIC) & 15u;
+    const unsigned l = __float_as_uint(fminf(lo[r], 8.f) + MAGIC) & 15u;
+    cover |= ((0xffu >> h) & (0xffu << l)) << (8 * r);
+  }
+  return cover;
+}
+
+// Transpose of a 32 x 32 bit matrix, lane r holding row r: five exchanges of off-diagonal blocks.
+__device__ __forceinline__ unsigned transpose32(unsigned x, int lane) {
+#pragma unroll
+  for (int j = 16; j > 0; j >>= 1) {
+    const unsigned low = j == 16 ? 0x0000ffffu : j == 8 ? 0x00ff00ffu : j == 4 ? 0x0f0f0f0fu : j == 2 ? 0x33333333u : 0x55555555u;
+    const unsigned y = __shfl_xor_sync(FULL, x, j);
+    const bool upper = (lane & j) != 0;
+    const unsigned take = upper ? low : ~low;  // the bits that come from the partner
+    const unsigned rot = __funnelshift_l(y, y, upper ? 32 - j : j);
+    x = (x & ~take) | (rot & take);
+  }
+  return x;
+}
+
+// Forward of one tile.  Stage st is staged in buffer st & 1.
 template <int TW, int TH, bool AUX, bool FUSED = false>
 __device__ __forceinline__ void fwd_tile(const RenderArgs& a, long long tile, float4* smrec, RenderSmem& sm,
-                                         FwdMasks& fm, int& seq, TileCarry* carry = nullptr,
+                                         FwdMasks& fm, TileCarry* carry = nullptr,
                                          const TileGeom<TW, TH>* gin = nullptr) {
   const TileGeom<TW, TH> g = FUSED ? *gin : tile_geom<TW, TH>(a, tile, sm);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -259,104 +305,110 @@ __device__ __forceinline__ void fwd_tile(const RenderArgs& a, long long tile, fl
   int nl = 0;
   bool done = !g.inimg;
   unsigned contrib = 0;
-  int st_last = -1, b_last = 0;
+  int st_last = -1;
   bool prefetched = false;
   if (n > 0) {
     const int S = a.S;
     const int nst = (n + S - 1) / S;
     const float4* vbase = a.frec + (size_t)g.view * (size_t)a.M * 8;
     const float4* nbase = AUX ? a.aux + (size_t)g.view * (size_t)a.M : nullptr;
-    issue_stage<AUX>(a, smrec, seq & 1, 0, rg.x, n, vbase, nbase, TW * TH);
+    const float bx = g.px - (float)(lane & 7), by = g.py - (float)(lane >> 3);  // the warp's first pixel centre
+    issue_stage<AUX>(a, smrec, 0, 0, rg.x, n, vbase, nbase, TW * TH);
+    if (a.cov)
+      for (int j = threadIdx.x; j < 2 * 128; j += TW * TH) (&fm.cv[0][0])[j] = 0u;
+    wait_stage();
     for (int st = 0; st < nst; ++st) {
-      const int b = seq & 1;
+      const int b = st & 1;
       const int cnt = min(S, n - st * S);
-      wait_stage();
-      ++seq;
       st_last = st;
-      b_last = b;
-      const float* rb = reinterpret_cast<const float*>(smrec + (size_t)b * S * 8);
-      const float4* nb = smrec + (size_t)2 * S * 8 + (size_t)b * S;
-      stage_masks<TW, TH>(rb, sm.smask[b], cnt, g.X0, g.Y0);
-      if (a.cov)
-        for (int j = threadIdx.x; j < cnt; j += TW * TH) fm.cv[b][j] = 0u;
-      __syncthreads();
+      // every warp is done with the other buffer (the barrier that ended the stage before)
       if (st + 1 < nst) issue_stage<AUX>(a, smrec, b ^ 1, st + 1, rg.x, n, vbase, nbase, TW * TH);
+      const float4* rb = smrec + (size_t)b * S * SG;
+      const float4* nb = smrec + (size_t)2 * S * SG + (size_t)b * S;
       for (int q = 0; q * 32 < cnt; ++q) {
         const int jq = q * 32 + lane;
-        unsigned lm = 0;  // lane L: this warp's pixels that blended face q * 32 + L
-        unsigned bits = __ballot_sync(FULL, jq < cnt && ((sm.smask[b][min(jq, cnt - 1)] >> warp) & 1u));
-        while (bits) {
-          const int j0 = q * 32 + __ffs(bits) - 1;
-          bits &= bits - 1;
-          const bool two = bits != 0;
-          const int j1 = two ? q * 32 + __ffs(bits) - 1 : j0;
-          if (two) bits &= bits - 1;
-          // two faces per pass: both edge functions first (independent work the scheduler can overlap),
-          // then the compositing in list order, exactly as one face at a time
-          const float* r0 = rb + j0 * TS_REC_WORDS;
-          const float* r1 = rb + j1 * TS_REC_WORDS;
-          const TsPix e0 = ts_eval_edges(r0, g.px, g.py);
-          const TsPix e1 = ts_eval_edges(r1, g.px, g.py);
+        unsigned lm = 0;  // this warp's pixels that blended face jq
+        if (!__all_sync(FULL, done)) {
+          unsigned bits = jq < cnt ? block_cover(rb + jq * SG, bx, by) : 0u;
+          if (__any_sync(FULL, bits != 0u)) {
+            bits = transpose32(bits, lane);  // this pixel's faces
+            if (done) bits = 0u;
+            unsigned blended = 0u;
+            while (bits) {
+              const int j0 = __ffs(bits) - 1;
+              bits &= bits - 1;
+              const bool two = bits != 0;
+              const int j1 = two ? __ffs(bits) - 1 : j0;
+              bits &= bits - 1;
+              // two faces per pass: both edge functions first (independent work the scheduler can overlap),
+              // then the compositing in list order, exactly as one face at a time
+              const float4* r0 = rb + (q * 32 + j0) * SG;
+              const float4* r1 = rb + (q * 32 + j1) * SG;
+              const float4 k0 = r0[2], k1 = r1[2];
+              const TsPix e0 = eval_edges(r0[0], r0[1], k0, g.px, g.py);
+              const TsPix e1 = eval_edges(r1[0], r1[1], k1, g.px, g.py);
 #pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            if (h == 1 && !two) break;
-            const int j = h ? j1 : j0;
-            const float* r = h ? r1 : r0;
-            const TsPix e = h ? e1 : e0;
-            bool blended = false;
-            if (!done && e.m > 0.f) {
-              const float sig = (AUX && a.face_sigma) ? nb[j].w : a.sigma;
-              const float I = ts_window(e.m, sig);
-              const float al = fminf(r[R_OF] * I, a.alpha_max);
-              if (al >= a.alpha_min) {
-                const float Tn = T * (1.f - al);
-                if (Tn < a.T_min) {
-                  done = true;
-                } else {
-                  const float invD = r[R_INVD];
-                  const float l0 = e.cr1 * invD, l1 = e.cr2 * invD, l2 = e.cr0 * invD;
-                  const float w = al * T;
-                  C0 += w * (l0 * r[R_C0] + l1 * r[R_C1] + l2 * r[R_C2]);
-                  C1 += w * (l0 * r[R_C0 + 1] + l1 * r[R_C1 + 1] + l2 * r[R_C2 + 1]);
-                  C2 += w * (l0 * r[R_C0 + 2] + l1 * r[R_C1 + 2] + l2 * r[R_C2 + 2]);
-                  D += w * (l0 * r[R_Z0] + l1 * r[R_Z1] + l2 * r[R_Z2]);
-                  if (AUX && a.normals) {
-                    const float4 nn = nb[j];
-                    N0 += w * nn.x;
-                    N1 += w * nn.y;
-                    N2 += w * nn.z;
+              for (int h = 0; h < 2; ++h) {
+                if (h == 1 && !two) break;
+                const int j = h ? j1 : j0;
+                const float4* r = h ? r1 : r0;
+                const TsPix e = h ? e1 : e0;
+                if (!done && e.m > 0.f) {
+                  const float4 q4 = r[3];  // o_F, colour of vertex 0
+                  const float sig = (AUX && a.face_sigma) ? nb[q * 32 + j].w : a.sigma;
+                  const float I = ts_window(e.m, sig);
+                  const float al = fminf(q4.x * I, a.alpha_max);
+                  if (al >= a.alpha_min) {
+                    const float Tn = T * (1.f - al);
+                    if (Tn < a.T_min) {
+                      done = true;
+                      bits = 0u;
+                    } else {
+                      const float invD = h ? k1.w : k0.w;
+                      const float l0 = e.cr1 * invD, l1 = e.cr2 * invD, l2 = e.cr0 * invD;
+                      const float w = al * T;
+                      const float4 q5 = r[4], q6 = r[5];  // colours of vertices 1 and 2, depths z_0, z_1
+                      C0 += w * (l0 * q4.y + l1 * q5.x + l2 * q5.w);
+                      C1 += w * (l0 * q4.z + l1 * q5.y + l2 * q6.x);
+                      C2 += w * (l0 * q4.w + l1 * q5.z + l2 * q6.y);
+                      D += w * (l0 * q6.z + l1 * q6.w + l2 * r[6].x);
+                      if (AUX && a.normals) {
+                        const float4 nn = nb[q * 32 + j];
+                        N0 += w * nn.x;
+                        N1 += w * nn.y;
+                        N2 += w * nn.z;
+                      }
+                      T = Tn;
+                      nl = st * S + q * 32 + j + 1;
+                      blended |= 1u << j;
+                    }
                   }
-                  T = Tn;
-                  nl = st * S + j + 1;
-                  ++contrib;
-                  blended = true;
                 }
               }
             }
+            contrib += __popc(blended);
             // the backward takes exactly these (face, pixel) contributions
-            const unsigned bl = __ballot_sync(FULL, blended);
-            if (lane == (j & 31)) lm = bl;
-            if (bl && lane == 0 && a.cov) atomicAdd(&fm.cv[b][j], (unsigned)__popc(bl));
+            if (a.lmask || a.cov) lm = transpose32(blended, lane);
+            if (a.cov && lm) atomicAdd(&fm.cv[b][jq], (unsigned)__popc(lm));
           }
         }
         if (a.lmask && jq < cnt) a.lmask[(size_t)(rg.x + (uint32_t)(st * S + jq)) * (TW * TH / 32) + warp] = lm;
       }
+      if (st + 1 == nst && !a.cov) break;  // nothing reads the buffers or the counts after this stage
+      ts_cp_async_wait_all();              // the next stage, published by the barrier
       const int alive = __syncthreads_count(!done);
       if (a.cov) {
         for (int j = threadIdx.x; j < cnt; j += TW * TH) {
           if (fm.cv[b][j]) {  // face m of the record's slot m * V + view
-            const uint32_t slot = __float_as_uint(rb[j * TS_REC_WORDS + R_SLOT]);
+            const uint32_t slot = __float_as_uint(rb[j * SG + 6].w);
             const long long m = (long long)(slot / (uint32_t)a.V);
             if (m < a.M) atomicAdd(a.cov + (long long)g.view * a.M + m, fm.cv[b][j]);
+            fm.cv[b][j] = 0u;  // for the stage after next, a barrier away
           }
         }
       }
       if (alive == 0) {
-        if (st + 1 < nst) {  // a prefetched stage is in flight: let it land before leaving
-          wait_stage();
-          ++seq;
-          prefetched = true;
-        }
+        prefetched = st + 1 < nst;
         break;
       }
     }
@@ -370,7 +422,6 @@ __device__ __forceinline__ void fwd_tile(const RenderArgs& a, long long tile, fl
     carry->D = D;
     carry->nl = nl;
     carry->st_last = st_last;
-    carry->b_last = b_last;
     carry->prev_in = st_last >= 1 && !prefetched;
   }
   if (g.inimg) {
@@ -430,27 +481,9 @@ __device__ __forceinline__ bool ring_word(int lane, int& ia, int& ib) {
   return true;
 }
 
-// The edge evaluation of ts_eval_edges from the record's first four 16-byte groups (one vector
-// load each; lanes holding different faces then conflict only within a quarter warp).
-static_assert(R_U0 == 0 && R_V0 == 3 && R_V1 == 4 && R_E0X == 6 && R_E1X == 8 && R_E2X == 10 && R_K0 == 12 &&
-                  R_INVD == 15 && R_OF == 16 && R_C0 == 17 && R_C1 == 20 && R_C2 == 23 && R_Z0 == 26 && R_Z2 == 28,
-              "record layout assumed by the vector loads");
-__device__ __forceinline__ TsPix eval_edges_v(float4 q0, float4 q1, float4 q2, float4 q3, float px, float py) {
-  TsPix o;
-  o.cr0 = ts_det2(q1.z, q1.w, px - q0.x, py - q0.w);
-  o.cr1 = ts_det2(q2.x, q2.y, px - q0.y, py - q1.x);
-  o.cr2 = ts_det2(q2.z, q2.w, px - q0.z, py - q1.y);
-  const float e0 = o.cr0 * q3.x, e1 = o.cr1 * q3.y, e2 = o.cr2 * q3.z;
-  o.m = e0;
-  o.arg = 0;
-  if (e1 < o.m) { o.m = e1; o.arg = 1; }
-  if (e2 < o.m) { o.m = e2; o.arg = 2; }
-  return o;
-}
-
 template <int TW, int TH, bool AUX, bool FUSED = false>
 __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, float4* smrec, RenderSmem& sm,
-                                         int& seq, const PixIn* pin = nullptr, const TileCarry* carry = nullptr,
+                                         const PixIn* pin = nullptr, const TileCarry* carry = nullptr,
                                          const TileGeom<TW, TH>* gin = nullptr) {
   const TileGeom<TW, TH> g = FUSED ? *gin : tile_geom<TW, TH>(a, tile, sm);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -510,9 +543,9 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
     const int nst = (n + S - 1) / S;
     const float4* vbase = a.frec + (size_t)g.view * (size_t)a.M * 8;
     const float4* nbase = AUX ? a.aux + (size_t)g.view * (size_t)a.M : nullptr;
-    if (!FUSED) issue_stage<AUX>(a, smrec, seq & 1, nst - 1, rg.x, n, vbase, nbase, TW * TH);
+    if (!FUSED) issue_stage<AUX>(a, smrec, (nst - 1) & 1, nst - 1, rg.x, n, vbase, nbase, TW * TH);
     constexpr int EW = Ring<AUX>::EW;
-    unsigned char* wbase = reinterpret_cast<unsigned char*>(smrec + (size_t)2 * S * (AUX ? 9 : 8)) +
+    unsigned char* wbase = reinterpret_cast<unsigned char*>(smrec + (size_t)2 * S * (AUX ? SG + 1 : SG)) +
                            (size_t)warp * Ring<AUX>::BYTES_PER_WARP;
     float* ring = reinterpret_cast<float*>(wbase);
     float2* pst = reinterpret_cast<float2*>(wbase + RING_CAP * EW * 4);  // per pixel lane: (T, S)
@@ -522,7 +555,7 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
     const int xw = g.x - (lane & 7), yw = g.y - (lane >> 3);  // the warp's first pixel
     for (int k = 0; k < nst; ++k) {
       const int st = nst - 1 - k;
-      int b = seq & 1;
+      int b = st & 1;
       const int cnt = min(S, n - st * S);
       // The forward's lane masks (positions below the tile's largest list position after a
       // contribution were all written by it) give, per face, the pixels of this warp that blended
@@ -542,11 +575,7 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
       if (FUSED) {
         // the forward's last stage, and the one before it unless a prefetch replaced it, are
         // still staged; other stages are staged again (all warps are done with both buffers)
-        if (st == carry->st_last) {
-          b = carry->b_last;
-        } else if (st == carry->st_last - 1 && carry->prev_in) {
-          b = carry->b_last ^ 1;
-        } else {
+        if (st != carry->st_last && !(st == carry->st_last - 1 && carry->prev_in)) {
           __syncthreads();
           b = 0;
           issue_stage<AUX>(a, smrec, b, st, rg.x, n, vbase, nbase, TW * TH);
@@ -554,11 +583,10 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
         }
       } else {
         wait_stage();
-        ++seq;
         if (k + 1 < nst) issue_stage<AUX>(a, smrec, b ^ 1, st - 1, rg.x, n, vbase, nbase, TW * TH);
       }
-      const float* rb = reinterpret_cast<const float*>(smrec + (size_t)b * S * 8);
-      const float4* nb = smrec + (size_t)2 * S * 8 + (size_t)b * S;
+      const float4* rb = smrec + (size_t)b * S * SG;
+      const float4* nb = smrec + (size_t)2 * S * SG + (size_t)b * S;
       {
         // lane L's faces have popc of their masks entries; their numbers start at the exclusive
         // scan over the lanes, face by face within a lane
@@ -617,12 +645,12 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
           const int j = act ? F * (32 - ow) - 1 - fi : 0;
           const int p = act ? pb : lane;
           // -- one entry per lane: face j at pixel lane p ---------------------------------------
-          const float4* r4 = reinterpret_cast<const float4*>(rb + j * TS_REC_WORDS);
+          const float4* r4 = rb + j * SG;
           const float px = (float)(xw + (p & 7)) + 0.5f, py = (float)(yw + (p >> 3)) + 0.5f;
           const float sig = (AUX && a.face_sigma) ? nb[j].w : a.sigma;
-          const float4 q3 = r4[3];  // k_0, k_1, k_2, invD
-          const TsPix e = eval_edges_v(r4[0], r4[1], r4[2], q3, px, py);
-          const float4 q4 = r4[4];  // o_F, colour of vertex 0
+          const float4 q3 = r4[2];  // k_0, k_1, k_2, invD
+          const TsPix e = eval_edges(r4[0], r4[1], q3, px, py);
+          const float4 q4 = r4[3];  // o_F, colour of vertex 0
           const float oF = q4.x;
           const float I = act ? ts_window(e.m, sig) : 0.f;
           const float al = fminf(oF * I, a.alpha_max);
@@ -654,8 +682,8 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
           }
           const float invD = q3.w;
           const float l0 = e.cr1 * invD, l1 = e.cr2 * invD, l2 = e.cr0 * invD;
-          const float4 q5 = r4[5], q6 = r4[6];  // colours of vertices 1 and 2, depths z_0, z_1
-          const float4 q7 = r4[7];
+          const float4 q5 = r4[4], q6 = r4[5];  // colours of vertices 1 and 2, depths z_0, z_1
+          const float4 q7 = r4[6];
           const float z2 = q7.x;
           const uint32_t slot = __float_as_uint(q7.w);
           const float c0 = l0 * q4.y + l1 * q5.x + l2 * q5.w;
@@ -737,10 +765,10 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
 // ts_l1_loss and ts_render_bwd give, without the images' round trip through memory.
 template <int TW, int TH>
 __device__ __forceinline__ void step_tile(const RenderArgs& a, long long tile, float4* smrec, RenderSmem& sm,
-                                          FwdMasks& fm, int& seq) {
+                                          FwdMasks& fm) {
   TileCarry c;
   const TileGeom<TW, TH> g = tile_geom<TW, TH>(a, tile, sm);
-  fwd_tile<TW, TH, false, true>(a, tile, smrec, sm, fm, seq, &c, &g);
+  fwd_tile<TW, TH, false, true>(a, tile, smrec, sm, fm, &c, &g);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   PixIn pin{c.T, 0.f, 0.f, 0.f, 0.f, c.nl, 0};
   float lc = 0.f, ld = 0.f;
@@ -789,7 +817,7 @@ __device__ __forceinline__ void step_tile(const RenderArgs& a, long long tile, f
   }
 #pragma unroll
   for (int w = 0; w < TW * TH / 32; ++w) pin.nmax = max(pin.nmax, sm.lmax[w]);
-  bwd_tile<TW, TH, false, true>(a, tile, smrec, sm, seq, &pin, &c, &g);
+  bwd_tile<TW, TH, false, true>(a, tile, smrec, sm, &pin, &c, &g);
 }
 
 // Next tile of a persistent CTA (the same value in every thread), or -1 when none is left.
@@ -805,12 +833,11 @@ __global__ void __launch_bounds__(TW * TH, raster_min_blocks(TW * TH)) k_render_
   extern __shared__ __align__(128) float4 smrec[];
   __shared__ RenderSmem sm;
   __shared__ FwdMasks fm;
-  int seq = 0;
   if constexpr (!PERSIST) {
-    fwd_tile<TW, TH, AUX>(a, blockIdx.x, smrec, sm, fm, seq);
+    fwd_tile<TW, TH, AUX>(a, blockIdx.x, smrec, sm, fm);
   } else {
     for (long long t = next_tile(a, sm); t >= 0; t = next_tile(a, sm))
-      fwd_tile<TW, TH, AUX>(a, t, smrec, sm, fm, seq);
+      fwd_tile<TW, TH, AUX>(a, t, smrec, sm, fm);
   }
 }
 
@@ -818,12 +845,11 @@ template <int TW, int TH, bool PERSIST, bool AUX>
 __global__ void __launch_bounds__(TW * TH, raster_min_blocks(TW * TH)) k_render_bwd(RenderArgs a) {
   extern __shared__ __align__(128) float4 smrec[];
   __shared__ RenderSmem sm;
-  int seq = 0;
   if constexpr (!PERSIST) {
-    bwd_tile<TW, TH, AUX>(a, blockIdx.x, smrec, sm, seq);
+    bwd_tile<TW, TH, AUX>(a, blockIdx.x, smrec, sm);
   } else {
     for (long long t = next_tile(a, sm); t >= 0; t = next_tile(a, sm))
-      bwd_tile<TW, TH, AUX>(a, t, smrec, sm, seq);
+      bwd_tile<TW, TH, AUX>(a, t, smrec, sm);
   }
 }
 
@@ -834,12 +860,11 @@ __global__ void __launch_bounds__(TW * TH, raster_min_blocks(TW * TH)) k_render_
   extern __shared__ __align__(128) float4 smrec[];
   __shared__ RenderSmem sm;
   static_assert(sizeof(FwdMasks) <= (TW * TH / 32) * Ring<false>::BYTES_PER_WARP, "coverage counts fit the rings");
-  FwdMasks& fm = *reinterpret_cast<FwdMasks*>(smrec + (size_t)2 * a.S * 8);
-  int seq = 0;
+  FwdMasks& fm = *reinterpret_cast<FwdMasks*>(smrec + (size_t)2 * a.S * SG);
   if constexpr (!PERSIST) {
-    step_tile<TW, TH>(a, blockIdx.x, smrec, sm, fm, seq);
+    step_tile<TW, TH>(a, blockIdx.x, smrec, sm, fm);
   } else {
-    for (long long t = next_tile(a, sm); t >= 0; t = next_tile(a, sm)) step_tile<TW, TH>(a, t, smrec, sm, fm, seq);
+    for (long long t = next_tile(a, sm); t >= 0; t = next_tile(a, sm)) step_tile<TW, TH>(a, t, smrec, sm, fm);
   }
 }
 
@@ -872,7 +897,7 @@ __global__ void __launch_bounds__(256) k_loss_tiles(const TsView* __restrict__ v
 
 template <int TW, int TH>
 cudaError_t launch_step(bool persist, const RenderArgs& a, cudaStream_t s) {
-  const size_t smem = (size_t)2 * a.S * 128 + (size_t)(TW * TH / 32) * Ring<false>::BYTES_PER_WARP;
+  const size_t smem = (size_t)2 * a.S * SG * 16 + (size_t)(TW * TH / 32) * Ring<false>::BYTES_PER_WARP;
   if (a.n_tiles == 0) return cudaSuccess;
   const void* f = persist ? (const void*)k_render_step<TW, TH, true> : (const void*)k_render_step<TW, TH, false>;
   cudaError_t e = ts_smem_limit(f, (int)smem);
@@ -892,11 +917,11 @@ cudaError_t launch_step(bool persist, const RenderArgs& a, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-// Dynamic shared memory: two stage buffers of S 128-byte records, then (with the side array) two
+// Dynamic shared memory: two stage buffers of S staged records, then (with the side array) two
 // of S 16-byte side entries, then in the backward the warps' rings and their headers.
 template <int TW, int TH, bool AUX>
 cudaError_t launch_pair(bool fwd, bool persist, const RenderArgs& a, cudaStream_t s) {
-  const size_t smem = (size_t)2 * a.S * (AUX ? 144 : 128) + (fwd ? 0 : (size_t)(TW * TH / 32) * Ring<AUX>::BYTES_PER_WARP);
+  const size_t smem = (size_t)2 * a.S * (AUX ? SG + 1 : SG) * 16 + (fwd ? 0 : (size_t)(TW * TH / 32) * Ring<AUX>::BYTES_PER_WARP);
   if (a.n_tiles == 0) return cudaSuccess;
   {
     const void* f = fwd ? (persist ? (const void*)k_render_fwd<TW, TH, true, AUX> : (const void*)k_render_fwd<TW, TH, false, AUX>)

@@ -41,8 +41,6 @@ enum {
   R_OF, R_C0 = 17, R_C1 = 20, R_C2 = 23, R_Z0 = 26, R_Z1, R_Z2,
   R_BOXX = 29, R_BOXY = 30, R_SLOT = 31
 };
-// In shared memory the render kernels overwrite R_BOXY with the per-warp sub-block mask.
-#define R_MASK R_BOXY
 
 // Gradient word indices: G_E[i][k] = sum_p dL/dE_i * lambda_k (edge i nearest), G_c[ch][k] =
 // sum_p dL/dc_ch * lambda_k, G_z[k] = sum_p dL/dz * lambda_k, G_o = dL/do_F, count = pixels.
@@ -282,19 +280,6 @@ struct TsPix {
   float m;              // min_i E_i
   int arg;              // argmin
 };
-
-__device__ __forceinline__ TsPix ts_eval_edges(const float* r, float px, float py) {
-  TsPix o;
-  o.cr0 = ts_det2(r[R_E0X], r[R_E0Y], px - r[R_U0], py - r[R_V0]);
-  o.cr1 = ts_det2(r[R_E1X], r[R_E1Y], px - r[R_U1], py - r[R_V1]);
-  o.cr2 = ts_det2(r[R_E2X], r[R_E2Y], px - r[R_U2], py - r[R_V2]);
-  const float e0 = o.cr0 * r[R_K0], e1 = o.cr1 * r[R_K1], e2 = o.cr2 * r[R_K2];
-  o.m = e0;
-  o.arg = 0;
-  if (e1 < o.m) { o.m = e1; o.arg = 1; }
-  if (e2 < o.m) { o.m = e2; o.arg = 2; }
-  return o;
-}
 
 __device__ __forceinline__ float ts_sqrt_approx(float x) {
   float r;

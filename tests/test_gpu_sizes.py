@@ -1,9 +1,9 @@
 """Kernels at the sizes where their splits change: tile lists around the sort's register, warp and CTA
-limits, and the chain rule around its faces per warp (needs a GB300)."""
+limits, the chain rule around its faces per warp, the forward's pixel lists (needs a GB300)."""
 import numpy as np
 import pytest
 
-from harness import assert_grad, assert_pose_grad, gpu_run, oracle_run, params_pair
+from harness import assert_grad, assert_images, assert_pose_grad, gpu_run, oracle_run, params_pair
 from ts_synth.scenes import Scene, noise_targets, random_triangles_scene
 
 pytestmark = pytest.mark.gpu
@@ -53,3 +53,19 @@ def test_chain_rule_views_and_faces(oracle, n_views, n_faces):
     dev = lambda a: torch.as_tensor(np.asarray(a), dtype=torch.float32, device="cuda")  # noqa: E731
     rast.backward(dev(r["dC_used"]), dev(r["dD_used"]))
     assert_pose_grad(rast.pose_grad().cpu().numpy().astype(np.float64), r["dtau"], r["dtau_abs"])
+
+
+@pytest.mark.parametrize("size", [(1, 1), (7, 3), (8, 4), (17, 9), (33, 18)])
+@pytest.mark.parametrize("n_faces", [1, 31, 32, 33, 65, 129])
+def test_forward_pixel_lists(oracle, n_faces, size):
+    """The per-pixel face lists of the forward at ragged images and around 32 and 64 staged faces, with faces
+    far larger than the image (vertices close to the camera) among them."""
+    W, H = size
+    sc = random_triangles_scene(seed=n_faces + W, n_faces=n_faces, W=W, H=H, f=20.0, z_lo=0.2, z_hi=2.0, side_lo=0.05,
+                                side_hi=0.8, opa_lo=0.05, opa_hi=0.6, target_seed=None)
+    p, po = params_pair()
+    g = gpu_run(sc, p, backward=False, pair_capacity=4096)
+    r = oracle_run(oracle, sc, po, backward=False)
+    for k in ("color", "depth", "alpha", "T_final"):
+        assert_images(g[k], r[k], k)
+    assert np.array_equal(g["n_last"], r["n_last"])
