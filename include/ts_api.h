@@ -294,7 +294,7 @@ ts_status ts_l1_loss(const ts_plan* plan, void* ws, const float* color, const fl
  * dD = dloss/dD (overwritten; sign(0) = 0).  Pointers and packing as in ts_l1_loss; loss: device
  * float [n_views], overwritten.  lambda_ssim = 0 gives the ts_l1_loss value.  lambda_ssim outside
  * [0, 1] or a negative or non-finite lambda_dep returns TS_ERR_INVALID_ARG.  Deterministic: the
- * partial sums per 32 x 32 tile are reduced in a fixed order.  Like ts_l1_loss it needs no earlier
+ * partial sums per image strip are reduced in a fixed order.  Like ts_l1_loss it needs no earlier
  * call on the workspace. */
 ts_status ts_pho_loss(const ts_plan* plan, void* ws, const float* color, const float* depth,
                       const float* tgt_color, const float* tgt_depth, float lambda_ssim, float lambda_dep,

@@ -128,7 +128,7 @@ struct TsWs {
   float* grad;
   float* pose;
   float* loss;
-  float* pho;  // per (view, 32 x 32 tile): L1, SSIM and depth partial sums of the photometric loss
+  float* pho;  // per (view, channel, strip): L1, SSIM and depth partial sums of the photometric loss
   float* equi;  // per block of 256 faces: partial sums of the equilateral regulariser
   float4* aux;  // per (view, face): camera-space unit normal (TS_FLAG_NORMALS) and the face's sigma
                // (TS_FLAG_FACE_SIGMA) in .w; null without either flag

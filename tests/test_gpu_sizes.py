@@ -1,5 +1,6 @@
 """Kernels at the sizes where their splits change: tile lists around the sort's register, warp and CTA
-limits, the chain rule around its faces per warp, the forward's pixel lists (needs a GB300)."""
+limits, the chain rule around its faces per warp, the forward's pixel lists, the photometric loss's
+strips (needs a GB300)."""
 import numpy as np
 import pytest
 
@@ -69,3 +70,13 @@ def test_forward_pixel_lists(oracle, n_faces, size):
     for k in ("color", "depth", "alpha", "T_final"):
         assert_images(g[k], r[k], k)
     assert np.array_equal(g["n_last"], r["n_last"])
+
+
+def test_pho_loss_strip_edges(oracle):
+    """The photometric loss around its strips: widths and heights on both sides of 64 columns and of 22 rows
+    (the strip height of a small batch), and images smaller than the window."""
+    from test_gpu_pho import _cams, _check, _gpu, _scene_arrays
+    from ts_synth.scenes import loss_images
+    cams = _cams([(63, 21), (64, 22), (65, 23), (128, 44), (129, 45), (5, 3), (3, 30), (70, 1)])
+    C, D, tC, tD = loss_images(21, cams)
+    _check(cams, _gpu(cams, C, D, tC, tD, 0.2, 0.05), oracle.pho_loss(_scene_arrays(cams), C, D, tC, tD, 0.2, 0.05))
