@@ -8,7 +8,7 @@
 //   * o_F = (o_i + o_j + o_k) / 3 (Sec. 3.1): each vertex opacity gets a third;
 //   * with TS_FLAG_NORMALS, the face normal of the normal map (Eq. 12) through the cross product
 //     of the camera-space edge vectors; with TS_FLAG_FACE_SIGMA, dL/dsigma_F (a sum the raster
-//     backward already formed, word 24) is summed over views;
+//     backward already formed) is summed over views;
 //   * the pinhole (Eq. 1) to camera space, R^T to world space, and the left-perturbation pose
 //     Jacobian [I, -[v_C]x] (Eq. 7): dL/dtau += [g_C ; v_C x g_C].
 //
@@ -61,38 +61,31 @@ __device__ __forceinline__ long long face_vertex(const TsDevHeader* h, long long
   return (j >= 0 && j < h->n_vertices) ? j : 0;
 }
 
-// A slot's sums in registers: words 0..23, and with the side array 24, 30 and 31.
+// A slot's sums in registers: G as numbered by G_E .. G_O, dL/dn_F and dL/dsigma_F.
 struct SlotSums {
-  float G[24], w24, w30, w31;
+  float G[22], n[3], sig;
 };
-// Floats between the lanes' slot copies in shared memory: 7 or 9 16-byte groups, so that the lanes of a
-// quarter warp read distinct banks.
-__host__ __device__ constexpr int slot_stride(bool aux) { return aux ? 36 : 28; }
+// A lane's slot copy in shared memory: its eight 16-byte groups in an order of the lane's own, so that the
+// lanes of a quarter warp read distinct banks.
+__device__ __forceinline__ int group_place(int i) { return (i ^ (threadIdx.x & 7)) * 4; }
 
 // This lane copies a slot into its place `dst`; wait_slot waits for the lane's own copies only.
 __device__ __forceinline__ void fetch_slot(const PBArgs& a, float* dst, long long slot) {
   const float* src = a.grad + slot * TS_GRAD_WORDS;
 #pragma unroll
-  for (int i = 0; i < 6; ++i) ts_cp_async16(dst + 4 * i, src + 4 * i);
-  if (a.aux) {
-    ts_cp_async16(dst + 24, src + 24);
-    ts_cp_async16(dst + 28, src + 28);
-  }
+  for (int i = 0; i < 8; ++i) ts_cp_async16(dst + group_place(i), src + 4 * i);
   ts_cp_async_commit();
 }
-__device__ __forceinline__ void wait_slot(const PBArgs& a, const float* src, SlotSums& s) {
+__device__ __forceinline__ void wait_slot(const float* src, SlotSums& s) {
   ts_cp_async_wait_all();
 #pragma unroll
-  for (int i = 0; i < 6; ++i) {
-    const float4 q = reinterpret_cast<const float4*>(src)[i];
-    s.G[4 * i] = q.x; s.G[4 * i + 1] = q.y; s.G[4 * i + 2] = q.z; s.G[4 * i + 3] = q.w;
+  for (int i = 0; i < 7; ++i) {
+    const float4 q = *reinterpret_cast<const float4*>(src + group_place(i));
+    s.G[3 * i] = q.x; s.G[3 * i + 1] = q.y; s.G[3 * i + 2] = q.z;
+    if (i < 3) s.n[i] = q.w;
+    if (i == 3) s.sig = q.w;
   }
-  s.w24 = s.w30 = s.w31 = 0.f;
-  if (a.aux) {
-    s.w24 = src[24];
-    s.w30 = src[30];
-    s.w31 = src[31];
-  }
+  s.G[G_O] = src[group_place(7)];
 }
 
 // 4-byte asynchronous copy of one value.
@@ -139,7 +132,7 @@ struct SlotTerms {
 // (vertex k, coordinate c at 3k + c) and then its vertex colours, vp its view (stage_view).
 __device__ __forceinline__ void chain_terms(const PBArgs& a, int v, long long m, const SlotSums& sl, const float* X,
                                             const float* vp, SlotTerms& t) {
-  const float(&G)[24] = sl.G;
+  const float(&G)[22] = sl.G;
   TsView vw;
   vw.fx = vp[0];
   vw.fy = vp[1];
@@ -222,12 +215,12 @@ __device__ __forceinline__ void chain_terms(const PBArgs& a, int v, long long m,
     gu[j1] += cx; gv[j1] += cy;
     gu[j] -= cx; gv[j] -= cy;
   }
-  // normal map (Eq. 12): dL/dn_F from words 23, 30, 31 through n = s u / |u|, u = e1 x e2 with
+  // normal map (Eq. 12): dL/dn_F through n = s u / |u|, u = e1 x e2 with
   // e1 = v1 - v0, e2 = v2 - v0 in camera space and s = +-1 the camera-facing turn of the forward:
   // dL/du = s (g - n (n . g)) / |u|, dL/de1 = e2 x dL/du, dL/de2 = dL/du x e1
   float ng[3][3] = {{0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}};
   if (a.normals) {
-    const float gn[3] = {G[23], sl.w30, sl.w31};
+    const float gn[3] = {sl.n[0], sl.n[1], sl.n[2]};
     if (gn[0] != 0.f || gn[1] != 0.f || gn[2] != 0.f) {
       const float4 nn = a.aux[(long long)v * a.M + m];
       const float e1[3] = {xc[1] - xc[0], yc[1] - yc[0], zc[1] - zc[0]};
@@ -272,22 +265,22 @@ __device__ __forceinline__ void chain_terms(const PBArgs& a, int v, long long m,
 #pragma unroll
   for (int i = 0; i < 9; ++i) t.gc[i] = G[G_C + i];
   t.go = G[G_O];
-  t.gsig = sl.w24;
+  t.gsig = sl.sig;
 }
 
 constexpr int PB_WARPS = 4;
 constexpr int PB_T = 32 * PB_WARPS;
 constexpr int PB_RS = 21;   // floats per entry row (positions 9, colours 9, opacity, sigma; odd: no bank conflicts)
 constexpr int PB_FS = 19;   // floats per staged face (positions 9, colours 9)
-constexpr int PB_PS = 7;    // floats per view's pose sums (6 used)
+constexpr int PB_PS = 6;    // floats per view's pose sums
 
 // Views whose visibility the lanes of one face look up at a time (64 bits each).
 __host__ __device__ constexpr int pbwd_view_chunk(int faces) { return 64 * (32 / faces); }
 // Shared floats of one warp (a multiple of 4): slot copies, entry rows, staged faces, per-face sums,
 // per-view pose sums, entry list.
-__host__ __device__ constexpr int pbwd_warp_floats(int V, int faces, bool aux) {
+__host__ __device__ constexpr int pbwd_warp_floats(int V, int faces) {
   const int chunk = V < pbwd_view_chunk(faces) ? V : pbwd_view_chunk(faces);
-  return (32 * slot_stride(aux) + 32 * PB_RS + faces * (PB_FS + PB_RS) + V * PB_PS + (faces * chunk + 1) / 2 + 3) & ~3;
+  return (32 * TS_GRAD_WORDS + 32 * PB_RS + faces * (PB_FS + PB_RS) + V * PB_PS + (faces * chunk + 1) / 2 + 3) & ~3;
 }
 
 // With map gradients: FPW faces per warp iteration, 32 / FPW lanes looking up each face's views.
@@ -297,16 +290,15 @@ __global__ void __launch_bounds__(PB_T, 4) k_pbwd_map(PBArgs a) {
   extern __shared__ __align__(16) float pv[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const TsDevHeader* h = a.hdr;
-  const bool aux = a.aux != nullptr;
-  const int per_warp = pbwd_warp_floats(a.V, FPW, aux);
+  const int per_warp = pbwd_warp_floats(a.V, FPW);
   float* views = pv + (size_t)PB_WARPS * per_warp;  // [V][VP]
   float* slots = pv + (size_t)warp * per_warp;
-  float* rows = slots + 32 * slot_stride(aux);
+  float* rows = slots + 32 * TS_GRAD_WORDS;
   float* fdat = rows + 32 * PB_RS;
   float* fsum = fdat + FPW * PB_FS;
   float* my = fsum + FPW * PB_RS;
   uint16_t* list = reinterpret_cast<uint16_t*>(my + a.V * PB_PS);  // face * 256 + view
-  float* slot_here = slots + lane * slot_stride(aux);
+  float* slot_here = slots + lane * TS_GRAD_WORDS;
   for (int v = threadIdx.x; v < a.V; v += PB_T) stage_view(a, views + v * VP, v);
   for (int i = lane; i < a.V * PB_PS; i += 32) my[i] = 0.f;
   __syncthreads();
@@ -362,7 +354,7 @@ __global__ void __launch_bounds__(PB_T, 4) k_pbwd_map(PBArgs a) {
         const int code = act ? next : 0;
         const int fe = code >> 8, v = code & 255;
         SlotSums sl;
-        if (act) wait_slot(a, slot_here, sl);
+        if (act) wait_slot(slot_here, sl);
         next = b0 + 32 + lane < total ? list[b0 + 32 + lane] : -1;
         if (next >= 0) fetch_slot(a, slot_here, (m0 + (next >> 8)) * a.V + (next & 255));
         float tau[6];
@@ -477,8 +469,8 @@ __global__ void __launch_bounds__(PB_T, 4) k_pbwd_pose(PBArgs a) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, v = blockIdx.y;
   const TsDevHeader* h = a.hdr;
   const uint32_t* cnt = a.count + (long long)v * a.M;
-  float* slot_here = pv + threadIdx.x * slot_stride(a.aux != nullptr);
-  float* face_here = pv + PB_T * slot_stride(a.aux != nullptr) + threadIdx.x * PB_FS;
+  float* slot_here = pv + threadIdx.x * TS_GRAD_WORDS;
+  float* face_here = pv + PB_T * TS_GRAD_WORDS + threadIdx.x * PB_FS;
   if (threadIdx.x == 0) stage_view(a, view, v);
   __syncthreads();
   float tau[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
@@ -489,7 +481,7 @@ __global__ void __launch_bounds__(PB_T, 4) k_pbwd_pose(PBArgs a) {
     SlotSums sl;
     float X[18];
     if (m >= 0) {
-      wait_slot(a, slot_here, sl);
+      wait_slot(slot_here, sl);
 #pragma unroll
       for (int i = 0; i < 18; ++i) X[i] = face_here[i];
     }
@@ -569,8 +561,9 @@ __global__ void __launch_bounds__(256) k_pose_reduce(const float* __restrict__ p
 
 }  // namespace
 
-// The faces per warp and block fix the partial sums of the pose gradient and so its summation order: they
-// depend on the map's size alone, so that a view's dtau is the same alone and among others, and on every GPU.
+// The faces per warp and block fix the partial sums of the pose gradient and so its summation order: without
+// map gradients they depend on the map's size alone, so that a tracked view's dtau is the same alone and
+// among others, and on every GPU.
 constexpr long long MAP_BLOCKS = 608;    // 4 resident blocks on 152 SMs
 constexpr long long POSE_BLOCKS = 2432;  // most blocks per view of the form without map gradients
 int ts_pose_blocks(long long M) {        // the most either form uses
@@ -581,7 +574,7 @@ namespace {
 template <int FPW>
 cudaError_t launch_pbwd_map(const PBArgs& a, cudaStream_t s) {
   const int smem =
-      (PB_WARPS * pbwd_warp_floats(a.V, FPW, a.aux != nullptr) + a.V * VP) * (int)sizeof(float);  // <= 146 KB
+      (PB_WARPS * pbwd_warp_floats(a.V, FPW) + a.V * VP) * (int)sizeof(float);  // <= 146 KB
   const cudaError_t e = ts_smem_limit((const void*)k_pbwd_map<FPW>, smem);
   if (e != cudaSuccess) return e;
   const long long want = (a.M + PB_WARPS * FPW - 1) / (PB_WARPS * FPW);
@@ -621,13 +614,16 @@ cudaError_t ts_launch_project_bwd(const TsPlanImpl* p, const TsWs& w, const ts_m
     const long long least = (p->M + PB_WARPS * POSE_BLOCKS - 1) / (PB_WARPS * POSE_BLOCKS);
     a.unit = p->M >= (1 << 16) ? (int)std::max<long long>(512, (least + 31) / 32 * 32) : (p->M >= (1 << 14) ? 128 : 32);
     const long long nb = (p->M + PB_WARPS * a.unit - 1) / (PB_WARPS * a.unit);
-    const int smem = PB_T * (slot_stride(a.aux != nullptr) + PB_FS) * (int)sizeof(float);  // <= 28 KB
+    const int smem = PB_T * (TS_GRAD_WORDS + PB_FS) * (int)sizeof(float);  // 26 KB
     k_pbwd_pose<<<dim3((unsigned)nb, (unsigned)p->V), PB_T, smem, s>>>(a);
     return cudaGetLastError();
   }
-  // 32 faces a warp once every warp of the grid has some, fewer of smaller maps
-  if (p->M > MAP_BLOCKS * PB_WARPS * 16) return launch_pbwd_map<32>(a, s);
-  if (p->M > MAP_BLOCKS * PB_WARPS * 8) return launch_pbwd_map<16>(a, s);
+  // 32 faces a warp once every warp of the grid has some, fewer of smaller maps and where more views would
+  // leave room for three blocks on an SM instead of four (and the grid a second wave)
+  const int most = p->V <= 20 ? 32 : (p->V <= 48 ? 16 : 8);
+  const int faces = std::min(most, p->M > MAP_BLOCKS * PB_WARPS * 16 ? 32 : (p->M > MAP_BLOCKS * PB_WARPS * 8 ? 16 : 8));
+  if (faces == 32) return launch_pbwd_map<32>(a, s);
+  if (faces == 16) return launch_pbwd_map<16>(a, s);
   return launch_pbwd_map<8>(a, s);
 }
 

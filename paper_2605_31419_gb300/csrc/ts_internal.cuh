@@ -13,7 +13,7 @@
 
 #define TS_PLAN_MAGIC 0x54535031u  // "TSP1"
 #define TS_REC_WORDS 32            // 128-byte record, a multiple of 16 B for cp.async.bulk
-#define TS_GRAD_WORDS 32           // per-(view, face) gradient slot: 24 accumulators, 32 with the side array
+#define TS_GRAD_WORDS 32           // per-(view, face) gradient slot
 #define TS_SCAN_ITEMS 4096         // items per scan block (1024 threads x 4)
 #define TS_BIN_FACES 8192          // faces per block of the shared-memory tile counts
 #define TS_BIN_MAX_TILES 40960     // the most tiles of a view those counts hold (160 KB)
@@ -42,10 +42,12 @@ enum {
   R_BOXX = 29, R_BOXY = 30, R_SLOT = 31
 };
 
-// Gradient word indices: G_E[i][k] = sum_p dL/dE_i * lambda_k (edge i nearest), G_c[ch][k] =
-// sum_p dL/dc_ch * lambda_k, G_z[k] = sum_p dL/dz * lambda_k, G_o = dL/do_F, count = pixels.
-// The raster backward accumulates words 0..23; the chain-rule pass reads them.
-enum { G_E = 0, G_C = 9, G_Z = 18, G_O = 21, G_CNT = 22 };
+// A gradient slot holds eight groups of four words, which the raster backward adds into and the chain-rule
+// pass reads.  Group i < 3: sum_p dL/dE_i lambda_k (edge i nearest), k = 0..2; groups 3..5: sum_p dL/dc_ch
+// lambda_k of the colour channels; group 6: sum_p dL/dz lambda_k; group 7: dL/do_F.  With the side array the
+// fourth words of groups 0..2 hold dL/dn_F and that of group 3 dL/dsigma_F.  In registers the first 22 are
+// numbered without the fourth words:
+enum { G_E = 0, G_C = 9, G_Z = 18, G_O = 21 };
 
 struct TsView {
   float fx, fy, cx, cy;
