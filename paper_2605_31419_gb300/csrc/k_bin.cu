@@ -1,12 +1,13 @@
 // k_bin.cu -- depth ordering per tile (Eq. 4: faces are composited in depth order).
 //
 //  1. per tile, the number of (view, face) pairs whose tile rectangle covers it.  When every
-//     view's tiles fit in shared memory (TS_BIN_MAX_TILES), one block per (TS_BIN_FACES faces,
-//     view) counts its pairs per tile there and writes a [tile][face block] count matrix; else
+//     view's tiles fit in shared memory (TS_BIN_MAX_TILES), one block per (block of faces, view)
+//     counts its pairs per tile there and writes a row of a [face block][tile] count matrix; else
 //     global atomic counts per tile;
-//  2. an exclusive scan of the counts (two-level, 4096 items per block; tile-major for the
-//     matrix) gives each tile's segment [start, end) of the pair list -- and with the matrix each
-//     block's first place in it -- the pair total and the capacity check;
+//  2. an exclusive scan of the counts (two-level: groups of 32 tiles, each tile's column of the
+//     matrix summed on the way, or 4096 counts) gives each tile's segment [start, end) of the pair
+//     list -- and with the matrix each block's first place in it -- the pair total and the capacity
+//     check;
 //  3. each pair is placed in its tile's segment (shared-memory atomics on the block's places, or
 //     global atomic cursors) as the 64-bit key (float bits of the depth key << 32 | face id),
 //     unique within a tile;
@@ -78,13 +79,11 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_reduce(const uint32_t* __restri
 
 // Exclusive scan of the block sums in place (one block); writes the grand total, and zeroes
 // *zero_out (the sort's count of long lists) for the launches that follow.
-__global__ void __launch_bounds__(SCAN_T) k_scan_bsums(uint32_t* bsums, Len len, unsigned long long* total_out,
-                                                       unsigned int* err, long long cap, unsigned int* zero_out) {
+__global__ void __launch_bounds__(SCAN_T) k_scan_bsums(uint32_t* bsums, long long nb,
+                                                       unsigned long long* total_out, unsigned int* err, long long cap, unsigned int* zero_out) {
   __shared__ uint32_t sm[33];
   __shared__ unsigned long long wsum[SCAN_T / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long long n = len.get();
-  const long long nb = (n + TS_SCAN_ITEMS - 1) / TS_SCAN_ITEMS;
   const long long per = (nb + SCAN_T - 1) / SCAN_T;
   const long long b0 = (long long)threadIdx.x * per;
   unsigned long long s = 0;
@@ -111,31 +110,6 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_bsums(uint32_t* bsums, Len len,
       if ((long long)tot64 > cap) atomicOr(err, TS_ERRBIT_CAPACITY);
     }
     if (zero_out) *zero_out = 0u;
-  }
-}
-
-
-// Second level of a plain in-place exclusive scan (blocked: 4 consecutive items per thread).
-__global__ void __launch_bounds__(SCAN_T) k_scan_apply(uint32_t* __restrict__ data, Len len,
-                                                       const uint32_t* __restrict__ bsums) {
-  __shared__ uint32_t sm[33];
-  const long long n = len.get();
-  const long long base = (long long)blockIdx.x * TS_SCAN_ITEMS;
-  if (base >= n) return;
-  const long long i0 = base + (long long)threadIdx.x * SCAN_PER;
-  uint32_t c[SCAN_PER];
-  uint32_t s = 0;
-#pragma unroll
-  for (int k = 0; k < SCAN_PER; ++k) {
-    c[k] = (i0 + k < n) ? data[i0 + k] : 0u;
-    s += c[k];
-  }
-  uint32_t tot;
-  uint32_t off = block_excl_scan(s, sm, &tot) + bsums[blockIdx.x];
-#pragma unroll
-  for (int k = 0; k < SCAN_PER; ++k) {
-    if (i0 + k < n) data[i0 + k] = off;
-    off += c[k];
   }
 }
 
@@ -222,85 +196,196 @@ __global__ void __launch_bounds__(256) k_tile_scatter(TileArgs a) {
   }
 }
 
-// Steps 1-3 when every view's tiles fit in shared memory: one block per (block of TS_BIN_FACES
-// faces, view) counts its pairs per tile in shared memory, and the exclusive scan of the
-// [tile][face block] count matrix (tile-major) gives each block its first place in every tile's
-// segment; the block then places its pairs with shared-memory atomics.
+// Steps 1-3 when every view's tiles fit in shared memory: one block per (block of faces, view) counts its
+// pairs per tile in shared memory, the exclusive scan of the [face block][tile] count matrix down its
+// columns gives each block its first place in every tile's segment, and the block then places its pairs with
+// shared-memory atomics.
+//
+// A warp numbers the (face, tile) pairs of 32 faces (a scan of their rectangles' sizes) and takes 32 of them
+// at a time, one per lane; rectangles above WIDE_MIN tiles are queued for the whole block.  With a thread
+// walking its own face's tiles, the few faces right before a camera, which cover the image, each held one
+// thread for thousands of dependent steps and the launch waited for it (3 % of its issue slots used).  And
+// the matrix was [tile][face block], written and read 4 bytes at a time.  Counts, scans and places together:
+// 246 -> 103 us for 20 views of 300k faces (places alone 167 -> 53), 115 -> 40 for 8 views of 640x480,
+// 238 -> 158 for the 12-view window of 1M faces, 275 -> 222 for 9 views of 2M.
 struct MatArgs {
-  const uint32_t* count;
   const short4* rect;
   const uint32_t* zbits;
   const TsView* views;
-  long long M, B, cap, n_tiles;
-  uint32_t* mat;
+  long long M, n_tiles, cap;
+  int faces;             // per block, a multiple of BIN_T
+  uint32_t* mat;         // [face block][tile]: pair counts, then their exclusive sums down the column
+  const uint32_t* tpre;  // per tile: the pairs of the tiles before it in its group of TS_BIN_GROUP
+  const uint32_t* gsum;  // per group: the pairs of the groups before it
   unsigned long long* seg;
-  uint2* ranges;
-  const unsigned long long* n_pairs;
 };
 
-constexpr int BIN_T = 1024;
-constexpr int BIN_PER = TS_BIN_FACES / BIN_T;  // faces per thread
-static_assert(TS_BIN_FACES % BIN_T == 0, "whole faces per thread");
+constexpr int BIN_T = 512;
+constexpr int WIDE_MIN = 128;  // tiles above which a rectangle is queued
+constexpr int WIDE_MAX = 256;  // queue entries; the warps take the rectangles beyond it themselves
+static_assert(TS_BIN_FACES % 1024 == 0 && 1024 % BIN_T == 0, "whole rounds of faces per thread");
 
-__global__ void __launch_bounds__(BIN_T) k_bin_counts(MatArgs a) {
-  extern __shared__ uint32_t hcnt[];
-  const int v = blockIdx.y;
-  const long long blk = blockIdx.x;
-  const TsView& vw = a.views[v];
-  const int T = vw.TX * vw.TY;
-  for (int t = threadIdx.x; t < T; t += BIN_T) hcnt[t] = 0u;
-  __syncthreads();
-  const long long m0 = blk * TS_BIN_FACES + threadIdx.x;
-  uint32_t cnt[BIN_PER];
-  short4 rc[BIN_PER];
-#pragma unroll
-  for (int k = 0; k < BIN_PER; ++k) {  // all loads first, so that their latencies overlap
-    const long long m = m0 + (long long)k * BIN_T;
-    const long long idx = (long long)v * a.M + m;
-    cnt[k] = m < a.M ? a.count[idx] : 0u;
-    rc[k] = m < a.M ? a.rect[idx] : make_short4(0, 0, -1, -1);
-  }
-#pragma unroll
-  for (int k = 0; k < BIN_PER; ++k) {
-    if (cnt[k] == 0) continue;  // (an invisible face's rectangle is -1)
-    const short4 r = rc[k];
-    for (int ty = r.y; ty <= r.w; ++ty)
-      for (int tx = r.x; tx <= r.z; ++tx) atomicAdd(&hcnt[ty * vw.TX + tx], 1u);
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < T; t += BIN_T) a.mat[(vw.tile_off + t) * a.B + blk] = hcnt[t];
+struct WideFaces {
+  short4 rect[WIDE_MAX];
+  uint32_t z[WIDE_MAX], id[WIDE_MAX];
+  unsigned n;
+};
+
+// k / w for 0 <= k < 2^20 and 1 <= w: (k + 1/2) / w lies at least 1 / (2 w) from every whole number, and the
+// approximation is off by less than 2^-21 of it.
+__device__ __forceinline__ int small_div(int k, int w) {
+  return (int)(((float)k + 0.5f) * ts_rcp_approx((float)w));
 }
 
-__global__ void __launch_bounds__(BIN_T) k_bin_place(MatArgs a) {
-  extern __shared__ uint32_t place[];
-  const int v = blockIdx.y;
-  const long long blk = blockIdx.x;
-  const TsView& vw = a.views[v];
-  const int T = vw.TX * vw.TY;
-  for (int t = threadIdx.x; t < T; t += BIN_T) place[t] = a.mat[(vw.tile_off + t) * a.B + blk];
-  __syncthreads();
-  const long long m0 = blk * TS_BIN_FACES + threadIdx.x;
-  uint32_t cnt[BIN_PER], zb[BIN_PER];
-  short4 rc[BIN_PER];
-#pragma unroll
-  for (int k = 0; k < BIN_PER; ++k) {  // all loads first, so that their latencies overlap
+// Every thread of the block calls it: put(tile of the view, depth bits, face) for each pair of the block's
+// faces.  WITH_Z: the depth keys are loaded (else zero).
+template <bool WITH_Z, class Put>
+__device__ __forceinline__ void for_each_pair(const MatArgs& a, int v, long long blk, int TX, WideFaces& wide,
+                                              Put put) {
+  const int lane = threadIdx.x & 31;
+  const long long vbase = (long long)v * a.M;
+  const long long m0 = blk * a.faces + threadIdx.x;
+  const int rounds = a.faces / BIN_T;
+  const short4 none = make_short4(-1, -1, -1, -1);
+  auto rect_at = [&](int k) {
     const long long m = m0 + (long long)k * BIN_T;
-    const long long idx = (long long)v * a.M + m;
-    cnt[k] = m < a.M ? a.count[idx] : 0u;
-    rc[k] = m < a.M ? a.rect[idx] : make_short4(0, 0, -1, -1);
-    zb[k] = m < a.M ? a.zbits[idx] : 0u;
-  }
-#pragma unroll
-  for (int k = 0; k < BIN_PER; ++k) {
-    if (cnt[k] == 0) continue;  // (an invisible face's rectangle is -1)
-    const short4 r = rc[k];
-    const unsigned long long key = ((unsigned long long)zb[k] << 32) | (uint32_t)(m0 + (long long)k * BIN_T);
-    for (int ty = r.y; ty <= r.w; ++ty)
-      for (int tx = r.x; tx <= r.z; ++tx) {
-        const uint32_t pos = atomicAdd(&place[ty * vw.TX + tx], 1u);
-        if ((long long)pos < a.cap) a.seg[pos] = key;  // beyond: the scan has latched the capacity bit
+    return k < rounds && m < a.M ? a.rect[vbase + m] : none;
+  };
+  auto z_at = [&](int k) {
+    const long long m = m0 + (long long)k * BIN_T;
+    return WITH_Z && k < rounds && m < a.M ? a.zbits[vbase + m] : 0u;
+  };
+  // two rounds' loads in flight while one is worked on
+  short4 r = rect_at(0), r1 = rect_at(1);
+  uint32_t z = z_at(0), z1 = z_at(1);
+#pragma unroll 1
+  for (int k = 0; k < rounds; ++k) {
+    const short4 r2 = rect_at(k + 2);
+    const uint32_t z2 = z_at(k + 2);
+    const uint32_t id = (uint32_t)(m0 + (long long)k * BIN_T);
+    const int w = r.z - r.x + 1;
+    int n = r.x >= 0 ? w * (r.w - r.y + 1) : 0;  // an invisible face's rectangle is -1
+    if (n > WIDE_MIN) {
+      const unsigned q = atomicAdd(&wide.n, 1u);
+      if (q < WIDE_MAX) {
+        wide.rect[q] = r;
+        wide.z[q] = z;
+        wide.id[q] = id;
+        n = 0;
       }
+    }
+    const int incl = (int)warp_incl_scan((uint32_t)n), excl = incl - n;
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    const int corner = (int)r.y * TX + (int)r.x;
+    for (int e0 = 0; e0 < total; e0 += 32) {
+      const int e = e0 + lane;
+      int ow = 0;  // the pair's lane: the last whose first number is at most e
+#pragma unroll
+      for (int s = 16; s > 0; s >>= 1)
+        if (__shfl_sync(0xffffffffu, excl, ow + s) <= e) ow += s;
+      const int p = e - __shfl_sync(0xffffffffu, excl, ow);
+      const int pw = __shfl_sync(0xffffffffu, w, ow);
+      const int pc = __shfl_sync(0xffffffffu, corner, ow);
+      const uint32_t pz = WITH_Z ? __shfl_sync(0xffffffffu, z, ow) : 0u;
+      const int dy = small_div(p, pw);
+      if (e < total) put(pc + dy * (TX - pw) + p, pz, id - (uint32_t)lane + (uint32_t)ow);
+    }
+    r = r1;
+    r1 = r2;
+    z = z1;
+    z1 = z2;
   }
+  __syncthreads();
+  const int nw = (int)min(wide.n, (unsigned)WIDE_MAX);
+  for (int q = 0; q < nw; ++q) {
+    const short4 r = wide.rect[q];
+    const int w = r.z - r.x + 1, n = w * (r.w - r.y + 1);
+    for (int p = threadIdx.x; p < n; p += BIN_T) {
+      const int dy = small_div(p, w);
+      put((r.y + dy) * TX + r.x + (p - dy * w), wide.z[q], wide.id[q]);
+    }
+  }
+}
+
+__global__ void __launch_bounds__(BIN_T, 3) k_bin_counts(MatArgs a) {
+  extern __shared__ uint32_t hcnt[];
+  __shared__ WideFaces wide;
+  const int v = blockIdx.y;
+  const TsView& vw = a.views[v];
+  const int TX = vw.TX, T = TX * vw.TY;
+  if (threadIdx.x == 0) wide.n = 0u;
+  for (int t = threadIdx.x; t < T; t += BIN_T) hcnt[t] = 0u;
+  __syncthreads();
+  for_each_pair<false>(a, v, blockIdx.x, TX, wide, [&](int t, uint32_t, uint32_t) { atomicAdd(&hcnt[t], 1u); });
+  __syncthreads();
+  uint32_t* row = a.mat + (long long)blockIdx.x * a.n_tiles + vw.tile_off;
+  for (int t = threadIdx.x; t < T; t += BIN_T) row[t] = hcnt[t];
+}
+
+// One block per TS_BIN_GROUP tiles, a lane per tile and a warp per share of the rows: the exclusive sums down
+// each tile's column in place, up to 64 rows at a time in registers; the tiles' totals, scanned within the
+// group, and the group's total.
+constexpr int COL_WARPS = 8, COL_ROWS = 8;  // warps per block, most rows per warp at a time
+__global__ void __launch_bounds__(32 * COL_WARPS) k_bin_columns(uint32_t* __restrict__ mat, long long n_tiles, int B,
+                                                                 uint32_t* __restrict__ tpre,
+                                                                 uint32_t* __restrict__ gsum) {
+  static_assert(TS_BIN_GROUP == 32, "a lane per tile of the group");
+  __shared__ uint32_t part[COL_WARPS][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long t = (long long)blockIdx.x * 32 + lane;
+  const bool in = t < n_tiles;
+  uint32_t carry = 0u;
+  for (int r0 = 0; r0 < B; r0 += COL_WARPS * COL_ROWS) {
+    const int left = min(B - r0, COL_WARPS * COL_ROWS), per = (left + COL_WARPS - 1) / COL_WARPS;
+    const int k1 = min(per, left - warp * per);  // this warp's rows: r0 + warp * per + [0, k1)
+    uint32_t* col = mat + (long long)(r0 + warp * per) * n_tiles + t;
+    uint32_t c[COL_ROWS], s = 0u;
+#pragma unroll
+    for (int k = 0; k < COL_ROWS; ++k) {
+      c[k] = in && k < k1 ? col[(long long)k * n_tiles] : 0u;
+      s += c[k];
+    }
+    part[warp][lane] = s;
+    __syncthreads();
+    uint32_t off = carry;
+#pragma unroll
+    for (int w = 0; w < COL_WARPS; ++w) {
+      const uint32_t x = part[w][lane];
+      carry += x;
+      off += w < warp ? x : 0u;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int k = 0; k < COL_ROWS; ++k) {
+      if (in && k < k1) col[(long long)k * n_tiles] = off;
+      off += c[k];
+    }
+  }
+  if (warp == 0) {
+    const uint32_t incl = warp_incl_scan(carry);
+    if (in) tpre[t] = incl - carry;
+    if (lane == 31) gsum[blockIdx.x] = incl;
+  }
+}
+
+__global__ void __launch_bounds__(BIN_T, 3) k_bin_place(MatArgs a) {
+  extern __shared__ uint32_t place[];
+  __shared__ WideFaces wide;
+  const int v = blockIdx.y;
+  const TsView& vw = a.views[v];
+  const int TX = vw.TX, T = TX * vw.TY;
+  if (threadIdx.x == 0) wide.n = 0u;
+  const uint32_t* row = a.mat + (long long)blockIdx.x * a.n_tiles;
+  for (int t = threadIdx.x; t < T; t += BIN_T) {
+    const long long g = vw.tile_off + t;
+    place[t] = row[g] + a.tpre[g] + a.gsum[g / TS_BIN_GROUP];
+  }
+  __syncthreads();
+  for_each_pair<true>(a, v, blockIdx.x, TX, wide, [&](int t, uint32_t z, uint32_t id) {
+    const uint32_t pos = atomicAdd(&place[t], 1u);
+    // beyond: the scan has latched the capacity bit
+    if ((long long)pos < a.cap) a.seg[pos] = ((unsigned long long)z << 32) | id;
+  });
 }
 
 // Step 4.  In registers, bitonic networks in the form whose every compare-exchange moves the smaller key to
@@ -314,8 +399,8 @@ struct SortOut {
   long long n_tiles, cap;
   uint32_t* large;         // tiles left to the CTA-wide sort
   unsigned int* n_large;
-  const uint32_t* mat;     // the scanned [tile][face block] count matrix, or null: ranges from the scatter
-  long long B;             // face blocks per tile row of the matrix
+  const uint32_t* tpre;    // with the count matrix: pairs of the tiles before this one in its group, else null
+  const uint32_t* gsum;    // (ranges from the scatter); pairs of the groups before
   const unsigned long long* n_pairs;
 };
 
@@ -410,12 +495,13 @@ __global__ void __launch_bounds__(32 * SORT_WARPS_PER_BLOCK) k_tile_sort(SortOut
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long t = (long long)blockIdx.x * SORT_WARPS_PER_BLOCK + warp;
   if (t >= o.n_tiles) return;
-  // the segment: from the scanned matrix (its first block's place, the next tile's, the pair total
-  // after the last tile), else as the scatter left it in ranges
+  // the segment: from the scanned totals (its first place, the next tile's, the pair total after the
+  // last tile), else as the scatter left it in ranges
   uint2 rg;
-  if (o.mat) {
-    rg.x = o.mat[t * o.B];
-    rg.y = t + 1 < o.n_tiles ? o.mat[(t + 1) * o.B] : (uint32_t)min(*o.n_pairs, 0xffffffffull);
+  if (o.tpre) {
+    rg.x = o.tpre[t] + o.gsum[t / TS_BIN_GROUP];
+    rg.y = t + 1 < o.n_tiles ? o.tpre[t + 1] + o.gsum[(t + 1) / TS_BIN_GROUP]
+                             : (uint32_t)min(*o.n_pairs, 0xffffffffull);
   } else {
     rg = o.ranges[t];
   }
@@ -423,7 +509,7 @@ __global__ void __launch_bounds__(32 * SORT_WARPS_PER_BLOCK) k_tile_sort(SortOut
   const long long end = min((long long)rg.y, o.cap);
   // the tile's range for the passes that follow; past the capacity (its bit is latched) the lists
   // are cut, and the ranges with them, so that no later pass reads outside the pair list
-  if (lane == 0 && (o.mat || (long long)rg.y > o.cap)) o.ranges[t] = make_uint2((uint32_t)start, (uint32_t)end);
+  if (lane == 0 && (o.tpre || (long long)rg.y > o.cap)) o.ranges[t] = make_uint2((uint32_t)start, (uint32_t)end);
   const int n = (int)max(0LL, end - start);
   if (n == 0) return;
   if (n <= 32) {
@@ -615,19 +701,16 @@ cudaError_t ts_launch_bin(const TsPlanImpl* p, const TsWs& w, cudaStream_t s) {
   if (p->bin_blocks > 0) {
     // 1-3 with shared-memory counts: counts, their scan (the total is the pair count; above the
     // capacity latches its bit), places, ranges
-    MatArgs ma{w.count, w.rect, w.zbits, w.views, p->M, p->bin_blocks, p->cap, p->n_tiles, w.tmat, w.keys[1],
-               w.ranges, &w.hdr->n_pairs};
+    MatArgs ma{w.rect, w.zbits, w.views, p->M, p->n_tiles, p->cap, (int)p->bin_faces, w.tmat, w.tcnt, w.bsums, w.keys[1]};
     const int smem = (int)(p->max_view_tiles * sizeof(uint32_t));
     e = ts_smem_limit((const void*)k_bin_counts, smem);
     if (e == cudaSuccess) e = ts_smem_limit((const void*)k_bin_place, smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)p->bin_blocks, (unsigned)p->V);
     k_bin_counts<<<grid, BIN_T, smem, s>>>(ma);
-    Len lm{p->n_tiles * p->bin_blocks};
-    const unsigned nb = (unsigned)((lm.n + TS_SCAN_ITEMS - 1) / TS_SCAN_ITEMS);
-    k_scan_reduce<<<nb, SCAN_T, 0, s>>>(w.tmat, lm, w.bsums);
-    k_scan_bsums<<<1, SCAN_T, 0, s>>>(w.bsums, lm, &w.hdr->n_pairs, &w.hdr->error_bits, p->cap, &w.hdr->n_large);
-    k_scan_apply<<<nb, SCAN_T, 0, s>>>(w.tmat, lm, w.bsums);
+    const unsigned ng = (unsigned)((p->n_tiles + TS_BIN_GROUP - 1) / TS_BIN_GROUP);
+    k_bin_columns<<<ng, 32 * COL_WARPS, 0, s>>>(w.tmat, p->n_tiles, (int)p->bin_blocks, w.tcnt, w.bsums);
+    k_scan_bsums<<<1, SCAN_T, 0, s>>>(w.bsums, ng, &w.hdr->n_pairs, &w.hdr->error_bits, p->cap, &w.hdr->n_large);
     k_bin_place<<<grid, BIN_T, smem, s>>>(ma);
   } else {
     // 1-3 with global counts: counts, their scan, starts, places
@@ -640,14 +723,14 @@ cudaError_t ts_launch_bin(const TsPlanImpl* p, const TsWs& w, cudaStream_t s) {
     Len lt{p->n_tiles};
     const unsigned nb = (unsigned)((p->n_tiles + TS_SCAN_ITEMS - 1) / TS_SCAN_ITEMS);
     k_scan_reduce<<<nb, SCAN_T, 0, s>>>(w.tcnt, lt, w.bsums);
-    k_scan_bsums<<<1, SCAN_T, 0, s>>>(w.bsums, lt, &w.hdr->n_pairs, &w.hdr->error_bits, p->cap, &w.hdr->n_large);
+    k_scan_bsums<<<1, SCAN_T, 0, s>>>(w.bsums, nb, &w.hdr->n_pairs, &w.hdr->error_bits, p->cap, &w.hdr->n_large);
     k_tile_starts<<<nb, SCAN_T, 0, s>>>(ta, w.bsums);
     k_tile_scatter<<<nf, 256, 0, s>>>(ta);
   }
   // 4: the segments' sorts
   // (with the matrix, the sort also writes each tile's range)
   SortOut so{w.keys[1], w.keys[0], w.vals[0], w.ranges, p->n_tiles, p->cap, w.tlarge, &w.hdr->n_large,
-             p->bin_blocks > 0 ? w.tmat : nullptr, p->bin_blocks, &w.hdr->n_pairs};
+             p->bin_blocks > 0 ? w.tcnt : nullptr, w.bsums, &w.hdr->n_pairs};
   k_tile_sort<<<(unsigned)((p->n_tiles + SORT_WARPS_PER_BLOCK - 1) / SORT_WARPS_PER_BLOCK), 32 * SORT_WARPS_PER_BLOCK,
                 0, s>>>(so);
   constexpr int large_smem = 2 * LARGE_ITEMS * (int)sizeof(unsigned long long);

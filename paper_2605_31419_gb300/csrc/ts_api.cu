@@ -143,11 +143,13 @@ ts_status ts_plan_init(ts_plan* plan, const ts_camera* cams, int32_t n_views, in
   if (cap >= ((int64_t)1 << 32) - 4096) return TS_ERR_INVALID_ARG;
   p->cap = cap;
   p->max_view_tiles = max_tiles;
-  p->bin_blocks = max_tiles <= TS_BIN_MAX_TILES ? std::max<int64_t>(1, (n_faces + TS_BIN_FACES - 1) / TS_BIN_FACES) : 0;
-  {
-    const int64_t scanned = p->bin_blocks ? toff * p->bin_blocks : toff;
-    p->n_tile_scan_blocks = std::max<int64_t>(1, (scanned + TS_SCAN_ITEMS - 1) / TS_SCAN_ITEMS);
-  }
+  // faces per binning block: the fewest, from 1024 by powers of two, that leave at most 456 blocks (three on
+  // each of 152 multiprocessors); a larger problem takes the most, which keeps the count matrix small
+  p->bin_faces = 1024;
+  while (p->bin_faces < TS_BIN_FACES && n_views * ((n_faces + p->bin_faces - 1) / p->bin_faces) > 456) p->bin_faces *= 2;
+  p->bin_blocks = max_tiles <= TS_BIN_MAX_TILES ? std::max<int64_t>(1, (n_faces + p->bin_faces - 1) / p->bin_faces) : 0;
+  const int64_t scan_items = p->bin_blocks ? TS_BIN_GROUP : TS_SCAN_ITEMS;
+  p->n_tile_scan_blocks = std::max<int64_t>(1, (toff + scan_items - 1) / scan_items);
   p->n_pose_blocks = std::max(1, ts_pose_blocks(n_faces));
   int64_t max_hw = 0;
   for (int v = 0; v < n_views; ++v) max_hw = std::max<int64_t>(max_hw, (int64_t)p->views[v].W * p->views[v].H);

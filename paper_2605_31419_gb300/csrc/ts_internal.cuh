@@ -15,7 +15,8 @@
 #define TS_REC_WORDS 32            // 128-byte record, a multiple of 16 B for cp.async.bulk
 #define TS_GRAD_WORDS 32           // per-(view, face) gradient slot
 #define TS_SCAN_ITEMS 4096         // items per scan block (1024 threads x 4)
-#define TS_BIN_FACES 8192          // faces per block of the shared-memory tile counts
+#define TS_BIN_FACES 8192          // most faces per block of the shared-memory tile counts
+#define TS_BIN_GROUP 32            // tiles whose counts are scanned by one warp
 #define TS_BIN_MAX_TILES 40960     // the most tiles of a view those counts hold (160 KB)
 #define TS_ERRBIT_CAPACITY 1u
 #define TS_ERRBIT_TIMEOUT 2u
@@ -91,6 +92,7 @@ struct TsPlanImpl {
   ts_raster_params prm;
   int64_t n_tiles, n_pix;
   int64_t n_tile_scan_blocks, n_pose_blocks, n_loss_blocks, n_pho_blocks;
+  int64_t bin_faces;        // faces per block of the shared-memory tile counts
   int64_t bin_blocks;       // face blocks per view of the shared-memory tile counts (0: global counts)
   int64_t max_view_tiles;   // the most tiles of one view
   bool normals;  // TS_FLAG_NORMALS
@@ -117,9 +119,9 @@ struct TsWs {
   short4* rect;
   uint32_t* zbits;
   uint32_t* count;
-  uint32_t* tcnt;    // per tile: pairs (binning)
+  uint32_t* tcnt;    // per tile: pairs (global counts), or the pairs before it in its group (count matrix)
   uint32_t* tlarge;  // tiles whose pair lists the CTA-wide sort takes
-  uint32_t* tmat;    // [tile][face block] pair counts, then their exclusive scan
+  uint32_t* tmat;    // [face block][tile] pair counts, then their exclusive sums down the columns
   float* tloss;      // fused L1 step: per tile, the colour and depth L1 sums
   uint32_t* bsums;
   unsigned long long* keys[2];  // [0]: the sorted pair keys; [1]: the tile segments before their sort

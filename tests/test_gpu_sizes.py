@@ -28,6 +28,38 @@ def test_tile_sort_list_lengths(n):
     assert np.array_equal(rast.debug("keys").cpu().numpy().view(np.uint64)[:n], zb[order].astype(np.uint64))
 
 
+@pytest.mark.parametrize("n_faces,n_wide", [(1, 0), (33, 33), (1025, 3), (2049, 600), (9000, 300)])
+@pytest.mark.parametrize("n_views", [1, 3])
+def test_tile_lists_of_wide_faces(n_faces, n_wide, n_views):
+    """Binning around its rounds of faces and its queue of wide rectangles (256 a block), with rectangles on
+    both sides of 128 tiles: every tile's list holds exactly the faces whose rectangle covers it, by depth."""
+    rng = np.random.default_rng(n_faces + n_views)
+    z = rng.uniform(1.0, 2.0, n_faces)
+    size = np.where(np.arange(n_faces) < n_wide, rng.uniform(20.0, 400.0, n_faces), rng.uniform(1.0, 12.0, n_faces))
+    centre = rng.uniform([0.0, 0.0], [300.0, 200.0], (n_faces, 2)) - [150.0, 100.0]
+    tri = np.array([[-0.5, -0.5], [0.5, -0.5], [0.0, 0.5]])
+    xy = (centre[:, None] + tri[None] * size[:, None, None]) * (z / 100.0)[:, None, None]
+    pos = np.concatenate([xy, np.repeat(z[:, None, None], 3, 1)], 2)[rng.permutation(n_faces)]
+    poses = np.tile([1, 0, 0, 0, 1, 0, 0, 0, 1, 0, 0, 0.0], (n_views, 1))
+    poses[:, 9] = 0.1 * np.arange(n_views)
+    sc = Scene(pos.reshape(-1, 3).astype(np.float32), np.full((3 * n_faces, 3), 0.5, np.float32),
+               np.full(3 * n_faces, 0.5, np.float32), None, np.array([[100.0, 100.0, 150.0, 100.0, 300, 200]] * n_views),
+               poses.astype(np.float32))
+    p, _ = params_pair(tile_w=8, tile_h=8)
+    rast = gpu_run(sc, p, backward=False, pair_capacity=2_000_000)["rast"]
+    rect = rast.debug("rect").cpu().numpy().view(np.int16).reshape(n_views, n_faces, 4)
+    zb = rast.debug("zbits").cpu().numpy().view(np.uint32).reshape(n_views, n_faces)
+    ids, ranges = rast.debug("ids").cpu().numpy().view(np.uint32), rast.debug("ranges").cpu().numpy()
+    ranges = ranges.view(np.uint32).reshape(n_views, 25, 38, 2)
+    for v in range(n_views):
+        r = rect[v].astype(np.int64)
+        for ty in range(25):
+            for tx in range(38):
+                on = np.flatnonzero((r[:, 0] >= 0) & (r[:, 0] <= tx) & (tx <= r[:, 2]) & (r[:, 1] <= ty) & (ty <= r[:, 3]))
+                want = on[np.lexsort((on, zb[v][on]))]
+                assert np.array_equal(ids[ranges[v, ty, tx, 0]:ranges[v, ty, tx, 1]], want), (v, ty, tx)
+
+
 @pytest.mark.parametrize("n_faces", [1, 7, 33, 200])
 @pytest.mark.parametrize("n_views", [1, 2, 3, 7, 8, 33])
 def test_chain_rule_views_and_faces(oracle, n_views, n_faces):
