@@ -9,6 +9,8 @@
 //     keyframe selection compares.
 #include "ts_internal.cuh"
 
+static_assert(R_U0 == 0 && R_V0 == 3 && R_V1 == 4 && R_V2 == 5, "a record's first six words are its vertices");
+
 namespace {
 
 constexpr int ST_T = 256;
@@ -25,32 +27,60 @@ struct StatsArgs {
   uint32_t* n_visible;
 };
 
-// grid (ceil(M / 256), V): thread = face m of view v; a warp covers 32 faces of one view, so its
-// ballot is one word of the view's bitset
+// grid (ceil(M / 1024), V): 1024 faces of view v per block, 256 at a time; a warp covers 32 faces of one view,
+// so its ballot is one word of the view's bitset.  Bound by its 12 to 20 bytes per (view, face) and the
+// visible records' sectors.  The visible counts are summed per block: one add per warp queued 9,375 adds on
+// each view's address (8 views of 300k faces: 58 -> 23 us).
+constexpr int ST_PER = 4;
 __global__ void __launch_bounds__(ST_T) k_face_stats(StatsArgs a) {
+  __shared__ unsigned red[ST_T / 32];
   const int v = blockIdx.y;
-  const long long m = (long long)blockIdx.x * ST_T + threadIdx.x;
-  const long long idx = (long long)v * a.M + m;
-  const bool in = m < a.M;
-  const bool proj = in && a.count[idx] > 0;
-  const uint32_t cov = (proj && a.cov_in) ? a.cov_in[idx] : 0u;
-  if (in && a.coverage) a.coverage[idx] = cov;
-  if (in && a.area) {
-    float ar = 0.f;
-    if (proj) {
-      const float* r = reinterpret_cast<const float*>(a.frec + idx * (TS_REC_WORDS / 4));
-      const float du1 = __fsub_rn(r[R_U1], r[R_U0]), dv1 = __fsub_rn(r[R_V1], r[R_V0]);
-      const float du2 = __fsub_rn(r[R_U2], r[R_U0]), dv2 = __fsub_rn(r[R_V2], r[R_V0]);
-      ar = 0.5f * fabsf(__fsub_rn(__fmul_rn(du1, dv2), __fmul_rn(du2, dv1)));
-    }
-    a.area[idx] = ar;
+  unsigned seen = 0u;
+  const long long m0 = (long long)blockIdx.x * ST_PER * ST_T + threadIdx.x;
+  const long long base = (long long)v * a.M;
+  // all counts, then all coverages, then all records: the loads of one kind are in flight together
+  bool proj[ST_PER];
+  uint32_t cov[ST_PER];
+#pragma unroll
+  for (int k = 0; k < ST_PER; ++k) {
+    const long long m = m0 + k * ST_T;
+    proj[k] = m < a.M && a.count[base + m] > 0;
   }
-  if (a.visible || a.n_visible) {
-    const unsigned bal = __ballot_sync(0xffffffffu, cov > 0);
-    if ((threadIdx.x & 31) == 0 && m < a.M) {
-      if (a.visible) a.visible[(long long)v * a.words + (m >> 5)] = bal;
-      if (a.n_visible && bal) atomicAdd(a.n_visible + v, (unsigned)__popc(bal));
+#pragma unroll
+  for (int k = 0; k < ST_PER; ++k) cov[k] = (proj[k] && a.cov_in) ? a.cov_in[base + m0 + k * ST_T] : 0u;
+  if (a.area) {
+    float4 q[ST_PER];  // u0, u1, u2, v0
+    float2 p[ST_PER];  // v1, v2
+#pragma unroll
+    for (int k = 0; k < ST_PER; ++k) {
+      const float4* r = a.frec + (base + m0 + k * ST_T) * (TS_REC_WORDS / 4);
+      q[k] = proj[k] ? r[0] : make_float4(0.f, 0.f, 0.f, 0.f);
+      p[k] = proj[k] ? *reinterpret_cast<const float2*>(r + 1) : make_float2(0.f, 0.f);
     }
+#pragma unroll
+    for (int k = 0; k < ST_PER; ++k) {
+      const float du1 = __fsub_rn(q[k].y, q[k].x), dv1 = __fsub_rn(p[k].x, q[k].w);
+      const float du2 = __fsub_rn(q[k].z, q[k].x), dv2 = __fsub_rn(p[k].y, q[k].w);
+      if (m0 + k * ST_T < a.M)
+        a.area[base + m0 + k * ST_T] = 0.5f * fabsf(__fsub_rn(__fmul_rn(du1, dv2), __fmul_rn(du2, dv1)));
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < ST_PER; ++k) {
+    const long long m = m0 + k * ST_T;
+    if (a.coverage && m < a.M) a.coverage[base + m] = cov[k];
+    const unsigned bal = __ballot_sync(0xffffffffu, cov[k] > 0);
+    seen += __popc(bal);
+    if (a.visible && (threadIdx.x & 31) == 0 && m < a.M) a.visible[(long long)v * a.words + (m >> 5)] = bal;
+  }
+  if (!a.n_visible) return;
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = seen;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned s = 0u;
+#pragma unroll
+    for (int w = 0; w < ST_T / 32; ++w) s += red[w];
+    if (s) atomicAdd(a.n_visible + v, s);
   }
 }
 
@@ -107,7 +137,7 @@ cudaError_t ts_launch_face_stats(const TsPlanImpl* p, const TsWs& w, uint32_t* c
   a.area = area;
   a.visible = visible;
   a.n_visible = n_visible;
-  k_face_stats<<<dim3((unsigned)((p->M + ST_T - 1) / ST_T), (unsigned)p->V), ST_T, 0, s>>>(a);
+  k_face_stats<<<dim3((unsigned)((p->M + ST_PER * ST_T - 1) / (ST_PER * ST_T)), (unsigned)p->V), ST_T, 0, s>>>(a);
   return cudaGetLastError();
 }
 
