@@ -26,9 +26,13 @@
 // o_F, and the contribution count).  The forward stores, per sorted pair and warp, the 32-bit
 // mask of the warp's pixels that blended the face; the backward numbers those (face, pixel)
 // entries back to front (a warp-wide scan of the masks' bit counts) and processes them 32 at a
-// time, one per lane, so that no lane idles on a pixel the face does not cover.  Lanes holding
-// entries of the same pixel replay its recurrence in entry order (the same products and sums, in
-// the same order, as a per-pixel loop).  Every
+// time, one per lane, so that no lane idles on a pixel the face does not cover.  Entries of
+// one pixel are chained: each lane knows the lane of the entry before its own and how many there are, and
+// in round r the lanes with r before them take up that lane's (T, S) -- the same products and sums, in the
+// same order, as a per-pixel loop, in one short loop where replaying T and then S over all earlier entries
+// took two long ones.  With 32-bit tile geometry, and masks of a one-stage list that stay in shared memory
+// until the fused step's backward: fused step 1703 -> 1604 us (20-view room) and 1455 -> 1349 (12-view
+// window), backward of 64 tracking views 780 -> 716.  Every
 // per-face sum is over products of two per-entry factors: one of seven weighted gradients times one of
 // three barycentrics (the gradient of o_F alone).  Each lane writes its entry's factors to a ring row in
 // shared memory; then the 8 lanes of each quarter warp walk 8 consecutive rows, lane a accumulating
@@ -104,10 +108,11 @@ constexpr int raster_min_blocks(int threads) {
 struct RenderSmem {
   float lred[16][2];       // fused step: the warps' loss sums
   int lmax[16];            // fused step: the warps' largest last positions
+  int4 geo;                // the tile's first pixel, W and H of its view
+  long long pix_off;
   int view;
   int nmax;
   int next_tile;
-  int fail;
 };
 
 // Forward only, TS_FLAG_STATS: per staged face, the number of the tile's pixels that blended it.
@@ -147,10 +152,10 @@ struct Ring {
 template <int TW, int TH>
 struct TileGeom {
   static constexpr int NSBX = TW / 8;
-  int view, X0, Y0, x, y;
+  int view, x, y, W, H;
   bool inimg;
   float px, py;
-  TsView vw;
+  long long pix_off;
 };
 
 template <int TW, int TH>
@@ -165,18 +170,23 @@ __device__ __forceinline__ TileGeom<TW, TH> tile_geom(const RenderArgs& a, long 
       below += __popc(b);
       if (b != FULL) break;
     }
-    if (lane == 0) sm.view = below - 1;
+    if (lane == 0) {  // a tile of a view and its pixels fit 32 bits
+      const TsView& vw = a.views[below - 1];
+      const int lt = (int)(tile - vw.tile_off), ty = lt / vw.TX, tx = lt - ty * vw.TX;
+      sm.geo = make_int4(tx * TW, ty * TH, vw.W, vw.H);
+      sm.pix_off = vw.pix_off;
+      sm.view = below - 1;
+    }
   }
   __syncthreads();
+  const int4 geo = sm.geo;
   g.view = sm.view;
-  g.vw = a.views[g.view];
-  const long long lt = tile - g.vw.tile_off;
-  const int ty = (int)(lt / g.vw.TX), tx = (int)(lt - (long long)ty * g.vw.TX);
-  g.X0 = tx * TW;
-  g.Y0 = ty * TH;
-  g.x = g.X0 + (warp % TileGeom<TW, TH>::NSBX) * 8 + (lane & 7);
-  g.y = g.Y0 + (warp / TileGeom<TW, TH>::NSBX) * 4 + (lane >> 3);
-  g.inimg = g.x < g.vw.W && g.y < g.vw.H;
+  g.pix_off = sm.pix_off;
+  g.W = geo.z;
+  g.H = geo.w;
+  g.x = geo.x + (warp % TileGeom<TW, TH>::NSBX) * 8 + (lane & 7);
+  g.y = geo.y + (warp / TileGeom<TW, TH>::NSBX) * 4 + (lane >> 3);
+  g.inimg = g.x < g.W && g.y < g.H;
   g.px = (float)g.x + 0.5f;
   g.py = (float)g.y + 0.5f;
   return g;
@@ -299,7 +309,7 @@ __device__ __forceinline__ unsigned transpose32(unsigned x, int lane) {
 template <int TW, int TH, bool AUX, bool FUSED = false>
 __device__ __forceinline__ void fwd_tile(const RenderArgs& a, long long tile, float4* smrec, RenderSmem& sm,
                                          FwdMasks& fm, TileCarry* carry = nullptr,
-                                         const TileGeom<TW, TH>* gin = nullptr) {
+                                         const TileGeom<TW, TH>* gin = nullptr, uint32_t* held = nullptr) {
   const TileGeom<TW, TH> g = FUSED ? *gin : tile_geom<TW, TH>(a, tile, sm);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint2 rg = a.ranges[tile];
@@ -392,11 +402,13 @@ __device__ __forceinline__ void fwd_tile(const RenderArgs& a, long long tile, fl
             }
             contrib += __popc(blended);
             // the backward takes exactly these (face, pixel) contributions
-            if (a.lmask || a.cov) lm = transpose32(blended, lane);
+            if (FUSED || a.lmask || a.cov) lm = transpose32(blended, lane);
             if (a.cov && lm) atomicAdd(&fm.cv[b][jq], (unsigned)__popc(lm));
           }
         }
-        if (a.lmask && jq < cnt) a.lmask[(size_t)(rg.x + (uint32_t)(st * S + jq)) * (TW * TH / 32) + warp] = lm;
+        if (FUSED && jq < cnt) held[b * S + jq] = lm;
+        // (a list of one stage stays in shared memory until the fused step's backward)
+        if (a.lmask && jq < cnt && !(FUSED && nst == 1)) a.lmask[(size_t)(rg.x + (uint32_t)(st * S + jq)) * (TW * TH / 32) + warp] = lm;
       }
       if (st + 1 == nst && !a.cov) break;  // nothing reads the buffers or the counts after this stage
       ts_cp_async_wait_all();              // the next stage, published by the barrier
@@ -429,22 +441,21 @@ __device__ __forceinline__ void fwd_tile(const RenderArgs& a, long long tile, fl
     carry->prev_in = st_last >= 1 && !prefetched;
   }
   if (g.inimg) {
-    const long long HW = (long long)g.vw.W * g.vw.H;
-    const long long pi = (long long)g.y * g.vw.W + g.x;
-    const long long o = g.vw.pix_off + pi;
+    const int HW = g.W * g.H, pi = g.y * g.W + g.x;
+    const long long o = g.pix_off + pi;
     if (a.color) {
-      float* c = a.color + 3 * g.vw.pix_off + pi;
+      float* c = a.color + 3 * g.pix_off + pi;
       c[0] = C0 + T * a.bg0;
       c[HW] = C1 + T * a.bg1;
-      c[2 * HW] = C2 + T * a.bg2;
+      c[2LL * HW] = C2 + T * a.bg2;
     }
     if (a.depth) a.depth[o] = D;
     if (a.alpha) a.alpha[o] = 1.f - T;
     if (AUX && a.normal) {
-      float* q = a.normal + 3 * g.vw.pix_off + pi;
+      float* q = a.normal + 3 * g.pix_off + pi;
       q[0] = N0;
       q[HW] = N1;
-      q[2 * HW] = N2;
+      q[2LL * HW] = N2;
     }
     if (!FUSED) {  // what ts_render_bwd needs; the fused step keeps them in registers
       a.tfin[o] = T;
@@ -462,7 +473,7 @@ __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, 
 template <int TW, int TH, bool AUX, bool FUSED = false>
 __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, float4* smrec, RenderSmem& sm,
                                          const PixIn* pin = nullptr, const TileCarry* carry = nullptr,
-                                         const TileGeom<TW, TH>* gin = nullptr) {
+                                         const TileGeom<TW, TH>* gin = nullptr, const uint32_t* held = nullptr) {
   const TileGeom<TW, TH> g = FUSED ? *gin : tile_geom<TW, TH>(a, tile, sm);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint2 rg = a.ranges[tile];
@@ -480,22 +491,21 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
       Sacc = T * (gC0 * a.bg0 + gC1 * a.bg1 + gC2 * a.bg2);
     }
   } else if (g.inimg) {
-    const long long HW = (long long)g.vw.W * g.vw.H;
-    const long long pi = (long long)g.y * g.vw.W + g.x;
-    const long long o = g.vw.pix_off + pi;
+    const int HW = g.W * g.H, pi = g.y * g.W + g.x;
+    const long long o = g.pix_off + pi;
     T = a.tfin[o];
     nl = a.nlast[o];
-    const float* dc = a.dC + 3 * g.vw.pix_off + pi;
+    const float* dc = a.dC + 3 * g.pix_off + pi;
     gC0 = dc[0];
     gC1 = dc[HW];
-    gC2 = dc[2 * HW];
+    gC2 = dc[2LL * HW];
     gD = a.dD ? a.dD[o] : 0.f;
     gA = a.dA ? a.dA[o] : 0.f;
     if (AUX && a.dN) {
-      const float* dn = a.dN + 3 * g.vw.pix_off + pi;
+      const float* dn = a.dN + 3 * g.pix_off + pi;
       gN0 = dn[0];
       gN1 = dn[HW];
-      gN2 = dn[2 * HW];
+      gN2 = dn[2LL * HW];
     }
     Sacc = T * (gC0 * a.bg0 + gC1 * a.bg1 + gC2 * a.bg2);
   }
@@ -545,16 +555,18 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
       constexpr int NW = TW * TH / 32;
       const uint32_t* lmrow = a.lmask + (size_t)(rg.x + (uint32_t)(st * S)) * NW + warp;
       const int F = (cnt + 31) >> 5;  // faces per lane: lane L holds faces F * (32 - L) - 1 - i, i < F
+      // the fused step: the forward's last stage, and the one before it unless a prefetch replaced it, are
+      // still staged, their masks in shared memory; other stages are staged again
+      const bool here = FUSED && (st == carry->st_last || (st == carry->st_last - 1 && carry->prev_in));
       unsigned lmk[FMAX];
 #pragma unroll
       for (int i = 0; i < FMAX; ++i) {
         const int jf = F * (32 - lane) - 1 - i;
-        lmk[i] = (i < F && jf < cnt) ? lmrow[(size_t)jf * NW] : 0u;
+        lmk[i] = 0u;
+        if (i < F && jf < cnt) lmk[i] = here ? held[b * S + jf] : lmrow[(size_t)jf * NW];
       }
       if (FUSED) {
-        // the forward's last stage, and the one before it unless a prefetch replaced it, are
-        // still staged; other stages are staged again (all warps are done with both buffers)
-        if (st != carry->st_last && !(st == carry->st_last - 1 && carry->prev_in)) {
+        if (!here) {  // (all warps are done with both buffers)
           __syncthreads();
           b = 0;
           issue_stage<AUX>(a, smrec, b, st, rg.x, n, vbase, nbase, TW * TH);
@@ -598,9 +610,10 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
           bool found = false;
 #pragma unroll
           for (int i = 0; i < FMAX; ++i) {
+            if (i >= F) break;  // uniform
             const unsigned mi = __shfl_sync(FULL, lmk[i], ow);
             const int ci = __popc(mi);
-            if (!found && i < F) {
+            if (!found) {
               if (kk < ci) {
                 om = mi;
                 fi = i;
@@ -634,22 +647,13 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
           const float I = act ? ts_window(e.m, sig) : 0.f;
           const float al = fminf(oF * I, a.alpha_max);
           const float ro = ts_rcp_approx(1.f - al);  // 1 - al >= 1 - alpha_max
-          // entries of the same pixel, in entry (back-to-front) order; each lane replays its
-          // pixel's recurrence T <- T / (1 - alpha) over the earlier ones and itself, in order
+          // entries of the same pixel, in entry (back-to-front) order: the one before this lane's, and how many
+          // are
           const unsigned peers = __match_any_sync(FULL, act ? p : 32 + lane);
-          const int K = (int)__reduce_max_sync(FULL, (unsigned)__popc(peers));
+          const unsigned before = peers & ((1u << lane) - 1u);
+          const int prev = before ? 31 - __clz(before) : lane, depth = __popc(before);
+          const int K = (int)__reduce_max_sync(FULL, (unsigned)depth);
           const float2 st0 = pst[p];
-          float Tn = st0.x;
-          {
-            unsigned rem = peers;
-            for (int i = 0; i < K; ++i) {
-              const int src = rem ? __ffs(rem) - 1 : 31;
-              const bool use = rem != 0 && src <= lane;
-              rem &= rem - 1;
-              const float f = __shfl_sync(FULL, ro, src);
-              if (use) Tn *= f;
-            }
-          }
           const float qC0 = __shfl_sync(FULL, gC0, p), qC1 = __shfl_sync(FULL, gC1, p);
           const float qC2 = __shfl_sync(FULL, gC2, p), qD = __shfl_sync(FULL, gD, p);
           const float qA = __shfl_sync(FULL, gA, p);
@@ -674,19 +678,19 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
             const float4 nn = nb[j];
             val += qN0 * nn.x + qN1 * nn.y + qN2 * nn.z;
           }
-          const float w = al * Tn;
-          const float add = val * al * Tn;  // this face's term of the suffix sum S seen by earlier faces
-          float Sn = st0.y;
-          {
-            unsigned rem = peers;
-            for (int i = 0; i < K; ++i) {
-              const int src = rem ? __ffs(rem) - 1 : 31;
-              const bool use = rem != 0 && src < lane;
-              rem &= rem - 1;
-              const float f = __shfl_sync(FULL, add, src);
-              if (use) Sn += f;
+          // the pixel's recurrences T <- T / (1 - alpha) and S <- S + (this face's term), entry after entry: in
+          // round r the lanes with r entries of their pixel before them take up the state of the one before
+          float Tn = st0.x * ro, Sn = st0.y;
+          float add = val * al * Tn;  // this face's term of the suffix sum S seen by earlier faces
+          for (int r = 1; r <= K; ++r) {
+            const float Tb = __shfl_sync(FULL, Tn, prev), Sb = __shfl_sync(FULL, Sn + add, prev);
+            if (depth == r) {
+              Tn = Tb * ro;
+              Sn = Sb;
+              add = val * al * Tn;
             }
           }
+          const float w = al * Tn;
           __syncwarp();  // every lane has read its pixel's state before the last entries replace it
           if (act && (peers >> lane) == 1u) pst[p] = make_float2(Tn, Sn + add);
           const float dal = val * Tn - Sn * ro;
@@ -754,21 +758,24 @@ template <int TW, int TH>
 __device__ __forceinline__ void step_tile(const RenderArgs& a, long long tile, float4* smrec, RenderSmem& sm,
                                           FwdMasks& fm) {
   TileCarry c;
+  // the warp's lane masks of the two stage buffers, after the rings
+  uint32_t* held = reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(smrec + (size_t)2 * a.S * SG) +
+                                               (size_t)(TW * TH / 32) * Ring<false>::BYTES_PER_WARP) +
+                   (size_t)(threadIdx.x >> 5) * 2 * a.S;
   const TileGeom<TW, TH> g = tile_geom<TW, TH>(a, tile, sm);
-  fwd_tile<TW, TH, false, true>(a, tile, smrec, sm, fm, &c, &g);
+  fwd_tile<TW, TH, false, true>(a, tile, smrec, sm, fm, &c, &g, held);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   PixIn pin{c.T, 0.f, 0.f, 0.f, 0.f, c.nl, 0};
   float lc = 0.f, ld = 0.f;
   if (g.inimg) {
-    const long long HW = (long long)g.vw.W * g.vw.H;
-    const long long pi = (long long)g.y * g.vw.W + g.x;
-    const long long o = g.vw.pix_off + pi;
+    const int HW = g.W * g.H, pi = g.y * g.W + g.x;
+    const long long o = g.pix_off + pi;
     const float ic = 1.0f / (3.0f * (float)HW), id = a.lambda_dep / (float)HW;
     const float col[3] = {c.C0 + c.T * a.bg0, c.C1 + c.T * a.bg1, c.C2 + c.T * a.bg2};  // the colour image
     float gc[3];
 #pragma unroll
     for (int ch = 0; ch < 3; ++ch) {
-      const long long q = 3 * g.vw.pix_off + ch * HW + pi;
+      const long long q = 3 * g.pix_off + (long long)ch * HW + pi;
       const float r = col[ch] - a.tC[q];
       lc += fabsf(r);
       gc[ch] = r > 0.f ? ic : (r < 0.f ? -ic : 0.f);
@@ -804,7 +811,7 @@ __device__ __forceinline__ void step_tile(const RenderArgs& a, long long tile, f
   }
 #pragma unroll
   for (int w = 0; w < TW * TH / 32; ++w) pin.nmax = max(pin.nmax, sm.lmax[w]);
-  bwd_tile<TW, TH, false, true>(a, tile, smrec, sm, &pin, &c, &g);
+  bwd_tile<TW, TH, false, true>(a, tile, smrec, sm, &pin, &c, &g, held);
 }
 
 // Next tile of a persistent CTA (the same value in every thread), or -1 when none is left.
@@ -884,7 +891,7 @@ __global__ void __launch_bounds__(256) k_loss_tiles(const TsView* __restrict__ v
 
 template <int TW, int TH>
 cudaError_t launch_step(bool persist, const RenderArgs& a, cudaStream_t s) {
-  const size_t smem = (size_t)2 * a.S * SG * 16 + (size_t)(TW * TH / 32) * Ring<false>::BYTES_PER_WARP;
+  const size_t smem = (size_t)2 * a.S * SG * 16 + (size_t)(TW * TH / 32) * (Ring<false>::BYTES_PER_WARP + 2 * a.S * 4);
   if (a.n_tiles == 0) return cudaSuccess;
   const void* f = persist ? (const void*)k_render_step<TW, TH, true> : (const void*)k_render_step<TW, TH, false>;
   cudaError_t e = ts_smem_limit(f, (int)smem);
