@@ -37,10 +37,11 @@
 // three barycentrics (the gradient of o_F alone).  Each lane writes its entry's factors to a ring row in
 // shared memory; then the 8 lanes of each quarter warp walk 8 consecutive rows, lane a accumulating
 // factor a times the three barycentrics, and add them into the face's accumulator with one four-word
-// reduction per lane where a face's entries end and after the last row: 8 unrolled steps a batch (about
-// 100 instructions) where a loop over the faces' runs, one word per lane, took about 210: the backward of
-// 64 tracking views 1034 -> 918 us, the fused step 1645 -> 1585 us (20-view room), 1441 -> 1313 (12-view
-// window).
+// reduction per lane at the rows that end a face's entries or the quarter, which one ballot marks: 8
+// unrolled steps a batch.  The reductions themselves cost nothing measurable; the instructions do.  (A loop
+// over the faces' runs, one word per lane: the backward of 64 tracking views 1034 -> 918 us; testing every
+// row's sums for zero and the slot in 64 bits: fused step 1321 -> 1244 us for the 12-view window, backward
+// of 6 mapping views 172 -> 164.)  A list of one stage is staged whole while the pixels' inputs load.
 //
 // Launch forms: one CTA per tile, or persistent CTAs (as many as fit on the GPU) that take tiles
 // from a device counter.  The fused L1 step (ts_render_step_l1) runs a tile's forward, its loss
@@ -93,15 +94,15 @@ struct RenderArgs {
 
 constexpr unsigned FULL = 0xffffffffu;
 
-// Register budget of the raster kernels per thread (0: the compiler's choice), expressed as the
-// minimum number of resident CTAs in the launch bounds.  Both kernels are latency-bound: on the
-// room workload (tile 16x8) 56 registers beat the compiler's unconstrained 87-104 by 20 % and
-// 64 or 72 registers by 1-4 %, small spills included.
-#ifndef TS_RASTER_REGS
-#define TS_RASTER_REGS 56
-#endif
-constexpr int raster_min_blocks(int threads) {
-  return TS_RASTER_REGS > 0 ? (65536 / (threads * TS_RASTER_REGS) > 0 ? 65536 / (threads * TS_RASTER_REGS) : 1) : 1;
+// Register budgets of the raster kernels per thread, expressed as the minimum number of resident CTAs in the
+// launch bounds.  More
+// resident CTAs hide more latency until spills cost more: 64 tracking views at 40 / 48 / 56 / 64 registers
+// take the forward 614 / 547 / 580 / 609 us and the backward 826 / 691 / 716 / 768; with the side array, 6
+// mapping views at 48 / 56 / 64 / 72 take the forward 124 / 116 / 119 / - and the backward 201 / 192 / 179 /
+// 166; the fused step of 20 views 1624 / 1604 / 1602 / -.
+constexpr int REGS_FWD = 48, REGS_BWD = 48, REGS_STEP = 56, REGS_FWD_AUX = 56, REGS_BWD_AUX = 72;
+constexpr int raster_min_blocks(int threads, int regs) {
+  return 65536 / (threads * regs) > 0 ? 65536 / (threads * regs) : 1;
 }
 
 // Shared state of a render CTA.
@@ -196,22 +197,26 @@ __device__ __forceinline__ TileGeom<TW, TH> tile_geom(const RenderArgs& a, long 
 // e1 and e2).
 constexpr int SG = 7;
 
+// Face id at place `at` of the sorted pair list.
+__device__ __forceinline__ uint32_t list_id(const RenderArgs& a, uint32_t at) {
+  const uint32_t id = __ldg(a.ids + at);
+  if ((long long)id < a.M) return id;
+  atomicOr(&a.hdr->error_bits, TS_ERRBIT_BOUNDS);  // never expected: record the fault, stage an in-bounds record
+  return 0u;
+}
+
 // Every thread of the CTA copies 16-byte groups of stage `st` (records [st*S, st*S + cnt) of the
 // tile's list) into buffer `b` with cp.async, SG groups per record and, with the side array, one more
 // for the record's side entry (normal, sigma_F) after both record buffers; one commit group per stage.
 template <bool AUX>
-__device__ __forceinline__ void issue_stage(const RenderArgs& a, float4* smrec, int b, int st, uint32_t start, int n,
-                                            const float4* vbase, const float4* nbase, int nthreads) {
+__device__ __forceinline__ void issue_stage(const RenderArgs& a, float4* smrec, int b, int st, uint32_t start,
+                                            int n, const float4* vbase, const float4* nbase, int nthreads) {
   const int S = a.S;
   const int cnt = min(S, n - st * S);
   constexpr int PER = AUX ? SG + 1 : SG;
   for (int i = threadIdx.x; i < cnt * PER; i += nthreads) {
     const int j = i / PER, c = i - j * PER;
-    uint32_t id = __ldg(a.ids + start + (uint32_t)(st * S + j));
-    if ((long long)id >= a.M) {  // never expected: record the fault and stage an in-bounds record
-      atomicOr(&a.hdr->error_bits, TS_ERRBIT_BOUNDS);
-      id = 0;
-    }
+    const uint32_t id = list_id(a, start + (uint32_t)(st * S + j));
     if (!AUX || c < SG) {
       ts_cp_async16(smrec + ((size_t)b * S + j) * SG + c, vbase + (size_t)id * 8 + (c < 2 ? c : c + 1));
     } else {
@@ -309,10 +314,12 @@ __device__ __forceinline__ unsigned transpose32(unsigned x, int lane) {
 template <int TW, int TH, bool AUX, bool FUSED = false>
 __device__ __forceinline__ void fwd_tile(const RenderArgs& a, long long tile, float4* smrec, RenderSmem& sm,
                                          FwdMasks& fm, TileCarry* carry = nullptr,
-                                         const TileGeom<TW, TH>* gin = nullptr, uint32_t* held = nullptr) {
+                                         const TileGeom<TW, TH>* gin = nullptr, const uint2* rgin = nullptr,
+                                         uint32_t* held = nullptr) {
+  // (the list's range loads while the view is looked up)
+  const uint2 rg = FUSED ? *rgin : a.ranges[tile];
   const TileGeom<TW, TH> g = FUSED ? *gin : tile_geom<TW, TH>(a, tile, sm);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint2 rg = a.ranges[tile];
   const int n = (int)(rg.y - rg.x);
   float T = 1.f, C0 = 0.f, C1 = 0.f, C2 = 0.f, D = 0.f;
   float N0 = 0.f, N1 = 0.f, N2 = 0.f;
@@ -473,10 +480,18 @@ __device__ __forceinline__ void red_add_v4(float* p, float a, float b, float c, 
 template <int TW, int TH, bool AUX, bool FUSED = false>
 __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, float4* smrec, RenderSmem& sm,
                                          const PixIn* pin = nullptr, const TileCarry* carry = nullptr,
-                                         const TileGeom<TW, TH>* gin = nullptr, const uint32_t* held = nullptr) {
+                                         const TileGeom<TW, TH>* gin = nullptr, const uint2* rgin = nullptr,
+                                         const uint32_t* held = nullptr) {
+  // (the list's range loads while the view is looked up)
+  const uint2 rg = FUSED ? *rgin : a.ranges[tile];
   const TileGeom<TW, TH> g = FUSED ? *gin : tile_geom<TW, TH>(a, tile, sm);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const uint2 rg = a.ranges[tile];
+  const int len = (int)(rg.y - rg.x);
+  const float4* vbase = a.frec + (size_t)g.view * (size_t)a.M * 8;
+  const float4* nbase = AUX ? a.aux + (size_t)g.view * (size_t)a.M : nullptr;
+  // a list of one stage is staged while the pixels' inputs load, without waiting for their last positions
+  const bool whole = !FUSED && len <= a.S;
+  if (whole && len > 0) issue_stage<AUX>(a, smrec, 0, 0, rg.x, len, vbase, nbase, TW * TH);
   float T = 0.f, Sacc = 0.f, gC0 = 0.f, gC1 = 0.f, gC2 = 0.f, gD = 0.f, gA = 0.f;
   float gN0 = 0.f, gN1 = 0.f, gN2 = 0.f;
   int nl = 0;
@@ -512,6 +527,8 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
   int nmax;
   if (FUSED) {
     nmax = pin->nmax;  // the tile's largest last position, reduced with the loss sums
+  } else if (whole) {
+    nmax = len;  // the forward wrote the masks of the whole stage
   } else {
     if (threadIdx.x == 0) sm.nmax = 0;
     __syncthreads();
@@ -524,14 +541,12 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
   }
   // positions come from the forward pass over the same lists; clamp in case the caller did not
   // run it after the last ts_bin
-  const int n = min(nmax, (int)(rg.y - rg.x));
+  const int n = min(nmax, len);
   unsigned contrib = 0;
   if (n > 0) {
     const int S = a.S;
     const int nst = (n + S - 1) / S;
-    const float4* vbase = a.frec + (size_t)g.view * (size_t)a.M * 8;
-    const float4* nbase = AUX ? a.aux + (size_t)g.view * (size_t)a.M : nullptr;
-    if (!FUSED) issue_stage<AUX>(a, smrec, (nst - 1) & 1, nst - 1, rg.x, n, vbase, nbase, TW * TH);
+    if (!FUSED && !whole) issue_stage<AUX>(a, smrec, (nst - 1) & 1, nst - 1, rg.x, n, vbase, nbase, TW * TH);
     constexpr int EW = Ring<AUX>::EW;
     unsigned char* wbase = reinterpret_cast<unsigned char*>(smrec + (size_t)2 * S * (AUX ? SG + 1 : SG)) +
                            (size_t)warp * Ring<AUX>::BYTES_PER_WARP;
@@ -541,6 +556,7 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
     float* row_here = ring + lane * EW + (lane >> 3) * 8;                      // this lane's entry's row
     const float* row_sum = ring + (lane >> 3) * (8 * EW + 8);                  // its quarter warp's first row
     const int fa = lane & 7;                                                   // the factor it sums
+    const uint32_t vm32 = (uint32_t)min(a.VM, 0xffffffffll);                   // slots
     const int xw = g.x - (lane & 7), yw = g.y - (lane >> 3);  // the warp's first pixel
     for (int k = 0; k < nst; ++k) {
       const int st = nst - 1 - k;
@@ -717,7 +733,8 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
           }
           // the batch's faces are runs of consecutive entries: rows that end one
           const int jnext = __shfl_down_sync(FULL, j, 1);
-          const unsigned ends = __ballot_sync(FULL, act && (lane == ne - 1 || j != jnext)) >> (lane & 24);
+          // and, so that every quarter's sums are added, the last active row of each
+          const unsigned ends = __ballot_sync(FULL, act && (lane == ne - 1 || j != jnext || (lane & 7) == 7)) >> (lane & 24);
           __syncwarp();
           float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
 #pragma unroll
@@ -728,15 +745,13 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
             s1 = fmaf(f, l.y, s1);
             s2 = fmaf(f, l.z, s2);
             if (AUX && fa < 4) s3 += row_sum[i * EW + 12 + fa];
-            if (i == 7 || (ends >> i) & 1u) {
+            if ((ends >> i) & 1u) {
               if (fa == 7) s1 = s2 = 0.f;
-              if (s0 != 0.f || s1 != 0.f || s2 != 0.f || s3 != 0.f) {
-                const uint32_t sl = __float_as_uint(l.w);
-                if ((long long)sl < a.VM) {
-                  red_add_v4(a.grad + (size_t)sl * TS_GRAD_WORDS + 4 * fa, s0, s1, s2, s3);
-                } else {
-                  atomicOr(&a.hdr->error_bits, TS_ERRBIT_BOUNDS);
-                }
+              const uint32_t sl = __float_as_uint(l.w);
+              if (sl < vm32) {
+                red_add_v4(a.grad + (size_t)sl * TS_GRAD_WORDS + 4 * fa, s0, s1, s2, s3);
+              } else {
+                atomicOr(&a.hdr->error_bits, TS_ERRBIT_BOUNDS);
               }
               s0 = s1 = s2 = s3 = 0.f;
             }
@@ -762,8 +777,9 @@ __device__ __forceinline__ void step_tile(const RenderArgs& a, long long tile, f
   uint32_t* held = reinterpret_cast<uint32_t*>(reinterpret_cast<unsigned char*>(smrec + (size_t)2 * a.S * SG) +
                                                (size_t)(TW * TH / 32) * Ring<false>::BYTES_PER_WARP) +
                    (size_t)(threadIdx.x >> 5) * 2 * a.S;
+  const uint2 rg = a.ranges[tile];
   const TileGeom<TW, TH> g = tile_geom<TW, TH>(a, tile, sm);
-  fwd_tile<TW, TH, false, true>(a, tile, smrec, sm, fm, &c, &g, held);
+  fwd_tile<TW, TH, false, true>(a, tile, smrec, sm, fm, &c, &g, &rg, held);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   PixIn pin{c.T, 0.f, 0.f, 0.f, 0.f, c.nl, 0};
   float lc = 0.f, ld = 0.f;
@@ -811,7 +827,7 @@ __device__ __forceinline__ void step_tile(const RenderArgs& a, long long tile, f
   }
 #pragma unroll
   for (int w = 0; w < TW * TH / 32; ++w) pin.nmax = max(pin.nmax, sm.lmax[w]);
-  bwd_tile<TW, TH, false, true>(a, tile, smrec, sm, &pin, &c, &g, held);
+  bwd_tile<TW, TH, false, true>(a, tile, smrec, sm, &pin, &c, &g, &rg, held);
 }
 
 // Next tile of a persistent CTA (the same value in every thread), or -1 when none is left.
@@ -823,7 +839,7 @@ __device__ __forceinline__ long long next_tile(const RenderArgs& a, RenderSmem& 
 }
 
 template <int TW, int TH, bool PERSIST, bool AUX>
-__global__ void __launch_bounds__(TW * TH, raster_min_blocks(TW * TH)) k_render_fwd(RenderArgs a) {
+__global__ void __launch_bounds__(TW * TH, raster_min_blocks(TW * TH, AUX ? REGS_FWD_AUX : REGS_FWD)) k_render_fwd(RenderArgs a) {
   extern __shared__ __align__(128) float4 smrec[];
   __shared__ RenderSmem sm;
   __shared__ FwdMasks fm;
@@ -836,7 +852,7 @@ __global__ void __launch_bounds__(TW * TH, raster_min_blocks(TW * TH)) k_render_
 }
 
 template <int TW, int TH, bool PERSIST, bool AUX>
-__global__ void __launch_bounds__(TW * TH, raster_min_blocks(TW * TH)) k_render_bwd(RenderArgs a) {
+__global__ void __launch_bounds__(TW * TH, raster_min_blocks(TW * TH, AUX ? REGS_BWD_AUX : REGS_BWD)) k_render_bwd(RenderArgs a) {
   extern __shared__ __align__(128) float4 smrec[];
   __shared__ RenderSmem sm;
   if constexpr (!PERSIST) {
@@ -850,7 +866,7 @@ __global__ void __launch_bounds__(TW * TH, raster_min_blocks(TW * TH)) k_render_
 // The fused step kernel.  Its forward's coverage counts (TS_FLAG_STATS) live in the space of the
 // backward's rings, which the forward does not use.
 template <int TW, int TH, bool PERSIST>
-__global__ void __launch_bounds__(TW * TH, raster_min_blocks(TW * TH)) k_render_step(RenderArgs a) {
+__global__ void __launch_bounds__(TW * TH, raster_min_blocks(TW * TH, REGS_STEP)) k_render_step(RenderArgs a) {
   extern __shared__ __align__(128) float4 smrec[];
   __shared__ RenderSmem sm;
   static_assert(sizeof(FwdMasks) <= (TW * TH / 32) * Ring<false>::BYTES_PER_WARP, "coverage counts fit the rings");
