@@ -10,13 +10,16 @@
 // Forward: for 32 staged faces at a time, lane = face computes which of the warp's 32 pixels its face
 // can cover (per pixel row the interval between its edges, widened: conservative); a 32 x 32 bit
 // transpose gives every pixel the faces to visit, and then lane = pixel walks its own faces front to
-// back, two per pass: window (Eq. 3) from cancellation-free edge functions, alpha = min(alpha_max,
+// back: window (Eq. 3) from cancellation-free edge functions, alpha = min(alpha_max,
 // o_F I), skip below alpha_min, stop before the face that would take T below T_min, accumulate colour,
 // depth and opacity (Eq. 4).  A warp's cost is its longest pixel list instead of all the faces of its
 // sub-block, each of which 5 of 32 pixels blend: issue-bound either way, the forward of 9 views of a
 // 2M-face map went from 1182 to 688 us, of 64 tracking views from 878 to 687, and the fused step from
-// 1893 to 1645 us (20-view room) and 1823 to 1441 (12-view window), images bit for bit.  The transpose of the blended bits gives, per face, the mask of the warp's pixels that
-// blended it.  Writes C + T bg, D, A = 1 - T, per pixel T_final and the list position after the last
+// 1893 to 1645 us (20-view room) and 1823 to 1441 (12-view window), images bit for bit.  (Two faces per
+// pass leave half a pass idle at the end of every odd list, and their code is twice as long: one per pass
+// takes the forward of 64 tracking views from 555 to 512 us at 40 registers, of 9 views of 2M faces from 697
+// to 663, the fused step of the 12-view window from 1244 to 1199.)  The transpose of the blended bits gives,
+// per face, the mask of the warp's pixels that blended it.  Writes C + T bg, D, A = 1 - T, per pixel T_final and the list position after the last
 // contribution, and per sorted pair and warp that mask.
 //
 // Backward: per pixel, back to front from that position: recover T_n = T_{n+1} / (1 - alpha_n),
@@ -96,11 +99,11 @@ constexpr unsigned FULL = 0xffffffffu;
 
 // Register budgets of the raster kernels per thread, expressed as the minimum number of resident CTAs in the
 // launch bounds.  More
-// resident CTAs hide more latency until spills cost more: 64 tracking views at 40 / 48 / 56 / 64 registers
-// take the forward 614 / 547 / 580 / 609 us and the backward 826 / 691 / 716 / 768; with the side array, 6
-// mapping views at 48 / 56 / 64 / 72 take the forward 124 / 116 / 119 / - and the backward 201 / 192 / 179 /
-// 166; the fused step of 20 views 1624 / 1604 / 1602 / -.
-constexpr int REGS_FWD = 48, REGS_BWD = 48, REGS_STEP = 56, REGS_FWD_AUX = 56, REGS_BWD_AUX = 72;
+// resident CTAs hide more latency until spills cost more: 64 tracking views take the forward 512 us at 40
+// and 538 at 48, the backward 686 at 48, 669 at 56 and 768 at 64; with the side array, 6 mapping views take
+// the forward 112 at 48 and 116 at 56, the backward 201 / 192 / 179 / 166 at 48 / 56 / 64 / 72; the fused step
+// of the 12-view window takes 1247 / 1216 / 1260 at 48 / 56 / 64.
+constexpr int REGS_FWD = 40, REGS_BWD = 56, REGS_STEP = 56, REGS_FWD_AUX = 48, REGS_BWD_AUX = 72;
 constexpr int raster_min_blocks(int threads, int regs) {
   return 65536 / (threads * regs) > 0 ? 65536 / (threads * regs) : 1;
 }
@@ -356,54 +359,38 @@ __device__ __forceinline__ void fwd_tile(const RenderArgs& a, long long tile, fl
             if (done) bits = 0u;
             unsigned blended = 0u;
             while (bits) {
-              const int j0 = __ffs(bits) - 1;
+              const int j = __ffs(bits) - 1;
               bits &= bits - 1;
-              const bool two = bits != 0;
-              const int j1 = two ? __ffs(bits) - 1 : j0;
-              bits &= bits - 1;
-              // two faces per pass: both edge functions first (independent work the scheduler can overlap),
-              // then the compositing in list order, exactly as one face at a time
-              const float4* r0 = rb + (q * 32 + j0) * SG;
-              const float4* r1 = rb + (q * 32 + j1) * SG;
-              const float4 k0 = r0[2], k1 = r1[2];
-              const TsPix e0 = eval_edges(r0[0], r0[1], k0, g.px, g.py);
-              const TsPix e1 = eval_edges(r1[0], r1[1], k1, g.px, g.py);
-#pragma unroll
-              for (int h = 0; h < 2; ++h) {
-                if (h == 1 && !two) break;
-                const int j = h ? j1 : j0;
-                const float4* r = h ? r1 : r0;
-                const TsPix e = h ? e1 : e0;
-                if (!done && e.m > 0.f) {
-                  const float4 q4 = r[3];  // o_F, colour of vertex 0
-                  const float sig = (AUX && a.face_sigma) ? nb[q * 32 + j].w : a.sigma;
-                  const float I = ts_window(e.m, sig);
-                  const float al = fminf(q4.x * I, a.alpha_max);
-                  if (al >= a.alpha_min) {
-                    const float Tn = T * (1.f - al);
-                    if (Tn < a.T_min) {
-                      done = true;
-                      bits = 0u;
-                    } else {
-                      const float invD = h ? k1.w : k0.w;
-                      const float l0 = e.cr1 * invD, l1 = e.cr2 * invD, l2 = e.cr0 * invD;
-                      const float w = al * T;
-                      const float4 q5 = r[4], q6 = r[5];  // colours of vertices 1 and 2, depths z_0, z_1
-                      C0 += w * (l0 * q4.y + l1 * q5.x + l2 * q5.w);
-                      C1 += w * (l0 * q4.z + l1 * q5.y + l2 * q6.x);
-                      C2 += w * (l0 * q4.w + l1 * q5.z + l2 * q6.y);
-                      D += w * (l0 * q6.z + l1 * q6.w + l2 * r[6].x);
-                      if (AUX && a.normals) {
-                        const float4 nn = nb[q * 32 + j];
-                        N0 += w * nn.x;
-                        N1 += w * nn.y;
-                        N2 += w * nn.z;
-                      }
-                      T = Tn;
-                      nl = st * S + q * 32 + j + 1;
-                      blended |= 1u << j;
-                    }
+              const float4* r = rb + (q * 32 + j) * SG;
+              const float4 kk = r[2];
+              const TsPix e = eval_edges(r[0], r[1], kk, g.px, g.py);
+              const float4 q4 = r[3];  // o_F, colour of vertex 0
+              const float sig = (AUX && a.face_sigma) ? nb[q * 32 + j].w : a.sigma;
+              // (the tests in one condition: where the window is not positive, alpha is not used)
+              const float al = fminf(q4.x * ts_window(e.m, sig), a.alpha_max);
+              const float Tn = T * (1.f - al);
+              if (e.m > 0.f && al >= a.alpha_min) {
+                if (Tn < a.T_min) {
+                  done = true;
+                  bits = 0u;
+                } else {
+                  const float invD = kk.w;
+                  const float l0 = e.cr1 * invD, l1 = e.cr2 * invD, l2 = e.cr0 * invD;
+                  const float w = al * T;
+                  const float4 q5 = r[4], q6 = r[5];  // colours of vertices 1 and 2, depths z_0, z_1
+                  C0 += w * (l0 * q4.y + l1 * q5.x + l2 * q5.w);
+                  C1 += w * (l0 * q4.z + l1 * q5.y + l2 * q6.x);
+                  C2 += w * (l0 * q4.w + l1 * q5.z + l2 * q6.y);
+                  D += w * (l0 * q6.z + l1 * q6.w + l2 * r[6].x);
+                  if (AUX && a.normals) {
+                    const float4 nn = nb[q * 32 + j];
+                    N0 += w * nn.x;
+                    N1 += w * nn.y;
+                    N2 += w * nn.z;
                   }
+                  T = Tn;
+                  nl = st * S + q * 32 + j + 1;
+                  blended |= 1u << j;
                 }
               }
             }
