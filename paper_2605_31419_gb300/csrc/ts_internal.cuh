@@ -92,6 +92,7 @@ struct TsPlanImpl {
   ts_raster_params prm;
   int64_t n_tiles, n_pix;
   int64_t n_tile_scan_blocks, n_pose_blocks, n_loss_blocks, n_pho_blocks;
+  int64_t loss_per;         // pixels per thread of the loss kernels
   int64_t bin_faces;        // faces per block of the shared-memory tile counts
   int64_t bin_blocks;       // face blocks per view of the shared-memory tile counts (0: global counts)
   int64_t max_view_tiles;   // the most tiles of one view
@@ -136,7 +137,7 @@ struct TsWs {
   float* equi;  // per block of 256 faces: partial sums of the equilateral regulariser
   float4* aux;  // per (view, face): camera-space unit normal (TS_FLAG_NORMALS) and the face's sigma
                // (TS_FLAG_FACE_SIGMA) in .w; null without either flag
-  float* nloss;  // per (view, 2048-pixel block): partial sums of the normal loss
+  float* nloss;  // per (view, block of pixels): partial sums of the normal loss
   uint32_t* cov;  // per (view, face): pixels blended by the forward (TS_FLAG_STATS), else null
   uint32_t* lmask;  // per sorted pair and warp of its tile: the lanes (pixels) that blended the face in the forward
   unsigned long long* ctr;  // [TS_N_CTR][TS_CTR_SLOTS] counters, TS_CTR_STRIDE words apart
