@@ -44,7 +44,7 @@
 // unrolled steps a batch.  The reductions themselves cost nothing measurable; the instructions do.  (A loop
 // over the faces' runs, one word per lane: the backward of 64 tracking views 1034 -> 918 us; testing every
 // row's sums for zero and the slot in 64 bits: fused step 1321 -> 1244 us for the 12-view window, backward
-// of 6 mapping views 172 -> 164.)  A list of one stage is staged whole while the pixels' inputs load.
+// of 6 mapping views 172 -> 164.)
 //
 // Launch forms: one CTA per tile, or persistent CTAs (as many as fit on the GPU) that take tiles
 // from a device counter.  The fused L1 step (ts_render_step_l1) runs a tile's forward, its loss
@@ -476,9 +476,6 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
   const int len = (int)(rg.y - rg.x);
   const float4* vbase = a.frec + (size_t)g.view * (size_t)a.M * 8;
   const float4* nbase = AUX ? a.aux + (size_t)g.view * (size_t)a.M : nullptr;
-  // a list of one stage is staged while the pixels' inputs load, without waiting for their last positions
-  const bool whole = !FUSED && len <= a.S;
-  if (whole && len > 0) issue_stage<AUX>(a, smrec, 0, 0, rg.x, len, vbase, nbase, TW * TH);
   float T = 0.f, Sacc = 0.f, gC0 = 0.f, gC1 = 0.f, gC2 = 0.f, gD = 0.f, gA = 0.f;
   float gN0 = 0.f, gN1 = 0.f, gN2 = 0.f;
   int nl = 0;
@@ -514,8 +511,6 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
   int nmax;
   if (FUSED) {
     nmax = pin->nmax;  // the tile's largest last position, reduced with the loss sums
-  } else if (whole) {
-    nmax = len;  // the forward wrote the masks of the whole stage
   } else {
     if (threadIdx.x == 0) sm.nmax = 0;
     __syncthreads();
@@ -533,7 +528,7 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
   if (n > 0) {
     const int S = a.S;
     const int nst = (n + S - 1) / S;
-    if (!FUSED && !whole) issue_stage<AUX>(a, smrec, (nst - 1) & 1, nst - 1, rg.x, n, vbase, nbase, TW * TH);
+    if (!FUSED) issue_stage<AUX>(a, smrec, (nst - 1) & 1, nst - 1, rg.x, n, vbase, nbase, TW * TH);
     constexpr int EW = Ring<AUX>::EW;
     unsigned char* wbase = reinterpret_cast<unsigned char*>(smrec + (size_t)2 * S * (AUX ? SG + 1 : SG)) +
                            (size_t)warp * Ring<AUX>::BYTES_PER_WARP;
