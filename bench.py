@@ -390,7 +390,7 @@ def bench_pho_loss(ts, torch, rast, tgt_c, tgt_d, flush, stream, pixels, alu_pea
     ach = FLOPS_PHO * 3 * pixels / (t / 1e3) / 1e12
     return {"workload": WORKLOAD.split(",")[0] + f", {rast.V} rendered views vs noise targets", "ms": t,
             "mpix_s": pixels / (t / 1e3) / 1e6,
-            "roofline": {"kernel": "k_pho_tile", "bound": "alu", "achieved": ach, "peak": alu_peak,
+            "roofline": {"kernel": "k_pho_strip", "bound": "alu", "achieved": ach, "peak": alu_peak,
                          "unit": "TFLOP/s", "frac": ach / alu_peak, "traffic": None,
                          "peak_source": f"derived: {n_sm} SMs x 128 FP32 lanes x 2 x {sm_max:.0f} MHz",
                          "work": f"{3 * pixels} pixel-channels x {FLOPS_PHO:.0f} flops"}}
