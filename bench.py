@@ -808,7 +808,7 @@ def main():
         # warp sort also writing the ranges), then either forward, loss (2) and raster backward, or
         # the fused step and its loss reduction; the chain-rule pass (one kernel from 8 views on,
         # two below), pose reduction
-        launches = 2 + 7 + (1 + 2 + 1 if args.separate else 2) + (1 if sc.n_views >= 8 else 2) + 1
+        launches = 2 + 6 + (1 + 2 + 1 if args.separate else 2) + 1 + 1
         line = {
             "metric": "Mpix/s fwd+bwd raster", "value": value, "unit": "Mpix/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": t_step * 1e3, "higher_is_better": True,
