@@ -409,10 +409,11 @@ __device__ __forceinline__ void fwd_tile(const RenderArgs& a, long long tile, fl
       const int alive = __syncthreads_count(!done);
       if (a.cov) {
         for (int j = threadIdx.x; j < cnt; j += TW * TH) {
-          if (fm.cv[b][j]) {  // face m of the record's slot m * V + view
-            const uint32_t slot = __float_as_uint(rb[j * SG + 6].w);
-            const long long m = (long long)(slot / (uint32_t)a.V);
-            if (m < a.M) atomicAdd(a.cov + (long long)g.view * a.M + m, fm.cv[b][j]);
+          // the face from the list: other warps may already be copying the stage after next over this
+          // stage's records, which nothing reads past the barrier
+          if (fm.cv[b][j]) {
+            const uint32_t id = list_id(a, rg.x + (uint32_t)(st * S + j));
+            atomicAdd(a.cov + (long long)g.view * a.M + id, fm.cv[b][j]);
             fm.cv[b][j] = 0u;  // for the stage after next, a barrier away
           }
         }
