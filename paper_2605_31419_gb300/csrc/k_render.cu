@@ -536,6 +536,7 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
     float* ring = reinterpret_cast<float*>(wbase);
     float2* pst = reinterpret_cast<float2*>(wbase + Ring<AUX>::WORDS * 4);  // per pixel lane: (T, S)
     pst[lane] = make_float2(T, Sacc);
+    __syncwarp();  // read by other lanes; a stage that is still staged has no barrier before its first batch
     float* row_here = ring + lane * EW + (lane >> 3) * 8;                      // this lane's entry's row
     const float* row_sum = ring + (lane >> 3) * (8 * EW + 8);                  // its quarter warp's first row
     const int fa = lane & 7;                                                   // the factor it sums

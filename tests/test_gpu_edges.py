@@ -3,7 +3,7 @@
 import numpy as np
 import pytest
 
-from harness import params_pair
+from harness import pack_targets, params_pair
 from ts_synth.scenes import Scene, random_triangles_scene
 
 pytestmark = pytest.mark.gpu
@@ -45,3 +45,32 @@ def test_coverage_of_lists_of_many_stages(fused, persistent):
             assert np.array_equal(cov, got.setdefault("cov", cov)), S
         longest = r.debug("ranges").cpu().numpy().view(np.uint32).reshape(-1, 2)
         assert 128 < int((longest[:, 1] - longest[:, 0]).max()) <= 256
+
+
+@pytest.mark.parametrize("persistent", [False, True])
+def test_fused_step_of_short_lists(persistent):
+    """Lists of one stage stay staged from the forward to the backward of the fused step, whose first batch
+    then reads other lanes' pixel state with no barrier of the staging between: the gradients are those of
+    the separate calls, run after run."""
+    import torch
+    import paper_2605_31419_gb300 as ts
+    sc = random_triangles_scene(seed=15, n_faces=400, W=96, H=64, f=70.0, side_lo=0.1, side_hi=0.6)
+    p, _ = params_pair(flags=ts.TS_FLAG_PERSISTENT if persistent else 0)
+    m, poses = ts.Map.from_numpy(sc.pos, sc.col, sc.opa), ts.poses_tensor(sc.poses)
+    tc, td = (torch.as_tensor(np.asarray(x), dtype=torch.float32, device="cuda") for x in pack_targets(sc))
+    r = ts.Rasterizer(sc.cams, sc.n_faces, p, pair_capacity=100_000)
+    r.forward(m, poses)
+    _, dC, dD = r.l1_loss(tc, td)
+    want = m.zeros_like()
+    r.backward(dC, dD, None, want)
+    lists = r.debug("ranges").cpu().numpy().view(np.uint32).reshape(-1, 2)
+    assert 32 < int((lists[:, 1] - lists[:, 0]).max()) <= 64
+    for _ in range(10):
+        r.project(m, poses)
+        r.bin()
+        g = m.zeros_like()
+        r.step_l1(tc, td, 0.05, g)
+        for k in ("pos", "col", "opa"):
+            a, b = getattr(g, k), getattr(want, k)
+            # the faces' sums are the same terms in another order (atomics): some 300 roundings of 2^-24
+            assert float((a - b).abs().max()) <= 2e-5 * float(b.abs().max()), k
