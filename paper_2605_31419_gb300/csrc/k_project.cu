@@ -276,6 +276,7 @@ __global__ void __launch_bounds__(PJ_T, 6) k_project(ProjArgs a, int views_per_b
     }
     head = (head + n) & (PJ_Q - 1);
     nq -= n;
+    __syncwarp();  // every lane has read its places before the next faces are pushed into them
   };
   // this lane's copies of the vertices of face m into places b; not a face of the map, or an index outside it:
   // not a number, which every view culls

@@ -74,3 +74,39 @@ def test_fused_step_of_short_lists(persistent):
             a, b = getattr(g, k), getattr(want, k)
             # the faces' sums are the same terms in another order (atomics): some 300 roundings of 2^-24
             assert float((a - b).abs().max()) <= 2e-5 * float(b.abs().max()), k
+
+
+def _random_soup(rng, n_faces, n_views, W, H, f):
+    """n_faces small triangles on all sides of n_views cameras near the origin, a quarter of them in view."""
+    centre = rng.normal(size=(n_faces, 3))
+    centre *= rng.uniform(0.5, 4.0, (n_faces, 1)) / np.linalg.norm(centre, axis=1, keepdims=True)
+    pos = centre[:, None] + rng.uniform(-0.06, 0.06, (n_faces, 3, 3))
+    poses = np.tile(np.array([1, 0, 0, 0, 1, 0, 0, 0, 1, 0, 0, 0.0]), (n_views, 1))
+    poses[:, 9:] = rng.uniform(-0.3, 0.3, (n_views, 3))
+    return Scene(pos.reshape(-1, 3).astype(np.float32), rng.random((3 * n_faces, 3), dtype=np.float32),
+                 rng.uniform(0.5, 1.0, 3 * n_faces).astype(np.float32), None,
+                 np.array([[f, f, W / 2, H / 2, W, H]] * n_views), poses.astype(np.float32))
+
+
+@pytest.mark.parametrize("n_views,n_faces", [(9, 70_001), (2, 1_900_033), (1, 2_300_017)])
+def test_projection_queue_of_large_maps(oracle, n_views, n_faces):
+    """Faces that can be seen are queued over views and, on maps of millions of faces, over several groups of
+    32 faces of a warp: every (view, face)'s tile box, tile count and depth key bit for bit, ragged ends
+    included, and records that hold the projected vertices."""
+    import paper_2605_31419_gb300 as ts
+    from oracle.oracle import SceneArrays
+    sc = _random_soup(np.random.default_rng(n_views), n_faces, n_views, 64, 48, 30.0)
+    p, po = params_pair()
+    r = ts.Rasterizer(sc.cams, n_faces, p)
+    r.project(ts.Map.from_numpy(sc.pos, sc.col, sc.opa), ts.poses_tensor(sc.poses))
+    want = oracle.project(SceneArrays.of(sc), po)
+    count = r.debug("count").cpu().numpy().view(np.uint32)
+    assert np.array_equal(count, want["count"])
+    seen = np.flatnonzero(want["count"])
+    assert len(seen) > 0.05 * n_views * n_faces
+    assert np.array_equal(r.debug("rect").cpu().numpy().view(np.int16).reshape(-1, 4)[seen], want["rect"][seen])
+    assert np.array_equal(r.debug("zbits").cpu().numpy().view(np.uint32)[seen], want["zbits"][seen])
+    rec = r.debug("records").cpu().numpy().reshape(-1, 32)
+    uvz = want["uvz"].reshape(-1, 9)[seen]
+    assert np.array_equal(rec[seen][:, [0, 1, 2, 3, 4, 5, 26, 27, 28]], uvz.astype(np.float32))
+    assert r.counters()["n_visible"] == len(seen)
