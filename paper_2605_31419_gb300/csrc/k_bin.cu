@@ -60,27 +60,42 @@ __device__ __forceinline__ uint32_t block_excl_scan(uint32_t x, uint32_t* sm, ui
   return r;
 }
 
+// What a group's 64-bit pair total leaves out of its 32-bit sum, for the total that k_scan_bsums forms: the
+// places past 2^32 wrap, but the pair count and with it the capacity check see every pair.
+__device__ __forceinline__ void keep_wraps(unsigned long long total, unsigned int* wraps) {
+  const unsigned int w = (unsigned int)(total >> 32);
+  if (w) atomicAdd(wraps, w);
+}
+
 __global__ void __launch_bounds__(SCAN_T) k_scan_reduce(const uint32_t* __restrict__ in, Len len,
-                                                        uint32_t* __restrict__ bsums) {
-  __shared__ uint32_t sm[33];
+                                                        uint32_t* __restrict__ bsums, unsigned int* wraps) {
+  __shared__ unsigned long long wsum[SCAN_T / 32];
   const long long n = len.get();
   const long long base = (long long)blockIdx.x * TS_SCAN_ITEMS;
   if (base >= n) return;
-  uint32_t s = 0;
+  unsigned long long s = 0;
 #pragma unroll
   for (int k = 0; k < SCAN_PER; ++k) {
     const long long i = base + (long long)k * SCAN_T + threadIdx.x;
     if (i < n) s += in[i];
   }
-  uint32_t tot;
-  block_excl_scan(s, sm, &tot);
-  if (threadIdx.x == 0) bsums[blockIdx.x] = tot;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if ((threadIdx.x & 31) == 0) wsum[threadIdx.x >> 5] = s;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long tot = 0;
+    for (int w = 0; w < SCAN_T / 32; ++w) tot += wsum[w];
+    bsums[blockIdx.x] = (uint32_t)tot;
+    keep_wraps(tot, wraps);
+  }
 }
 
-// Exclusive scan of the block sums in place (one block); writes the grand total, and zeroes
-// *zero_out (the sort's count of long lists) for the launches that follow.
-__global__ void __launch_bounds__(SCAN_T) k_scan_bsums(uint32_t* bsums, long long nb,
-                                                       unsigned long long* total_out, unsigned int* err, long long cap, unsigned int* zero_out) {
+// Exclusive scan of the block sums in place (one block); writes the grand total, takes up *wraps (and zeroes
+// it), and zeroes *zero_out (the sort's count of long lists) for the launches that follow.
+__global__ void __launch_bounds__(SCAN_T) k_scan_bsums(uint32_t* bsums, long long nb, unsigned long long* total_out,
+                                                       unsigned int* err, long long cap, unsigned int* wraps,
+                                                       unsigned int* zero_out) {
   __shared__ uint32_t sm[33];
   __shared__ unsigned long long wsum[SCAN_T / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -103,13 +118,12 @@ __global__ void __launch_bounds__(SCAN_T) k_scan_bsums(uint32_t* bsums, long lon
   }
   __syncthreads();
   if (threadIdx.x == 0) {
-    unsigned long long tot64 = 0;
+    unsigned long long tot64 = (unsigned long long)*wraps << 32;
     for (int w = 0; w < SCAN_T / 32; ++w) tot64 += wsum[w];
-    if (total_out) {
-      *total_out = tot64;
-      if ((long long)tot64 > cap) atomicOr(err, TS_ERRBIT_CAPACITY);
-    }
-    if (zero_out) *zero_out = 0u;
+    *wraps = 0u;
+    *total_out = tot64;
+    if ((long long)tot64 > cap) atomicOr(err, TS_ERRBIT_CAPACITY);
+    *zero_out = 0u;
   }
 }
 
@@ -328,7 +342,7 @@ __global__ void __launch_bounds__(BIN_T, 3) k_bin_counts(MatArgs a) {
 constexpr int COL_WARPS = 8, COL_ROWS = 8;  // warps per block, most rows per warp at a time
 __global__ void __launch_bounds__(32 * COL_WARPS) k_bin_columns(uint32_t* __restrict__ mat, long long n_tiles, int B,
                                                                  uint32_t* __restrict__ tpre,
-                                                                 uint32_t* __restrict__ gsum) {
+                                                                 uint32_t* __restrict__ gsum, unsigned int* wraps) {
   static_assert(TS_BIN_GROUP == 32, "a lane per tile of the group");
   __shared__ uint32_t part[COL_WARPS][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -364,7 +378,13 @@ __global__ void __launch_bounds__(32 * COL_WARPS) k_bin_columns(uint32_t* __rest
   if (warp == 0) {
     const uint32_t incl = warp_incl_scan(carry);
     if (in) tpre[t] = incl - carry;
-    if (lane == 31) gsum[blockIdx.x] = incl;
+    // the group's total in 64 bits (a tile's is below 2^31): 32 tiles of 2^27 faces each pass 2^32
+    const unsigned long long tot = ((unsigned long long)__reduce_add_sync(0xffffffffu, carry >> 16) << 16) +
+                                   __reduce_add_sync(0xffffffffu, carry & 0xffffu);
+    if (lane == 31) {
+      gsum[blockIdx.x] = incl;
+      keep_wraps(tot, wraps);
+    }
   }
 }
 
@@ -506,11 +526,11 @@ __global__ void __launch_bounds__(32 * SORT_WARPS_PER_BLOCK) k_tile_sort(SortOut
     rg = o.ranges[t];
   }
   const long long start = min((long long)rg.x, o.cap);
-  const long long end = min((long long)rg.y, o.cap);
+  const long long end = max(start, min((long long)rg.y, o.cap));  // (an end past 2^32 has wrapped to below its start)
   // the tile's range for the passes that follow; past the capacity (its bit is latched) the lists
   // are cut, and the ranges with them, so that no later pass reads outside the pair list
-  if (lane == 0 && (o.tpre || (long long)rg.y > o.cap)) o.ranges[t] = make_uint2((uint32_t)start, (uint32_t)end);
-  const int n = (int)max(0LL, end - start);
+  if (lane == 0 && (o.tpre || start != rg.x || end != rg.y)) o.ranges[t] = make_uint2((uint32_t)start, (uint32_t)end);
+  const int n = (int)(end - start);
   if (n == 0) return;
   if (n <= 32) {
     unsigned long long x = lane < n ? o.seg[start + lane] : ~0ull;
@@ -709,8 +729,10 @@ cudaError_t ts_launch_bin(const TsPlanImpl* p, const TsWs& w, cudaStream_t s) {
     const dim3 grid((unsigned)p->bin_blocks, (unsigned)p->V);
     k_bin_counts<<<grid, BIN_T, smem, s>>>(ma);
     const unsigned ng = (unsigned)((p->n_tiles + TS_BIN_GROUP - 1) / TS_BIN_GROUP);
-    k_bin_columns<<<ng, 32 * COL_WARPS, 0, s>>>(w.tmat, p->n_tiles, (int)p->bin_blocks, w.tcnt, w.bsums);
-    k_scan_bsums<<<1, SCAN_T, 0, s>>>(w.bsums, ng, &w.hdr->n_pairs, &w.hdr->error_bits, p->cap, &w.hdr->n_large);
+    k_bin_columns<<<ng, 32 * COL_WARPS, 0, s>>>(w.tmat, p->n_tiles, (int)p->bin_blocks, w.tcnt, w.bsums,
+                                             &w.hdr->pair_wraps);
+    k_scan_bsums<<<1, SCAN_T, 0, s>>>(w.bsums, ng, &w.hdr->n_pairs, &w.hdr->error_bits, p->cap,
+                                       &w.hdr->pair_wraps, &w.hdr->n_large);
     k_bin_place<<<grid, BIN_T, smem, s>>>(ma);
   } else {
     // 1-3 with global counts: counts, their scan, starts, places
@@ -722,8 +744,9 @@ cudaError_t ts_launch_bin(const TsPlanImpl* p, const TsWs& w, cudaStream_t s) {
     k_tile_count<<<nf, 256, 0, s>>>(ta);
     Len lt{p->n_tiles};
     const unsigned nb = (unsigned)((p->n_tiles + TS_SCAN_ITEMS - 1) / TS_SCAN_ITEMS);
-    k_scan_reduce<<<nb, SCAN_T, 0, s>>>(w.tcnt, lt, w.bsums);
-    k_scan_bsums<<<1, SCAN_T, 0, s>>>(w.bsums, nb, &w.hdr->n_pairs, &w.hdr->error_bits, p->cap, &w.hdr->n_large);
+    k_scan_reduce<<<nb, SCAN_T, 0, s>>>(w.tcnt, lt, w.bsums, &w.hdr->pair_wraps);
+    k_scan_bsums<<<1, SCAN_T, 0, s>>>(w.bsums, nb, &w.hdr->n_pairs, &w.hdr->error_bits, p->cap,
+                                       &w.hdr->pair_wraps, &w.hdr->n_large);
     k_tile_starts<<<nb, SCAN_T, 0, s>>>(ta, w.bsums);
     k_tile_scatter<<<nf, 256, 0, s>>>(ta);
   }

@@ -81,7 +81,8 @@ struct TsDevHeader {
   unsigned int tile_counter;  // work counter of the persistent raster launches
   unsigned int n_large;       // tiles listed for the CTA-wide pair sort
   unsigned int pose_blocks;   // per-view pose partials the last backward wrote
-  unsigned int pad[11];
+  unsigned int pair_wraps;    // binning: 2^32s of pairs that the 32-bit sums of groups of tiles dropped
+  unsigned int pad[10];
 };
 
 struct TsPlanImpl {

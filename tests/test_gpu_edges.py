@@ -110,3 +110,30 @@ def test_projection_queue_of_large_maps(oracle, n_views, n_faces):
     uvz = want["uvz"].reshape(-1, 9)[seen]
     assert np.array_equal(rec[seen][:, [0, 1, 2, 3, 4, 5, 26, 27, 28]], uvz.astype(np.float32))
     assert r.counters()["n_visible"] == len(seen)
+
+
+@pytest.mark.parametrize("n_faces,size,tri", [
+    # 2^27 faces over the 32 tiles of one group of the count matrix
+    (1 << 27, (256, 8), [[-10.0, -10.0], [600.0, -10.0], [-10.0, 40.0]]),
+    # 2^20 faces over the first 4096 tiles of a view that takes the global counts
+    (1 << 20, (4096, 2560), [[0.2, 0.2], [4095.8, 0.2], [0.2, 63.8]]),
+])
+def test_pair_total_beyond_32_bits(n_faces, size, tri):
+    """2^32 pairs in one group of tiles: the count is exact and latches the capacity error, also when the
+    binning runs again, and the ranges stay inside the pair list."""
+    import torch
+    import paper_2605_31419_gb300 as ts
+    W, H = size
+    pos = np.array([[(u - W / 2) / 100.0, (v - H / 2) / 100.0, 1.0] for u, v in tri], np.float32).T
+    m = ts.Map(torch.as_tensor(pos, device="cuda").contiguous(), torch.full((3, 3), 0.5, device="cuda"),
+               torch.full((3,), 0.5, device="cuda"),
+               torch.arange(3, dtype=torch.int32, device="cuda").repeat(n_faces, 1).contiguous())
+    p, _ = params_pair(tile_w=8, tile_h=8, flags=ts.TS_FLAG_FORWARD_ONLY)
+    r = ts.Rasterizer(np.array([[100.0, 100.0, W / 2, H / 2, W, H]]), n_faces, p, pair_capacity=1024)
+    r.project(m, ts.poses_tensor(np.array([[1, 0, 0, 0, 1, 0, 0, 0, 1, 0, 0, 0]], np.float32)))
+    for _ in range(2):
+        r.bin()
+        c = r.counters(raise_on_error=False)
+        assert c["n_pairs"] == 1 << 32 and c["error_bits"] == 1
+        lists = r.debug("ranges").cpu().numpy().view(np.uint32).reshape(-1, 2).astype(np.int64)
+        assert (lists[:, 0] <= lists[:, 1]).all() and (lists[:, 1] <= 1024).all()
