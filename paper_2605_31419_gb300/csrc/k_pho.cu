@@ -133,12 +133,6 @@ __device__ __forceinline__ void stage_block(float* xy, const float* xc, const fl
 // The weight of distance t along a window (both sides alike), or -1 outside it.
 __host__ __device__ constexpr int tap(int t) { return t < 0 || t >= NT ? -1 : (t <= RAD ? t : NT - 1 - t); }
 
-// Reciprocal of a normal number: the hardware approximation and one Newton-Raphson step.
-__device__ __forceinline__ float reciprocal(float x) {
-  const float r = ts_rcp_approx(x);
-  return fmaf(r, fmaf(-x, r, 1.f), r);
-}
-
 __device__ __forceinline__ float block_sum(float v, float* red) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -255,7 +249,7 @@ __global__ void __launch_bounds__(PT, 2)
           const float A1 = 2.f * mx * my + C1, A2 = 2.f * (exy - mx * my) + C2;
           const float dm = mx - my;
           const float B1 = fmaf(dm, dm, A1), B2 = A2 + fmaf(-dm, dm, edd);
-          const float iB = reciprocal(B1 * B2);
+          const float iB = 1.f / (B1 * B2);  // (0 where the product overflows: such a pixel's terms vanish)
           const float ssim = A1 * A2 * iB;
           // partials w.r.t. mu_x, e_xx and e_xy: zero outside the image
           float m0 = 2.f * (my * (A2 - A1) - mx * ssim * (B2 - B1)) * iB;

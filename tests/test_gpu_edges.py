@@ -137,3 +137,27 @@ def test_pair_total_beyond_32_bits(n_faces, size, tri):
         assert c["n_pairs"] == 1 << 32 and c["error_bits"] == 1
         lists = r.debug("ranges").cpu().numpy().view(np.uint32).reshape(-1, 2).astype(np.int64)
         assert (lists[:, 0] <= lists[:, 1]).all() and (lists[:, 1] <= 1024).all()
+
+
+def test_pho_loss_where_ssim_products_reach_the_range():
+    """SSIM divides by a product of two sums of squares.  Where that product overflows (values of 2e10) the
+    terms vanish and L1 is left; where its reciprocal is below the normal range (4e9) equal images still have
+    SSIM = 1.  Both finite."""
+    import torch
+    import paper_2605_31419_gb300 as ts
+    W, H, lam = 96, 80, 0.2
+    r = ts.Rasterizer(np.array([[50.0, 50.0, W / 2, H / 2, W, H]]), 0)
+    rng = np.random.default_rng(4)
+    x = torch.as_tensor(rng.uniform(-2e10, 2e10, 3 * W * H), dtype=torch.float32, device="cuda")
+    td = torch.zeros_like(r.depth)
+    r.color.copy_(x)
+    r.depth.zero_()
+    loss, dC, _ = r.pho_loss(torch.zeros_like(x), td, lam)
+    want = (1 - lam) * float(x.double().abs().mean()) + lam
+    assert abs(float(loss[0]) - want) <= 1e-5 * want
+    # SSIM's own gradient is below 1e-9 of the L1 one's
+    assert torch.allclose(dC, (1 - lam) / (3 * W * H) * torch.sign(x), rtol=1e-6, atol=0)
+    x = torch.as_tensor(4.16e9 * rng.uniform(0.5, 1.5, 3 * W * H), dtype=torch.float32, device="cuda")
+    r.color.copy_(x)
+    loss, dC, _ = r.pho_loss(x, td, lam)
+    assert abs(float(loss[0])) < 1e-3 and bool(torch.isfinite(dC).all())
