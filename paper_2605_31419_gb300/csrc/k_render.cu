@@ -98,15 +98,35 @@ struct RenderArgs {
 constexpr unsigned FULL = 0xffffffffu;
 
 // Register budgets of the raster kernels per thread, expressed as the minimum number of resident CTAs in the
-// launch bounds.  More
-// resident CTAs hide more latency until spills cost more: 64 tracking views take the forward 512 us at 40
-// and 538 at 48, the backward 686 at 48, 669 at 56 and 768 at 64; with the side array, 6 mapping views take
-// the forward 112 at 48 and 116 at 56, the backward 201 / 192 / 179 / 166 at 48 / 56 / 64 / 72; the fused step
-// of the 12-view window takes 1247 / 1216 / 1260 at 48 / 56 / 64.
-constexpr int REGS_FWD = 40, REGS_BWD = 56, REGS_STEP = 56, REGS_FWD_AUX = 48, REGS_BWD_AUX = 72;
+// launch bounds.  More resident CTAs hide more latency until spills cost more.  16 x 8 tiles: 64 tracking views
+// take the forward 512 us at 40 and 538 at 48, the backward 686 at 48, 669 at 56 and 768 at 64; with the side
+// array, 6 mapping views take the forward 112 at 48 and 116 at 56, the backward 201 / 192 / 179 / 166 at 48 / 56 /
+// 64 / 72; the fused step of the 12-view window takes 1247 / 1216 / 1260 at 48 / 56 / 64.  The forward of 8 x 8
+// tiles, of which shared memory holds 14 at 64 faces a stage, spills at 40: 187 / 153 / 152 / 148 us at 40 / 48 /
+// 56 / 72 for 16 views of 100k faces.
+// With the side array the backward of CTAs of 256 threads takes 266 us at 72 (three CTAs) and 227 at 64 (four).
+constexpr int REGS_FWD = 40, REGS_FWD_64 = 56, REGS_BWD = 56, REGS_STEP = 56, REGS_FWD_AUX = 48, REGS_BWD_AUX = 72;
+constexpr int REGS_BWD_AUX_256 = 64;
+// A quarter of a multiprocessor (16,384 registers) holds whole warps, so `regs` registers (a multiple of 8)
+// leave 4 floor(16384 / (32 regs)) warps; in CTAs of `threads` the nearest number, halves down.  (Dividing 65,536 by
+// threads x regs gave 8 x 8 tiles 32 registers for 40, and left CTAs of 512 threads one to a multiprocessor, with
+// 108 registers, for 72: the side-array backward of 16 x 32 tiles took 421 us where it takes 271, 16 views of 100k.)
 constexpr int raster_min_blocks(int threads, int regs) {
-  return 65536 / (threads * regs) > 0 ? 65536 / (threads * regs) : 1;
+  const int resident = 4 * (16384 / (32 * regs)) * 32;
+  return (2 * resident + threads - 1) / (2 * threads) > 0 ? (2 * resident + threads - 1) / (2 * threads) : 1;
 }
+constexpr int fwd_min_blocks(int threads, bool aux) {
+  return raster_min_blocks(threads, aux ? REGS_FWD_AUX : (threads == 64 ? REGS_FWD_64 : REGS_FWD));
+}
+constexpr int bwd_min_blocks(int threads, bool aux) {
+  return raster_min_blocks(threads, !aux ? REGS_BWD : (threads >= 256 ? REGS_BWD_AUX_256 : REGS_BWD_AUX));
+}
+// every tile shape gets its budget: 64 threads exactly, and 512 are not left with one CTA
+static_assert(raster_min_blocks(64, 40) == 24 && raster_min_blocks(64, 48) == 20 && raster_min_blocks(128, 72) == 7 &&
+                  raster_min_blocks(512, 72) == 2 && raster_min_blocks(512, 48) == 2 && raster_min_blocks(512, 40) == 3 &&
+                  fwd_min_blocks(64, false) == 18 && fwd_min_blocks(128, false) == 12 &&
+                  bwd_min_blocks(128, true) == 7 && bwd_min_blocks(256, true) == 4 && bwd_min_blocks(512, true) == 2,
+              "resident CTAs of a register budget");
 
 // Shared state of a render CTA.
 struct RenderSmem {
@@ -823,7 +843,7 @@ __device__ __forceinline__ long long next_tile(const RenderArgs& a, RenderSmem& 
 }
 
 template <int TW, int TH, bool PERSIST, bool AUX>
-__global__ void __launch_bounds__(TW * TH, raster_min_blocks(TW * TH, AUX ? REGS_FWD_AUX : REGS_FWD)) k_render_fwd(RenderArgs a) {
+__global__ void __launch_bounds__(TW * TH, fwd_min_blocks(TW * TH, AUX)) k_render_fwd(RenderArgs a) {
   extern __shared__ __align__(128) float4 smrec[];
   __shared__ RenderSmem sm;
   __shared__ FwdMasks fm;
@@ -836,7 +856,7 @@ __global__ void __launch_bounds__(TW * TH, raster_min_blocks(TW * TH, AUX ? REGS
 }
 
 template <int TW, int TH, bool PERSIST, bool AUX>
-__global__ void __launch_bounds__(TW * TH, raster_min_blocks(TW * TH, AUX ? REGS_BWD_AUX : REGS_BWD)) k_render_bwd(RenderArgs a) {
+__global__ void __launch_bounds__(TW * TH, bwd_min_blocks(TW * TH, AUX)) k_render_bwd(RenderArgs a) {
   extern __shared__ __align__(128) float4 smrec[];
   __shared__ RenderSmem sm;
   if constexpr (!PERSIST) {

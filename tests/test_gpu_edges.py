@@ -161,3 +161,31 @@ def test_pho_loss_where_ssim_products_reach_the_range():
     r.color.copy_(x)
     loss, dC, _ = r.pho_loss(x, td, lam)
     assert abs(float(loss[0])) < 1e-3 and bool(torch.isfinite(dC).all())
+
+
+@pytest.mark.parametrize("persistent", [False, True])
+@pytest.mark.parametrize("tile", [(16, 16), (8, 8), (32, 8), (16, 32), (32, 16)], ids=lambda t: f"{t[0]}x{t[1]}")
+def test_side_array_at_every_tile_shape(tile, persistent):
+    """Images with normals and the gradients of all of them at every tile shape (each compiled for its own
+    register budget) against those at 16 x 8: images bit for bit, gradients to the order of the faces' sums."""
+    import torch
+    import paper_2605_31419_gb300 as ts
+    sc = _two_views(random_triangles_scene(seed=23, n_faces=600, W=101, H=67, f=60.0, side_lo=0.2, side_hi=0.8))
+    m, poses = ts.Map.from_numpy(sc.pos, sc.col, sc.opa), ts.poses_tensor(sc.poses)
+    out = []
+    for tw, th in ((16, 8), tile):
+        flags = ts.TS_FLAG_NORMALS | (ts.TS_FLAG_PERSISTENT if persistent else 0)
+        r = ts.Rasterizer(sc.cams, sc.n_faces, ts.ts_default_params(tile_w=tw, tile_h=th, flags=flags), pair_capacity=400_000)
+        images = [t.clone() for t in r.forward(m, poses)] + [r.normal.clone()]
+        gen = torch.Generator(device="cuda").manual_seed(5)
+        dC, dN = (torch.rand(3 * r.n_pix, generator=gen, device="cuda") - 0.5 for _ in range(2))
+        dD, dA = (torch.rand(r.n_pix, generator=gen, device="cuda") - 0.5 for _ in range(2))
+        g = m.zeros_like()
+        r.backward(dC, dD, dA, g, dN=dN)
+        assert r.counters()["error_bits"] == 0
+        out.append((images, [g.pos, g.col, g.opa]))
+    for a, b in zip(*(o[0] for o in out)):
+        assert torch.equal(a, b)
+    for a, b in zip(*(o[1] for o in out)):
+        # some 300 roundings of 2^-24 in another order
+        assert float((a - b).abs().max()) <= 2e-5 * float(a.abs().max())
