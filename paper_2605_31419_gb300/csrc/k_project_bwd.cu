@@ -273,6 +273,9 @@ constexpr int PB_T = 32 * PB_WARPS;
 constexpr int PB_RS = 21;   // floats per entry row (positions 9, colours 9, opacity, sigma; odd: no bank conflicts)
 constexpr int PB_FS = 19;   // floats per staged face (positions 9, colours 9)
 constexpr int PB_PS = 6;    // floats per view's pose sums
+// Faces of a batch up to which lane w sums word w over each face's rows.  3 / 5 / 8: 342 / 329 / 329 us for 64 views of
+// 300k faces (354 without), 59 / 59 / 60 for 6 views, where a batch holds more.
+constexpr int PB_FEW = 5;
 
 // Views whose visibility the lanes of one face look up at a time (64 bits each).
 __host__ __device__ constexpr int pbwd_view_chunk(int faces) { return 64 * (32 / faces); }
@@ -382,36 +385,53 @@ __global__ void __launch_bounds__(PB_T, 4) k_pbwd_map(PBArgs a) {
           }
           __syncwarp();
         }
-        // map words: the lane of each (face, vertex) sums its words over the face's rows, views in order
-#pragma unroll
-        for (int r = 0; r < ROUNDS; ++r) {
-          const int lo = max(e0[r] - b0, 0), hi = min(e1[r] - b0, 32);
-          if (lo < hi) {
-            const int i = r * 32 + lane, k = i % 3;
-            float* w = fsum + i / 3 * PB_RS;
-            float sum[8];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) sum[c] = w[3 * k + c];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) sum[3 + c] = w[9 + 3 * c + k];
-            sum[6] = w[18];
-            sum[7] = w[19];
-            for (int e = lo; e < hi; ++e) {
-              const float* row = rows + e * PB_RS;
-#pragma unroll
-              for (int c = 0; c < 3; ++c) sum[c] += row[3 * k + c];
-#pragma unroll
-              for (int c = 0; c < 3; ++c) sum[3 + c] += row[9 + 3 * c + k];
-              sum[6] += row[18];
-              sum[7] += row[19];
+        // map words, views in order: where the batch holds many faces, the lane of each (face, vertex) sums its
+        // words over the face's rows; where it holds few (faces seen by many views), lane w sums word w over
+        // each face's rows, so that no lane walks all eight words of 32 rows.  The same sums either way.
+        const int fprev = __shfl_up_sync(0xffffffffu, fe, 1);
+        const unsigned firsts = __ballot_sync(0xffffffffu, act && (lane == 0 || fe != fprev));
+        if (__popc(firsts) <= PB_FEW) {
+          for (unsigned rem = firsts; rem; rem &= rem - 1) {
+            const int lo = __ffs(rem) - 1, hi = rem & (rem - 1) ? __ffs(rem & (rem - 1)) - 1 : ne;
+            const int face = __shfl_sync(0xffffffffu, fe, lo);
+            if (lane < PB_RS - 1) {
+              float sum = fsum[face * PB_RS + lane];
+#pragma unroll 4
+              for (int e = lo; e < hi; ++e) sum += rows[e * PB_RS + lane];
+              fsum[face * PB_RS + lane] = sum;
             }
+          }
+        } else {
 #pragma unroll
-            for (int c = 0; c < 3; ++c) w[3 * k + c] = sum[c];
+          for (int r = 0; r < ROUNDS; ++r) {
+            const int lo = max(e0[r] - b0, 0), hi = min(e1[r] - b0, 32);
+            if (lo < hi) {
+              const int i = r * 32 + lane, k = i % 3;
+              float* w = fsum + i / 3 * PB_RS;
+              float sum[8];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) w[9 + 3 * c + k] = sum[3 + c];
-            if (k == 0) {  // (the face's other two lanes drop these sums)
-              w[18] = sum[6];
-              w[19] = sum[7];
+              for (int c = 0; c < 3; ++c) sum[c] = w[3 * k + c];
+#pragma unroll
+              for (int c = 0; c < 3; ++c) sum[3 + c] = w[9 + 3 * c + k];
+              sum[6] = w[18];
+              sum[7] = w[19];
+              for (int e = lo; e < hi; ++e) {
+                const float* row = rows + e * PB_RS;
+#pragma unroll
+                for (int c = 0; c < 3; ++c) sum[c] += row[3 * k + c];
+#pragma unroll
+                for (int c = 0; c < 3; ++c) sum[3 + c] += row[9 + 3 * c + k];
+                sum[6] += row[18];
+                sum[7] += row[19];
+              }
+#pragma unroll
+              for (int c = 0; c < 3; ++c) w[3 * k + c] = sum[c];
+#pragma unroll
+              for (int c = 0; c < 3; ++c) w[9 + 3 * c + k] = sum[3 + c];
+              if (k == 0) {  // (the face's other two lanes drop these sums)
+                w[18] = sum[6];
+                w[19] = sum[7];
+              }
             }
           }
         }

@@ -189,3 +189,85 @@ def test_side_array_at_every_tile_shape(tile, persistent):
     for a, b in zip(*(o[1] for o in out)):
         # some 300 roundings of 2^-24 in another order
         assert float((a - b).abs().max()) <= 2e-5 * float(a.abs().max())
+
+
+def _padded(sc, n_faces, indexed):
+    """The scene's map with faces behind every camera between its first and its second half: n_faces in all,
+    and the places of the scene's own."""
+    M = sc.n_faces
+    keep = np.concatenate([np.arange(M // 2), np.arange(n_faces - (M - M // 2), n_faces)])
+    if indexed:
+        N = len(sc.pos)
+        behind = np.array([[0, 0, -5], [0.1, 0, -5], [0, 0.1, -5]], np.float32)
+        faces = np.tile(np.arange(N, N + 3, dtype=np.int32), (n_faces, 1))
+        faces[keep] = sc.faces
+        sigma = np.full(n_faces, 0.7, np.float32)
+        sigma[keep] = sc.sigma
+        out = Scene(np.concatenate([sc.pos, behind]), np.concatenate([sc.col, sc.col[:3]]),
+                    np.concatenate([sc.opa, sc.opa[:3]]), faces, sc.cams, sc.poses)
+        out.sigma = sigma
+        return out, keep, np.arange(N)
+    rows = (3 * keep[:, None] + np.arange(3)).reshape(-1)
+    pos = np.tile(np.array([[0, 0, -5], [0.1, 0, -5], [0, 0.1, -5]], np.float32), (n_faces, 1))
+    col, opa = np.full((3 * n_faces, 3), 0.5, np.float32), np.full(3 * n_faces, 0.5, np.float32)
+    pos[rows], col[rows], opa[rows] = sc.pos, sc.col, sc.opa
+    return Scene(pos, col, opa, None, sc.cams, sc.poses), keep, rows
+
+
+@pytest.mark.parametrize("n_faces,n_views,indexed", [
+    (19_457, 2, False), (19_500, 68, True), (19_457, 69, False),    # 16 faces a warp up to 68 views
+    (38_913, 1, True), (38_950, 23, False), (38_913, 24, True),     # 32 up to 23
+    (65_601, 1, False), (65_600, 3, True), (140_003, 2, False),     # 65 and more face blocks; 512 faces a warp, pose only
+])
+def test_padded_maps(n_faces, n_views, indexed):
+    """A map of 1000 faces, and the same faces at the two ends of a large map whose other faces nobody sees: the
+    same images and tile lists, and the same gradients with and without map gradients, whatever number of faces
+    a block bins and a warp of the chain rule takes."""
+    import torch
+    import paper_2605_31419_gb300 as ts
+    sc = random_triangles_scene(seed=n_views, n_faces=1000, W=64, H=48, f=50.0, side_lo=0.1, side_hi=0.4, z_lo=1.0, z_hi=3.0)
+    poses = np.repeat(sc.poses[:1], n_views, axis=0).copy()
+    poses[:, 9] = np.linspace(-0.8, 0.8, n_views) if n_views > 1 else 0.0
+    faces = None
+    if indexed:  # every vertex shared by about three faces
+        faces = np.random.default_rng(7).permutation(3000).astype(np.int32).reshape(-1, 3)
+        faces[1:, 0] = faces[:-1, 2]
+        pos = sc.pos.copy()
+        pos[faces[:, 1]] = pos[faces[:, 0]] + np.float32([0.2, 0.03, 0.02])
+        pos[faces[:, 2]] = pos[faces[:, 0]] + np.float32([0.05, 0.25, -0.03])
+        sc.pos[:] = pos
+    sc = Scene(sc.pos, sc.col, sc.opa, faces, np.repeat(sc.cams[:1], n_views, axis=0), poses)
+    sc.sigma = np.random.default_rng(8).uniform(0.5, 1.2, 1000).astype(np.float32) if indexed else None
+    big, keep, rows = _padded(sc, n_faces, indexed)
+    flags = ts.TS_FLAG_MIN_OPACITY | ts.TS_FLAG_FACE_SIGMA if indexed else 0
+    p, _ = params_pair(flags=flags)
+    out = []
+    for s in (sc, big):
+        r = ts.Rasterizer(s.cams, s.n_faces, p, pair_capacity=200 * 1000 * n_views)
+        m = ts.Map.from_numpy(s.pos, s.col, s.opa, s.faces, sigma=getattr(s, "sigma", None))
+        d = {"images": [t.clone() for t in r.forward(m, ts.poses_tensor(s.poses))]}
+        n = r.counters()["n_pairs"]
+        d["ids"], d["ranges"] = r.debug("ids")[:n].cpu().numpy().copy(), r.debug("ranges").cpu().numpy().copy()
+        gen = torch.Generator(device="cuda").manual_seed(5)
+        dC, dD = torch.rand(3 * r.n_pix, generator=gen, device="cuda") - 0.5, torch.rand(r.n_pix, generator=gen, device="cuda") - 0.5
+        g = m.zeros_like()
+        r.backward(dC, dD, None, g)
+        d["dtau"] = r.pose_grad().cpu().numpy().copy()
+        d["grad"] = [t.cpu().numpy() for t in (g.pos, g.col, g.opa)] + ([g.sigma.cpu().numpy()] if indexed else [])
+        r.forward(m, ts.poses_tensor(s.poses))
+        r.backward(dC, dD)
+        d["pose"] = r.pose_grad().cpu().numpy().copy()
+        assert r.counters()["error_bits"] == 0 and n > 0
+        out.append(d)
+    a, b = out
+    assert all(torch.equal(x, y) for x, y in zip(a["images"], b["images"]))
+    assert np.array_equal(keep[a["ids"]], b["ids"]) and np.array_equal(a["ranges"], b["ranges"])
+    for i, (x, y) in enumerate(zip(a["grad"], b["grad"])):
+        at = y[keep] if i == 3 else y[..., rows]
+        assert np.abs(x).max() > 0 and np.abs(x - at).max() <= 2e-5 * np.abs(x).max(), i  # the faces' sums in another order
+        rest = np.ones(y.shape[-1], bool)
+        rest[keep if i == 3 else rows] = False
+        assert not y[..., rest].any(), i
+    # sums over some 3000 vertices of such terms, which cancel in part
+    for x, y in ((a["dtau"], b["dtau"]), (a["pose"], b["pose"]), (a["dtau"], a["pose"])):
+        assert np.abs(x - y).max() <= 1e-4 * np.abs(x).max()
