@@ -277,13 +277,10 @@ constexpr int PB_PS = 6;    // floats per view's pose sums
 // 300k faces (354 without), 59 / 59 / 60 for 6 views, where a batch holds more.
 constexpr int PB_FEW = 5;
 
-// Views whose visibility the lanes of one face look up at a time (64 bits each).
-__host__ __device__ constexpr int pbwd_view_chunk(int faces) { return 64 * (32 / faces); }
 // Shared floats of one warp (a multiple of 4): slot copies, entry rows, staged faces, per-face sums,
 // per-view pose sums, entry list.
 __host__ __device__ constexpr int pbwd_warp_floats(int V, int faces) {
-  const int chunk = V < pbwd_view_chunk(faces) ? V : pbwd_view_chunk(faces);
-  return (32 * TS_GRAD_WORDS + 32 * PB_RS + faces * (PB_FS + PB_RS) + V * PB_PS + (faces * chunk + 1) / 2 + 3) & ~3;
+  return (32 * TS_GRAD_WORDS + 32 * PB_RS + faces * (PB_FS + PB_RS) + V * PB_PS + (faces * V + 1) / 2 + 3) & ~3;
 }
 
 // With map gradients: FPW faces per warp iteration, 32 / FPW lanes looking up each face's views.
@@ -316,127 +313,124 @@ __global__ void __launch_bounds__(PB_T, 4) k_pbwd_map(PBArgs a) {
     }
     ts_cp_async_commit();
     for (int i = lane; i < FPW * PB_RS; i += 32) fsum[i] = 0.f;
-    unsigned seen = 0u;
-    for (int c0 = 0; c0 < a.V; c0 += pbwd_view_chunk(FPW)) {
-      // this lane looks up views [va, vb) of face f
-      const int nvc = min(a.V - c0, pbwd_view_chunk(FPW)), Q = (nvc + LPF - 1) / LPF;
-      const int va = c0 + min((lane % LPF) * Q, nvc), vb = min(va + Q, c0 + nvc);
-      unsigned long long bits = 0ull;
-      {
-        const uint32_t* cp = a.count + (long long)va * a.M + m0 + f;
-        const int nv = m0 + f < a.M ? vb - va : 0;
+    // this lane looks up views [va, vb) of face f: at most 64, a bit each (the launch sees to it)
+    const int Q = (a.V + LPF - 1) / LPF;
+    const int va = min((lane % LPF) * Q, a.V), vb = min(va + Q, a.V);
+    unsigned long long bits = 0ull;
+    {
+      const uint32_t* cp = a.count + (long long)va * a.M + m0 + f;
+      const int nv = m0 + f < a.M ? vb - va : 0;
 #pragma unroll 8
-        for (int i = 0; i < nv; ++i) bits |= (unsigned long long)(cp[(long long)i * a.M] != 0u) << i;
-      }
-      const int mine = __popcll(bits);
-      int incl = mine;
+      for (int i = 0; i < nv; ++i) bits |= (unsigned long long)(cp[(long long)i * a.M] != 0u) << i;
+    }
+    const int mine = __popcll(bits);
+    int incl = mine;
 #pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += t;
-      }
-      const int total = __shfl_sync(0xffffffffu, incl, 31);
-      seen |= __ballot_sync(0xffffffffu, mine > 0);
-      for (int k = incl - mine; bits; bits &= bits - 1) list[k++] = (uint16_t)(f * 256 + va + __ffsll(bits) - 1);
-      // where this lane's vertices' faces have their entries: one round of lanes per 32 (face, vertex)s
-      int e0[ROUNDS], e1[ROUNDS];
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, incl, o);
+      if (lane >= o) incl += t;
+    }
+    const int total = __shfl_sync(0xffffffffu, incl, 31);
+    const unsigned seen = __ballot_sync(0xffffffffu, mine > 0);
+    for (int k = incl - mine; bits; bits &= bits - 1) list[k++] = (uint16_t)(f * 256 + va + __ffsll(bits) - 1);
+    // where this lane's vertices' faces have their entries: one round of lanes per 32 (face, vertex)s
+    int e0[ROUNDS], e1[ROUNDS];
 #pragma unroll
-      for (int r = 0; r < ROUNDS; ++r) {
-        const int fi = min((r * 32 + lane) / 3, FPW - 1);
-        e1[r] = __shfl_sync(0xffffffffu, incl, fi * LPF + LPF - 1);
-        e0[r] = __shfl_sync(0xffffffffu, incl - mine, fi * LPF);
-        if (r * 32 + lane >= 3 * FPW) e1[r] = e0[r];
-      }
-      if (c0 == 0) ts_cp_async_wait_all();  // this lane's share of the faces
-      __syncwarp();
-      int next = lane < total ? list[lane] : -1;
+    for (int r = 0; r < ROUNDS; ++r) {
+      const int fi = min((r * 32 + lane) / 3, FPW - 1);
+      e1[r] = __shfl_sync(0xffffffffu, incl, fi * LPF + LPF - 1);
+      e0[r] = __shfl_sync(0xffffffffu, incl - mine, fi * LPF);
+      if (r * 32 + lane >= 3 * FPW) e1[r] = e0[r];
+    }
+    ts_cp_async_wait_all();  // this lane's share of the faces
+    __syncwarp();
+    int next = lane < total ? list[lane] : -1;
+    if (next >= 0) fetch_slot(a, slot_here, (m0 + (next >> 8)) * a.V + (next & 255));
+    for (int b0 = 0; b0 < total; b0 += 32) {
+      const int ne = min(total - b0, 32);
+      const bool act = lane < ne;
+      const int code = act ? next : 0;
+      const int fe = code >> 8, v = code & 255;
+      SlotSums sl;
+      if (act) wait_slot(slot_here, sl);
+      next = b0 + 32 + lane < total ? list[b0 + 32 + lane] : -1;
       if (next >= 0) fetch_slot(a, slot_here, (m0 + (next >> 8)) * a.V + (next & 255));
-      for (int b0 = 0; b0 < total; b0 += 32) {
-        const int ne = min(total - b0, 32);
-        const bool act = lane < ne;
-        const int code = act ? next : 0;
-        const int fe = code >> 8, v = code & 255;
-        SlotSums sl;
-        if (act) wait_slot(slot_here, sl);
-        next = b0 + 32 + lane < total ? list[b0 + 32 + lane] : -1;
-        if (next >= 0) fetch_slot(a, slot_here, (m0 + (next >> 8)) * a.V + (next & 255));
-        float tau[6];
-        if (act) {
-          SlotTerms t;
-          chain_terms(a, v, m0 + fe, sl, fdat + fe * PB_FS, views + v * VP, t);
-          float* row = rows + lane * PB_RS;
+      float tau[6];
+      if (act) {
+        SlotTerms t;
+        chain_terms(a, v, m0 + fe, sl, fdat + fe * PB_FS, views + v * VP, t);
+        float* row = rows + lane * PB_RS;
 #pragma unroll
-          for (int i = 0; i < 9; ++i) row[i] = t.out[i];
+        for (int i = 0; i < 9; ++i) row[i] = t.out[i];
 #pragma unroll
-          for (int i = 0; i < 9; ++i) row[9 + i] = t.gc[i];
-          row[18] = t.go;
-          row[19] = t.gsig;
+        for (int i = 0; i < 9; ++i) row[9 + i] = t.gc[i];
+        row[18] = t.go;
+        row[19] = t.gsig;
 #pragma unroll
-          for (int i = 0; i < 6; ++i) tau[i] = t.tau[i];
-        }
-        // pose terms: the entries of one view, in face order, one after another
-        const unsigned same = __match_any_sync(0xffffffffu, act ? v : 256 + lane);
-        const int rank = __popc(same & ((1u << lane) - 1u));
-        const int rounds = (int)__reduce_max_sync(0xffffffffu, (unsigned)rank) + 1;
-        for (int r = 0; r < rounds; ++r) {
-          if (act && rank == r) {
-#pragma unroll
-            for (int i = 0; i < 6; ++i) my[v * PB_PS + i] += tau[i];
-          }
-          __syncwarp();
-        }
-        // map words, views in order: where the batch holds many faces, the lane of each (face, vertex) sums its
-        // words over the face's rows; where it holds few (faces seen by many views), lane w sums word w over
-        // each face's rows, so that no lane walks all eight words of 32 rows.  The same sums either way.
-        const int fprev = __shfl_up_sync(0xffffffffu, fe, 1);
-        const unsigned firsts = __ballot_sync(0xffffffffu, act && (lane == 0 || fe != fprev));
-        if (__popc(firsts) <= PB_FEW) {
-          for (unsigned rem = firsts; rem; rem &= rem - 1) {
-            const int lo = __ffs(rem) - 1, hi = rem & (rem - 1) ? __ffs(rem & (rem - 1)) - 1 : ne;
-            const int face = __shfl_sync(0xffffffffu, fe, lo);
-            if (lane < PB_RS - 1) {
-              float sum = fsum[face * PB_RS + lane];
-#pragma unroll 4
-              for (int e = lo; e < hi; ++e) sum += rows[e * PB_RS + lane];
-              fsum[face * PB_RS + lane] = sum;
-            }
-          }
-        } else {
-#pragma unroll
-          for (int r = 0; r < ROUNDS; ++r) {
-            const int lo = max(e0[r] - b0, 0), hi = min(e1[r] - b0, 32);
-            if (lo < hi) {
-              const int i = r * 32 + lane, k = i % 3;
-              float* w = fsum + i / 3 * PB_RS;
-              float sum[8];
-#pragma unroll
-              for (int c = 0; c < 3; ++c) sum[c] = w[3 * k + c];
-#pragma unroll
-              for (int c = 0; c < 3; ++c) sum[3 + c] = w[9 + 3 * c + k];
-              sum[6] = w[18];
-              sum[7] = w[19];
-              for (int e = lo; e < hi; ++e) {
-                const float* row = rows + e * PB_RS;
-#pragma unroll
-                for (int c = 0; c < 3; ++c) sum[c] += row[3 * k + c];
-#pragma unroll
-                for (int c = 0; c < 3; ++c) sum[3 + c] += row[9 + 3 * c + k];
-                sum[6] += row[18];
-                sum[7] += row[19];
-              }
-#pragma unroll
-              for (int c = 0; c < 3; ++c) w[3 * k + c] = sum[c];
-#pragma unroll
-              for (int c = 0; c < 3; ++c) w[9 + 3 * c + k] = sum[3 + c];
-              if (k == 0) {  // (the face's other two lanes drop these sums)
-                w[18] = sum[6];
-                w[19] = sum[7];
-              }
-            }
-          }
-        }
-        __syncwarp();  // every lane has read the rows before the next batch writes them
+        for (int i = 0; i < 6; ++i) tau[i] = t.tau[i];
       }
+      // pose terms: the entries of one view, in face order, one after another
+      const unsigned same = __match_any_sync(0xffffffffu, act ? v : 256 + lane);
+      const int rank = __popc(same & ((1u << lane) - 1u));
+      const int rounds = (int)__reduce_max_sync(0xffffffffu, (unsigned)rank) + 1;
+      for (int r = 0; r < rounds; ++r) {
+        if (act && rank == r) {
+#pragma unroll
+          for (int i = 0; i < 6; ++i) my[v * PB_PS + i] += tau[i];
+        }
+        __syncwarp();
+      }
+      // map words, views in order: where the batch holds many faces, the lane of each (face, vertex) sums its
+      // words over the face's rows; where it holds few (faces seen by many views), lane w sums word w over
+      // each face's rows, so that no lane walks all eight words of 32 rows.  The same sums either way.
+      const int fprev = __shfl_up_sync(0xffffffffu, fe, 1);
+      const unsigned firsts = __ballot_sync(0xffffffffu, act && (lane == 0 || fe != fprev));
+      if (__popc(firsts) <= PB_FEW) {
+        for (unsigned rem = firsts; rem; rem &= rem - 1) {
+          const int lo = __ffs(rem) - 1, hi = rem & (rem - 1) ? __ffs(rem & (rem - 1)) - 1 : ne;
+          const int face = __shfl_sync(0xffffffffu, fe, lo);
+          if (lane < PB_RS - 1) {
+            float sum = fsum[face * PB_RS + lane];
+#pragma unroll 4
+            for (int e = lo; e < hi; ++e) sum += rows[e * PB_RS + lane];
+            fsum[face * PB_RS + lane] = sum;
+          }
+        }
+      } else {
+#pragma unroll
+        for (int r = 0; r < ROUNDS; ++r) {
+          const int lo = max(e0[r] - b0, 0), hi = min(e1[r] - b0, 32);
+          if (lo < hi) {
+            const int i = r * 32 + lane, k = i % 3;
+            float* w = fsum + i / 3 * PB_RS;
+            float sum[8];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) sum[c] = w[3 * k + c];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) sum[3 + c] = w[9 + 3 * c + k];
+            sum[6] = w[18];
+            sum[7] = w[19];
+            for (int e = lo; e < hi; ++e) {
+              const float* row = rows + e * PB_RS;
+#pragma unroll
+              for (int c = 0; c < 3; ++c) sum[c] += row[3 * k + c];
+#pragma unroll
+              for (int c = 0; c < 3; ++c) sum[3 + c] += row[9 + 3 * c + k];
+              sum[6] += row[18];
+              sum[7] += row[19];
+            }
+#pragma unroll
+            for (int c = 0; c < 3; ++c) w[3 * k + c] = sum[c];
+#pragma unroll
+            for (int c = 0; c < 3; ++c) w[9 + 3 * c + k] = sum[3 + c];
+            if (k == 0) {  // (the face's other two lanes drop these sums)
+              w[18] = sum[6];
+              w[19] = sum[7];
+            }
+          }
+        }
+      }
+      __syncwarp();  // every lane has read the rows before the next batch writes them
     }
     // into the map gradient; a face seen by no view adds nothing
     for (int i = lane; i < 3 * FPW; i += 32) {
@@ -591,10 +585,19 @@ int ts_pose_blocks(long long M) {        // the most either form uses
 }
 
 namespace {
+// Shared memory of a block of the form with map gradients, and whether four such blocks fit on a
+// multiprocessor (228 KB, of which each block takes 1 KB more): up to 23 views of 32 faces, 68 of 16.
+constexpr int pbwd_smem(int V, int faces) {
+  return (PB_WARPS * pbwd_warp_floats(V, faces) + V * VP) * (int)sizeof(float);
+}
+constexpr bool pbwd_four_blocks(int V, int faces) { return 4 * (pbwd_smem(V, faces) + 1024) <= 228 * 1024; }
+static_assert(pbwd_four_blocks(23, 32) && !pbwd_four_blocks(65, 32) && pbwd_four_blocks(68, 16) &&
+                  !pbwd_four_blocks(129, 16) && TS_MAX_VIEWS <= 256,
+              "a lane looks up at most 64 views of its face, an entry holds its view in 8 bits");
+
 template <int FPW>
 cudaError_t launch_pbwd_map(const PBArgs& a, cudaStream_t s) {
-  const int smem =
-      (PB_WARPS * pbwd_warp_floats(a.V, FPW) + a.V * VP) * (int)sizeof(float);  // <= 146 KB
+  const int smem = pbwd_smem(a.V, FPW);  // at most 90.6 KB (256 views)
   const cudaError_t e = ts_smem_limit((const void*)k_pbwd_map<FPW>, smem);
   if (e != cudaSuccess) return e;
   const long long want = (a.M + PB_WARPS * FPW - 1) / (PB_WARPS * FPW);
@@ -639,8 +642,9 @@ cudaError_t ts_launch_project_bwd(const TsPlanImpl* p, const TsWs& w, const ts_m
     return cudaGetLastError();
   }
   // 32 faces a warp once every warp of the grid has some, fewer of smaller maps and where more views would
-  // leave room for three blocks on an SM instead of four (and the grid a second wave)
-  const int most = p->V <= 20 ? 32 : (p->V <= 48 ? 16 : 8);
+  // leave room for three blocks on an SM instead of four (and the grid a second wave): 300k faces take 141 us at
+  // 23 views of 32 faces and 150 of 16, 332 at 64 views of 16 and 346 of 8.  Above 110 views even 8 faces leave three.
+  const int most = pbwd_four_blocks(p->V, 32) ? 32 : (pbwd_four_blocks(p->V, 16) ? 16 : 8);
   const int faces = std::min(most, p->M > MAP_BLOCKS * PB_WARPS * 16 ? 32 : (p->M > MAP_BLOCKS * PB_WARPS * 8 ? 16 : 8));
   if (faces == 32) return launch_pbwd_map<32>(a, s);
   if (faces == 16) return launch_pbwd_map<16>(a, s);
