@@ -229,8 +229,9 @@ struct MatArgs {
   long long M, n_tiles, cap;
   int faces;             // per block, a multiple of BIN_T
   uint32_t* mat;         // [face block][tile]: pair counts, then their exclusive sums down the column
-  const uint32_t* tpre;  // per tile: the pairs of the tiles before it in its group of TS_BIN_GROUP
+  const uint32_t* tpre;  // per tile: the pairs of the tiles before it in its group of 2^shift
   const uint32_t* gsum;  // per group: the pairs of the groups before it
+  int shift;
   unsigned long long* seg;
 };
 
@@ -336,14 +337,15 @@ __global__ void __launch_bounds__(BIN_T, 3) k_bin_counts(MatArgs a) {
   for (int t = threadIdx.x; t < T; t += BIN_T) row[t] = hcnt[t];
 }
 
-// One block per TS_BIN_GROUP tiles, a lane per tile and a warp per share of the rows: the exclusive sums down
-// each tile's column in place, up to 64 rows at a time in registers; the tiles' totals, scanned within the
-// group, and the group's total.
+// The exclusive sums down each tile's column in place; the tiles' totals, scanned within the group, and the
+// group's total.  One block per 32 tiles, a lane per tile and a warp per share of the rows, up to 64 rows at a
+// time in registers; for many tiles of at most TS_BIN_FEW rows one block per 256 tiles, a thread per tile, so that
+// views of many tiles and few faces do not launch a block of mostly idle warps per 32 tiles, nor scan as many groups:
+// 16 views of 1920 x 1080 at 8 x 8 tiles, 2000 faces, columns and scan 46 -> 11 us.
 constexpr int COL_WARPS = 8, COL_ROWS = 8;  // warps per block, most rows per warp at a time
 __global__ void __launch_bounds__(32 * COL_WARPS) k_bin_columns(uint32_t* __restrict__ mat, long long n_tiles, int B,
                                                                  uint32_t* __restrict__ tpre,
                                                                  uint32_t* __restrict__ gsum, unsigned int* wraps) {
-  static_assert(TS_BIN_GROUP == 32, "a lane per tile of the group");
   __shared__ uint32_t part[COL_WARPS][32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const long long t = (long long)blockIdx.x * 32 + lane;
@@ -388,6 +390,33 @@ __global__ void __launch_bounds__(32 * COL_WARPS) k_bin_columns(uint32_t* __rest
   }
 }
 
+__global__ void __launch_bounds__(256) k_bin_columns_few(uint32_t* __restrict__ mat, long long n_tiles, int B,
+                                                         uint32_t* __restrict__ tpre, uint32_t* __restrict__ gsum) {
+  static_assert(256ll * TS_BIN_FEW * TS_BIN_FACES < (1ll << 32), "a group's pairs fit 32 bits");
+  __shared__ uint32_t wsum[8];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long t = (long long)blockIdx.x * 256 + threadIdx.x;
+  uint32_t c[TS_BIN_FEW], total = 0u;
+#pragma unroll
+  for (int k = 0; k < TS_BIN_FEW; ++k) c[k] = t < n_tiles && k < B ? mat[k * n_tiles + t] : 0u;
+#pragma unroll
+  for (int k = 0; k < TS_BIN_FEW; ++k) {
+    if (t < n_tiles && k < B) mat[k * n_tiles + t] = total;
+    total += c[k];
+  }
+  const uint32_t incl = warp_incl_scan(total);
+  if (lane == 31) wsum[warp] = incl;
+  __syncthreads();
+  uint32_t before = 0u, all = 0u;
+#pragma unroll
+  for (int w = 0; w < 8; ++w) {
+    before += w < warp ? wsum[w] : 0u;
+    all += wsum[w];
+  }
+  if (t < n_tiles) tpre[t] = before + incl - total;
+  if (threadIdx.x == 0) gsum[blockIdx.x] = all;
+}
+
 __global__ void __launch_bounds__(BIN_T, 3) k_bin_place(MatArgs a) {
   extern __shared__ uint32_t place[];
   __shared__ WideFaces wide;
@@ -398,7 +427,9 @@ __global__ void __launch_bounds__(BIN_T, 3) k_bin_place(MatArgs a) {
   const uint32_t* row = a.mat + (long long)blockIdx.x * a.n_tiles;
   for (int t = threadIdx.x; t < T; t += BIN_T) {
     const long long g = vw.tile_off + t;
-    place[t] = row[g] + a.tpre[g] + a.gsum[g / TS_BIN_GROUP];
+    // (a group of 32 or 256 tiles; a shift by a register leaves 32 registers for 36 and so four blocks on a
+    // multiprocessor for three: 62 us for 53 at 20 views of 300k faces, 69 for 77 at 12 of 1M)
+    place[t] = row[g] + a.tpre[g] + (a.shift == 5 ? a.gsum[g / 32] : a.gsum[g / 256]);
   }
   __syncthreads();
   for_each_pair<true>(a, v, blockIdx.x, TX, wide, [&](int t, uint32_t z, uint32_t id) {
@@ -421,6 +452,7 @@ struct SortOut {
   unsigned int* n_large;
   const uint32_t* tpre;    // with the count matrix: pairs of the tiles before this one in its group, else null
   const uint32_t* gsum;    // (ranges from the scatter); pairs of the groups before
+  int shift;               // log2 of the tiles of a group
   const unsigned long long* n_pairs;
 };
 
@@ -431,6 +463,8 @@ __device__ __forceinline__ void put_pair(const SortOut& o, long long t, long lon
 
 constexpr int WARP_SORT_MAX = 512;  // pairs a warp sorts in its registers (16 per lane)
 constexpr int SORT_WARPS_PER_BLOCK = 8;
+constexpr int SORT_TILES = 2;  // tiles a warp takes of at least SORT_TILES_FROM
+constexpr long long SORT_TILES_FROM = 40000;
 
 // Keep the smaller (lower) or the larger key of a compare-exchange with a lane that keeps the other.
 __device__ __forceinline__ unsigned long long keep_key(unsigned long long x, unsigned long long y, bool lower) {
@@ -504,34 +538,13 @@ __device__ __forceinline__ void sort_segment(const SortOut& o, long long t, long
 #pragma unroll
   for (int r = 0; r < K; ++r)
     if (r * 32 + lane < n) put_pair(o, t, start + r * 32 + lane, buf[key_place(r * 32 + lane)]);
+  __syncwarp();  // the warp's next tile writes the buffer
 }
 
-// One warp per tile, its keys in registers; segments longer than WARP_SORT_MAX are listed for the
-// CTA-wide kernel.  Issue-bound (about 6 warp instructions a key at 512 keys, 4.5 at 128).  Lists of
-// more than 64 pairs in shared memory, with an integer division per exchange, took 161 us where this
-// takes 73 (12 views of a 1M-face map, 127 pairs a tile) and 35 where it takes 9 (mesh, 561k pixels).
-__global__ void __launch_bounds__(32 * SORT_WARPS_PER_BLOCK) k_tile_sort(SortOut o) {
-  __shared__ unsigned long long sbuf[SORT_WARPS_PER_BLOCK][WARP_SORT_MAX];
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const long long t = (long long)blockIdx.x * SORT_WARPS_PER_BLOCK + warp;
-  if (t >= o.n_tiles) return;
-  // the segment: from the scanned totals (its first place, the next tile's, the pair total after the
-  // last tile), else as the scatter left it in ranges
-  uint2 rg;
-  if (o.tpre) {
-    rg.x = o.tpre[t] + o.gsum[t / TS_BIN_GROUP];
-    rg.y = t + 1 < o.n_tiles ? o.tpre[t + 1] + o.gsum[(t + 1) / TS_BIN_GROUP]
-                             : (uint32_t)min(*o.n_pairs, 0xffffffffull);
-  } else {
-    rg = o.ranges[t];
-  }
-  const long long start = min((long long)rg.x, o.cap);
-  const long long end = max(start, min((long long)rg.y, o.cap));  // (an end past 2^32 has wrapped to below its start)
-  // the tile's range for the passes that follow; past the capacity (its bit is latched) the lists
-  // are cut, and the ranges with them, so that no later pass reads outside the pair list
-  if (lane == 0 && (o.tpre || start != rg.x || end != rg.y)) o.ranges[t] = make_uint2((uint32_t)start, (uint32_t)end);
-  const int n = (int)(end - start);
-  if (n == 0) return;
+// Sort the n >= 1 pairs of tile t, which start at `start` of the segments; lists beyond WARP_SORT_MAX are listed for
+// the CTA-wide kernel.
+__device__ __forceinline__ void sort_tile(const SortOut& o, long long t, long long start, int n, int lane,
+                                          unsigned long long* buf) {
   if (n <= 32) {
     unsigned long long x = lane < n ? o.seg[start + lane] : ~0ull;
 #pragma unroll
@@ -597,9 +610,56 @@ __global__ void __launch_bounds__(32 * SORT_WARPS_PER_BLOCK) k_tile_sort(SortOut
     }
     return;
   }
-  if (n <= 128) sort_segment<4>(o, t, start, n, lane, sbuf[warp]);
-  else if (n <= 256) sort_segment<8>(o, t, start, n, lane, sbuf[warp]);
-  else sort_segment<16>(o, t, start, n, lane, sbuf[warp]);
+  if (n <= 128) sort_segment<4>(o, t, start, n, lane, buf);
+  else if (n <= 256) sort_segment<8>(o, t, start, n, lane, buf);
+  else sort_segment<16>(o, t, start, n, lane, buf);
+}
+
+// A warp takes TILES consecutive tiles, their keys in registers.  Issue-bound (about 6 warp instructions a key at 512
+// keys, 4.5 at 128).  Lists of more than 64 pairs in shared memory, with an integer division per exchange, took 161 us
+// where this takes 73 (12 views of a 1M-face map, 127 pairs a tile) and 35 where it takes 9 (mesh, 561k pixels).
+// An empty or short list is two dependent loads and a store, and with one tile a warp such tiles wait for the 32 places
+// of a multiprocessor that 64 registers leave; so from SORT_TILES_FROM tiles on a warp takes two, and the compiler's 48
+// registers leave 40 places: 518k tiles of 2000 faces 93 -> 54 us, 20 views of 300k faces 76 -> 69.  (Below, two tiles
+// a warp leave places empty: 57k tiles of the 12-view window 85 us either way, 117 with four.)
+template <int TILES>
+__global__ void __launch_bounds__(32 * SORT_WARPS_PER_BLOCK, TILES == 1 ? 4 : 5) k_tile_sort(SortOut o) {
+  __shared__ unsigned long long sbuf[SORT_WARPS_PER_BLOCK][WARP_SORT_MAX];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const long long t0 = ((long long)blockIdx.x * SORT_WARPS_PER_BLOCK + warp) * TILES;
+  if (t0 >= o.n_tiles) return;
+  // lane i: the segment of tile t0 + i, from the scanned totals (its first place, the next tile's, the pair total
+  // after the last tile), else as the scatter left it in ranges
+  const long long tl = TILES == 1 ? t0 : t0 + lane;
+  auto first_of = [&](long long t) {
+    return t < o.n_tiles ? o.tpre[t] + o.gsum[t >> o.shift] : (uint32_t)min(*o.n_pairs, 0xffffffffull);
+  };
+  uint2 rg = make_uint2(0u, 0u);
+  if (TILES == 1) {
+    rg = o.tpre ? make_uint2(first_of(tl), first_of(tl + 1)) : o.ranges[tl];
+  } else if (o.tpre) {
+    rg.x = lane <= TILES ? first_of(min(tl, o.n_tiles)) : 0u;
+    rg.y = __shfl_down_sync(0xffffffffu, rg.x, 1);
+  } else if (lane < TILES && tl < o.n_tiles) {
+    rg = o.ranges[tl];
+  }
+  const long long first = min((long long)rg.x, o.cap);
+  const long long last = max(first, min((long long)rg.y, o.cap));  // (an end past 2^32 has wrapped to below its start)
+  // the tile's range for the passes that follow; past the capacity (its bit is latched) the lists
+  // are cut, and the ranges with them, so that no later pass reads outside the pair list
+  const bool mine = lane < TILES && tl < o.n_tiles;
+  if (mine && (o.tpre || first != rg.x || last != rg.y)) o.ranges[tl] = make_uint2((uint32_t)first, (uint32_t)last);
+  const int len = (int)(last - first);
+  if constexpr (TILES == 1) {
+    if (len > 0) sort_tile(o, t0, first, len, lane, sbuf[warp]);
+  } else {
+#pragma unroll 1
+    for (unsigned rem = __ballot_sync(0xffffffffu, mine && len > 0); rem; rem &= rem - 1) {
+      const int i = __ffs(rem) - 1;
+      sort_tile(o, t0 + i, __shfl_sync(0xffffffffu, (unsigned int)first, i), __shfl_sync(0xffffffffu, len, i), lane,
+                sbuf[warp]);
+    }
+  }
 }
 
 constexpr int LARGE_T = 256;
@@ -721,16 +781,20 @@ cudaError_t ts_launch_bin(const TsPlanImpl* p, const TsWs& w, cudaStream_t s) {
   if (p->bin_blocks > 0) {
     // 1-3 with shared-memory counts: counts, their scan (the total is the pair count; above the
     // capacity latches its bit), places, ranges
-    MatArgs ma{w.rect, w.zbits, w.views, p->M, p->n_tiles, p->cap, (int)p->bin_faces, w.tmat, w.tcnt, w.bsums, w.keys[1]};
+    MatArgs ma{w.rect, w.zbits, w.views, p->M, p->n_tiles, p->cap, (int)p->bin_faces, w.tmat, w.tcnt, w.bsums,
+               (int)p->bin_shift, w.keys[1]};
     const int smem = (int)(p->max_view_tiles * sizeof(uint32_t));
     e = ts_smem_limit((const void*)k_bin_counts, smem);
     if (e == cudaSuccess) e = ts_smem_limit((const void*)k_bin_place, smem);
     if (e != cudaSuccess) return e;
     const dim3 grid((unsigned)p->bin_blocks, (unsigned)p->V);
     k_bin_counts<<<grid, BIN_T, smem, s>>>(ma);
-    const unsigned ng = (unsigned)((p->n_tiles + TS_BIN_GROUP - 1) / TS_BIN_GROUP);
-    k_bin_columns<<<ng, 32 * COL_WARPS, 0, s>>>(w.tmat, p->n_tiles, (int)p->bin_blocks, w.tcnt, w.bsums,
-                                             &w.hdr->pair_wraps);
+    const unsigned ng = (unsigned)(((p->n_tiles - 1) >> p->bin_shift) + 1);
+    if (p->bin_shift == 8)
+      k_bin_columns_few<<<ng, 256, 0, s>>>(w.tmat, p->n_tiles, (int)p->bin_blocks, w.tcnt, w.bsums);
+    else
+      k_bin_columns<<<ng, 32 * COL_WARPS, 0, s>>>(w.tmat, p->n_tiles, (int)p->bin_blocks, w.tcnt, w.bsums,
+                                                   &w.hdr->pair_wraps);
     k_scan_bsums<<<1, SCAN_T, 0, s>>>(w.bsums, ng, &w.hdr->n_pairs, &w.hdr->error_bits, p->cap,
                                        &w.hdr->pair_wraps, &w.hdr->n_large);
     k_bin_place<<<grid, BIN_T, smem, s>>>(ma);
@@ -753,9 +817,11 @@ cudaError_t ts_launch_bin(const TsPlanImpl* p, const TsWs& w, cudaStream_t s) {
   // 4: the segments' sorts
   // (with the matrix, the sort also writes each tile's range)
   SortOut so{w.keys[1], w.keys[0], w.vals[0], w.ranges, p->n_tiles, p->cap, w.tlarge, &w.hdr->n_large,
-             p->bin_blocks > 0 ? w.tcnt : nullptr, w.bsums, &w.hdr->n_pairs};
-  k_tile_sort<<<(unsigned)((p->n_tiles + SORT_WARPS_PER_BLOCK - 1) / SORT_WARPS_PER_BLOCK), 32 * SORT_WARPS_PER_BLOCK,
-                0, s>>>(so);
+             p->bin_blocks > 0 ? w.tcnt : nullptr, w.bsums, (int)p->bin_shift, &w.hdr->n_pairs};
+  const long long per = p->n_tiles >= SORT_TILES_FROM ? SORT_TILES : 1;
+  const unsigned nw = (unsigned)((p->n_tiles + per * SORT_WARPS_PER_BLOCK - 1) / (per * SORT_WARPS_PER_BLOCK));
+  if (per > 1) k_tile_sort<SORT_TILES><<<nw, 32 * SORT_WARPS_PER_BLOCK, 0, s>>>(so);
+  else k_tile_sort<1><<<nw, 32 * SORT_WARPS_PER_BLOCK, 0, s>>>(so);
   constexpr int large_smem = 2 * LARGE_ITEMS * (int)sizeof(unsigned long long);
   e = ts_smem_limit((const void*)k_tile_sort_large, large_smem);
   if (e != cudaSuccess) return e;

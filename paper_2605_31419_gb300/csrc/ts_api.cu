@@ -148,7 +148,8 @@ ts_status ts_plan_init(ts_plan* plan, const ts_camera* cams, int32_t n_views, in
   p->bin_faces = 1024;
   while (p->bin_faces < TS_BIN_FACES && n_views * ((n_faces + p->bin_faces - 1) / p->bin_faces) > 456) p->bin_faces *= 2;
   p->bin_blocks = max_tiles <= TS_BIN_MAX_TILES ? std::max<int64_t>(1, (n_faces + p->bin_faces - 1) / p->bin_faces) : 0;
-  const int64_t scan_items = p->bin_blocks ? TS_BIN_GROUP : TS_SCAN_ITEMS;
+  p->bin_shift = p->bin_blocks <= TS_BIN_FEW && toff >= 16384 ? 8 : 5;
+  const int64_t scan_items = p->bin_blocks ? int64_t(1) << p->bin_shift : TS_SCAN_ITEMS;
   p->n_tile_scan_blocks = std::max<int64_t>(1, (toff + scan_items - 1) / scan_items);
   p->n_pose_blocks = std::max(1, ts_pose_blocks(n_faces));
   int64_t max_hw = 0;

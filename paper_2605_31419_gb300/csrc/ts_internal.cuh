@@ -16,7 +16,7 @@
 #define TS_GRAD_WORDS 32           // per-(view, face) gradient slot
 #define TS_SCAN_ITEMS 4096         // items per scan block (1024 threads x 4)
 #define TS_BIN_FACES 8192          // most faces per block of the shared-memory tile counts
-#define TS_BIN_GROUP 32            // tiles whose counts are scanned by one warp
+#define TS_BIN_FEW 8               // rows of the count matrix up to which a thread sums a tile's column
 #define TS_BIN_MAX_TILES 40960     // the most tiles of a view those counts hold (160 KB)
 #define TS_ERRBIT_CAPACITY 1u
 #define TS_ERRBIT_TIMEOUT 2u
@@ -96,6 +96,7 @@ struct TsPlanImpl {
   int64_t loss_per;         // pixels per thread of the loss kernels
   int64_t bin_faces;        // faces per block of the shared-memory tile counts
   int64_t bin_blocks;       // face blocks per view of the shared-memory tile counts (0: global counts)
+  int64_t bin_shift;        // with them: a group of 2^bin_shift tiles is scanned by one warp (5) or block (8)
   int64_t max_view_tiles;   // the most tiles of one view
   bool normals;  // TS_FLAG_NORMALS
   bool stats;    // TS_FLAG_STATS

@@ -271,3 +271,53 @@ def test_padded_maps(n_faces, n_views, indexed):
     # sums over some 3000 vertices of such terms, which cancel in part
     for x, y in ((a["dtau"], b["dtau"]), (a["pose"], b["pose"]), (a["dtau"], a["pose"])):
         assert np.abs(x - y).max() <= 1e-4 * np.abs(x).max()
+
+
+@pytest.mark.parametrize("n_views,n_faces,size", [
+    (1, 700, (1021, 1030)),    # 16,512 tiles, one row of the count matrix: groups of 256 tiles, a tile per warp of the sort
+    (3, 1500, (1021, 1019)),   # 49,152 tiles, two rows: two tiles per warp
+    (5, 8200, (809, 803)),     # 51,510 tiles, nine rows: groups of 32
+    (3, 900, (1090, 1011)),    # 52,197 tiles: one left for the last warp, a last group that is not full
+])
+def test_tile_lists_of_many_tiles(n_views, n_faces, size):
+    """Every tile's list of views of many tiles, most of them empty and some with more than 512 faces: the whole
+    pair list and the ranges against the faces' rectangles."""
+    import paper_2605_31419_gb300 as ts
+    W, H = size
+    rng = np.random.default_rng(n_faces)
+    z = rng.uniform(1.0, 2.0, n_faces)
+    z[::3] = np.float32(1.5)  # ties go by the face
+    centre = rng.uniform([0.0, 0.0], [W, H], (n_faces, 2))
+    centre[:600] = rng.normal([0.7 * W, 0.3 * H], 5.0, (600, 2))  # a heap
+    side = rng.uniform(2.0, 40.0, n_faces)
+    tri = np.array([[-0.5, -0.5], [0.5, -0.5], [0.0, 0.5]])
+    xy = (centre - [W / 2, H / 2])[:, None] + tri[None] * side[:, None, None]
+    pos = np.concatenate([xy * (z / 500.0)[:, None, None], np.repeat(z[:, None, None], 3, 1)], 2)
+    poses = np.tile([1, 0, 0, 0, 1, 0, 0, 0, 1, 0, 0, 0.0], (n_views, 1))
+    poses[:, 9] = 0.3 * np.arange(n_views)
+    m = ts.Map.from_numpy(pos.reshape(-1, 3).astype(np.float32), np.full((3 * n_faces, 3), 0.5, np.float32),
+                          np.full(3 * n_faces, 0.5, np.float32))
+    r = ts.Rasterizer(np.array([[500.0, 500.0, W / 2, H / 2, W, H]] * n_views), n_faces,
+                      ts.ts_default_params(tile_w=8, tile_h=8), pair_capacity=2_000_000)
+    r.project(m, ts.poses_tensor(poses.astype(np.float32)))
+    r.bin()
+    TX, TY = (W + 7) // 8, (H + 7) // 8
+    rect = r.debug("rect").cpu().numpy().view(np.int16).reshape(n_views * n_faces, 4).astype(np.int64)
+    on = np.flatnonzero(rect[:, 0] >= 0)
+    wid, hei = rect[on, 2] - rect[on, 0] + 1, rect[on, 3] - rect[on, 1] + 1
+    n = wid * hei
+    of = np.repeat(on, n)
+    k = np.arange(n.sum()) - np.repeat(np.cumsum(n) - n, n)
+    w = np.repeat(wid, n)
+    tile = of // n_faces * (TX * TY) + (rect[of, 1] + k // w) * TX + rect[of, 0] + k % w
+    zb = r.debug("zbits").cpu().numpy().view(np.uint32)[of].astype(np.uint64)
+    order = np.lexsort((of % n_faces, zb, tile))
+    total = len(order)
+    assert r.counters()["n_pairs"] == total and r.counters()["error_bits"] == 0
+    assert np.array_equal(r.debug("ids").cpu().numpy().view(np.uint32)[:total], (of % n_faces)[order])
+    assert np.array_equal(r.debug("keys").cpu().numpy().view(np.uint64)[:total],
+                          (tile[order].astype(np.uint64) << np.uint64(32)) | zb[order])
+    ends = np.searchsorted(tile[order], np.arange(n_views * TX * TY), side="right")
+    starts = np.searchsorted(tile[order], np.arange(n_views * TX * TY), side="left")
+    assert np.array_equal(r.debug("ranges").cpu().numpy().view(np.uint32).reshape(-1, 2), np.stack([starts, ends], 1))
+    assert (ends - starts).max() > 512
