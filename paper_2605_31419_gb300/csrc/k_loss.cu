@@ -13,30 +13,33 @@
 namespace {
 
 constexpr int LOSS_T = 256;
-// Pixels per thread (PER): the plan's 8 or 2.  Eight keep the partial sums few; where that leaves fewer than
-// four blocks per multiprocessor, two give four times
-// the blocks: 7 views of 317x239 take 4.7 us instead of 9.6, three mixed views 5.3 instead of 11.2.
+// Two pixels per thread: with eight, the loads of a block's last pixels wait for its first ones' stores (20 views of
+// 1200x680 153 us, now 130; 7 views of 317x239 6.1 and 4.5).  A view's sums do not depend on the other views.
+constexpr int LOSS_PER = 2;
+static_assert(LOSS_T * LOSS_PER == TS_LOSS_PIXELS, "pixels of a block");
 
-template <int PER>
 __global__ void __launch_bounds__(LOSS_T) k_loss_partial(const TsImageTable tab, const float* __restrict__ C,
                                                          const float* __restrict__ D, const float* __restrict__ tC,
                                                          const float* __restrict__ tD, float lambda_dep,
                                                          float* __restrict__ dC, float* __restrict__ dD,
                                                          float* __restrict__ part, int nblk) {
   const int v = blockIdx.y;
-  ts_l1_loss_block<LOSS_T, PER>((long long)tab.W[v] * tab.H[v], tab.pix_off[v], (long long)blockIdx.x * LOSS_T * PER,
-                                C, D, tC, tD, lambda_dep, dC, dD, part + ((long long)v * nblk + blockIdx.x) * 2);
+  ts_l1_loss_block<LOSS_T, LOSS_PER>((long long)tab.W[v] * tab.H[v], tab.pix_off[v],
+                                     (long long)blockIdx.x * LOSS_T * LOSS_PER, C, D, tC, tD, lambda_dep, dC, dD,
+                                     part + ((long long)v * nblk + blockIdx.x) * 2);
 }
 
+// One block per view, over the view's own partial sums.
 __global__ void __launch_bounds__(LOSS_T) k_loss_final(const TsImageTable tab, const float* __restrict__ part,
-                                                       int nblk, float lambda_dep, float* __restrict__ loss) {
+                                                        int nblk, float lambda_dep, float* __restrict__ loss) {
   const int v = blockIdx.x;
-  ts_l1_loss_final<LOSS_T>((long long)tab.W[v] * tab.H[v], part + (long long)v * nblk * 2, nblk, lambda_dep, loss + v);
+  const long long HW = (long long)tab.W[v] * tab.H[v];
+  ts_l1_loss_final<LOSS_T>(HW, part + (long long)v * nblk * 2, (int)((HW + TS_LOSS_PIXELS - 1) / TS_LOSS_PIXELS),
+                            lambda_dep, loss + v);
 }
 
 // Normal loss of Eq. 12 per view: sum over pixels with a sensor normal (Nbar != 0) of
 // (1 - N . Nbar) / HW, with dN = weight * dloss/dN = -weight Nbar / HW there and 0 elsewhere.
-template <int PER>
 __global__ void __launch_bounds__(LOSS_T) k_nloss_partial(const TsImageTable tab, const float* __restrict__ N,
                                                           const float* __restrict__ tN, float weight,
                                                           float* __restrict__ dN, float* __restrict__ part, int nblk) {
@@ -44,12 +47,12 @@ __global__ void __launch_bounds__(LOSS_T) k_nloss_partial(const TsImageTable tab
   const int v = blockIdx.y;
   const long long HW = (long long)tab.W[v] * tab.H[v];
   const long long pix_off = tab.pix_off[v];
-  const long long base = (long long)blockIdx.x * LOSS_T * PER;
+  const long long base = (long long)blockIdx.x * LOSS_T * LOSS_PER;
   float l = 0.f;
   if (base < HW) {
     const float sc = -weight / (float)HW;
 #pragma unroll
-    for (int k = 0; k < PER; ++k) {
+    for (int k = 0; k < LOSS_PER; ++k) {
       const long long i = base + (long long)k * LOSS_T + threadIdx.x;
       if (i >= HW) break;
       float nb[3], dot = 0.f;
@@ -82,8 +85,17 @@ __global__ void __launch_bounds__(LOSS_T) k_nloss_final(const TsImageTable tab, 
                                                         int nblk, float* __restrict__ loss) {
   __shared__ double red[LOSS_T];
   const int v = blockIdx.x;
+  const int n = (int)(((long long)tab.W[v] * tab.H[v] + TS_LOSS_PIXELS - 1) / TS_LOSS_PIXELS);
+  const float* p = part + (long long)v * nblk;
   double a = 0;
-  for (int k = threadIdx.x; k < nblk; k += LOSS_T) a += part[(long long)v * nblk + k];
+  // four blocks' sums, 2048 pixels, per 64-bit addition (of which there are few a cycle)
+#pragma unroll 4
+  for (int k = 4 * threadIdx.x; k < n; k += 4 * LOSS_T) {
+    float q[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) q[i] = k + i < n ? p[k + i] : 0.f;
+    a += (q[0] + q[1]) + (q[2] + q[3]);
+  }
   red[threadIdx.x] = a;
   __syncthreads();
   for (int o = LOSS_T / 2; o > 0; o >>= 1) {
@@ -195,10 +207,7 @@ cudaError_t ts_launch_l1_loss(const TsPlanImpl* p, const TsWs& w, const float* c
   const int nblk = (int)p->n_loss_blocks;
   dim3 grid((unsigned)nblk, (unsigned)p->V);
   const TsImageTable tab = ts_image_table(p);
-  if (p->loss_per == 8)
-    k_loss_partial<8><<<grid, LOSS_T, 0, s>>>(tab, color, depth, tc, td, lambda_dep, dC, dD, w.loss, nblk);
-  else
-    k_loss_partial<2><<<grid, LOSS_T, 0, s>>>(tab, color, depth, tc, td, lambda_dep, dC, dD, w.loss, nblk);
+  k_loss_partial<<<grid, LOSS_T, 0, s>>>(tab, color, depth, tc, td, lambda_dep, dC, dD, w.loss, nblk);
   k_loss_final<<<p->V, LOSS_T, 0, s>>>(tab, w.loss, nblk, lambda_dep, loss);
   return cudaGetLastError();
 }
@@ -208,8 +217,7 @@ cudaError_t ts_launch_normal_loss(const TsPlanImpl* p, const TsWs& w, const floa
   const int nblk = (int)p->n_loss_blocks;
   const TsImageTable tab = ts_image_table(p);
   const dim3 grid((unsigned)nblk, (unsigned)p->V);
-  if (p->loss_per == 8) k_nloss_partial<8><<<grid, LOSS_T, 0, s>>>(tab, normal, tgt, weight, dN, w.nloss, nblk);
-  else k_nloss_partial<2><<<grid, LOSS_T, 0, s>>>(tab, normal, tgt, weight, dN, w.nloss, nblk);
+  k_nloss_partial<<<grid, LOSS_T, 0, s>>>(tab, normal, tgt, weight, dN, w.nloss, nblk);
   k_nloss_final<<<p->V, LOSS_T, 0, s>>>(tab, w.nloss, nblk, loss);
   return cudaGetLastError();
 }

@@ -154,9 +154,7 @@ ts_status ts_plan_init(ts_plan* plan, const ts_camera* cams, int32_t n_views, in
   p->n_pose_blocks = std::max(1, ts_pose_blocks(n_faces));
   int64_t max_hw = 0;
   for (int v = 0; v < n_views; ++v) max_hw = std::max<int64_t>(max_hw, (int64_t)p->views[v].W * p->views[v].H);
-  // pixels per thread of the loss kernels (256 threads): 8 once that gives four blocks per multiprocessor
-  p->loss_per = n_views * ((max_hw + 2047) / 2048) >= 608 ? 8 : 2;
-  p->n_loss_blocks = (max_hw + 256 * p->loss_per - 1) / (256 * p->loss_per);
+  p->n_loss_blocks = (max_hw + TS_LOSS_PIXELS - 1) / TS_LOSS_PIXELS;
   p->n_pho_blocks = ts_pho_blocks(p->views, n_views);
   p->normals = (prm->flags & TS_FLAG_NORMALS) != 0;
   p->stats = (prm->flags & TS_FLAG_STATS) != 0;

@@ -18,6 +18,7 @@
 #define TS_BIN_FACES 8192          // most faces per block of the shared-memory tile counts
 #define TS_BIN_FEW 8               // rows of the count matrix up to which a thread sums a tile's column
 #define TS_BIN_MAX_TILES 40960     // the most tiles of a view those counts hold (160 KB)
+#define TS_LOSS_PIXELS 512         // pixels per block of the L1 and normal losses
 #define TS_ERRBIT_CAPACITY 1u
 #define TS_ERRBIT_TIMEOUT 2u
 #define TS_ERRBIT_BOUNDS 4u  // an index failed its bounds check (the access was skipped)
@@ -93,7 +94,6 @@ struct TsPlanImpl {
   ts_raster_params prm;
   int64_t n_tiles, n_pix;
   int64_t n_tile_scan_blocks, n_pose_blocks, n_loss_blocks, n_pho_blocks;
-  int64_t loss_per;         // pixels per thread of the loss kernels
   int64_t bin_faces;        // faces per block of the shared-memory tile counts
   int64_t bin_blocks;       // face blocks per view of the shared-memory tile counts (0: global counts)
   int64_t bin_shift;        // with them: a group of 2^bin_shift tiles is scanned by one warp (5) or block (8)
@@ -409,9 +409,16 @@ __device__ __forceinline__ void ts_l1_loss_final(long long HW, const float* part
                                                  float* loss) {
   __shared__ float red[NT][2];
   float a = 0.f, b = 0.f;
-  for (int k = threadIdx.x; k < nblk; k += NT) {
-    a += part[2 * (long long)k];
-    b += part[2 * (long long)k + 1];
+  for (int k = threadIdx.x; k < nblk; k += 4 * NT) {  // four blocks' sums in flight, added in order
+    float2 q[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      q[i] = k + i * NT < nblk ? reinterpret_cast<const float2*>(part)[k + i * NT] : make_float2(0.f, 0.f);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      a += q[i].x;
+      b += q[i].y;
+    }
   }
   red[threadIdx.x][0] = a;
   red[threadIdx.x][1] = b;

@@ -321,3 +321,31 @@ def test_tile_lists_of_many_tiles(n_views, n_faces, size):
     starts = np.searchsorted(tile[order], np.arange(n_views * TX * TY), side="left")
     assert np.array_equal(r.debug("ranges").cpu().numpy().view(np.uint32).reshape(-1, 2), np.stack([starts, ends], 1))
     assert (ends - starts).max() > 512
+
+
+def test_losses_do_not_depend_on_the_batch():
+    """The L1 and the normal loss of a view, and their gradients, bit for bit alone and among others (values of
+    many magnitudes, so that another order of the sums shows)."""
+    import torch
+    import paper_2605_31419_gb300 as ts
+    sizes = [(640, 480)] * 4 + [(317, 239)] + [(640, 480)] * 4
+
+    def run(views, tensors):
+        r = ts.Rasterizer(np.array([[100.0, 100.0, W / 2, H / 2, W, H] for W, H in views]), 0,
+                          ts.ts_default_params(flags=ts.TS_FLAG_NORMALS))
+        C, D, N, tC, tD, tN = (torch.cat([t[i] for t in tensors]) for i in range(6))
+        r.color.copy_(C), r.depth.copy_(D), r.normal.copy_(N)
+        loss, dC, dD = (t.clone() for t in r.l1_loss(tC, tD))
+        nloss, dN = r.normal_loss(tN)[:2]
+        return [t.cpu() for t in (loss, dC, dD, nloss, dN)]
+
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    rnd = lambda n: torch.exp(3 * torch.randn(n, generator=gen, device="cuda"))  # noqa: E731
+    data = [[rnd(k * W * H) for k in (3, 1, 3, 3, 1, 3)] for W, H in sizes]
+    whole = run(sizes, data)
+    off = np.cumsum([0] + [W * H for W, H in sizes])
+    for v in range(len(sizes)):
+        alone = run([sizes[v]], [data[v]])
+        a, b = off[v], off[v + 1]
+        parts = (whole[0][v:v + 1], whole[1][3 * a:3 * b], whole[2][a:b], whole[3][v:v + 1], whole[4][3 * a:3 * b])
+        assert all(torch.equal(x, y) for x, y in zip(alone, parts)), v
