@@ -118,6 +118,18 @@ __device__ __forceinline__ void stage_view(const PBArgs& a, float* d, int v) {
   for (int i = 0; i < 3; ++i) d[13 + i] = a.poses[v].t[i];
 }
 
+// The same values from global memory, four 16-byte loads.
+__device__ __forceinline__ void load_view(const PBArgs& a, float* d, int v) {
+  static_assert(sizeof(TsView) % 16 == 0 && sizeof(ts_pose) == 48, "16-byte loads of a view and its pose");
+  const float4 k = *reinterpret_cast<const float4*>(a.views + v);
+  d[0] = k.x; d[1] = k.y; d[2] = k.z; d[3] = k.w;
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    const float4 q = reinterpret_cast<const float4*>(a.poses + v)[i];
+    d[4 + 4 * i] = q.x; d[5 + 4 * i] = q.y; d[6 + 4 * i] = q.z; d[7 + 4 * i] = q.w;
+  }
+}
+
 // What the chain rule of one visible (view, face) gives: the world-space vertex-position
 // gradients, the pose terms, and the slot's colour, opacity and sigma_F sums passed through.
 struct SlotTerms {
@@ -283,8 +295,9 @@ __host__ __device__ constexpr int pbwd_warp_floats(int V, int faces) {
   return (32 * TS_GRAD_WORDS + 32 * PB_RS + faces * (PB_FS + PB_RS) + V * PB_PS + (faces * V + 1) / 2 + 3) & ~3;
 }
 
-// With map gradients: FPW faces per warp iteration, 32 / FPW lanes looking up each face's views.
-template <int FPW>
+// With map gradients: FPW faces per warp iteration, 32 / FPW lanes looking up each face's views.  STAGED: the views'
+// constants in shared memory, else each entry loads its view's.
+template <int FPW, bool STAGED>
 __global__ void __launch_bounds__(PB_T, 4) k_pbwd_map(PBArgs a) {
   constexpr int LPF = 32 / FPW, ROUNDS = (3 * FPW + 31) / 32;
   extern __shared__ __align__(16) float pv[];
@@ -299,7 +312,8 @@ __global__ void __launch_bounds__(PB_T, 4) k_pbwd_map(PBArgs a) {
   float* my = fsum + FPW * PB_RS;
   uint16_t* list = reinterpret_cast<uint16_t*>(my + a.V * PB_PS);  // face * 256 + view
   float* slot_here = slots + lane * TS_GRAD_WORDS;
-  for (int v = threadIdx.x; v < a.V; v += PB_T) stage_view(a, views + v * VP, v);
+  if (STAGED)
+    for (int v = threadIdx.x; v < a.V; v += PB_T) stage_view(a, views + v * VP, v);
   for (int i = lane; i < a.V * PB_PS; i += 32) my[i] = 0.f;
   __syncthreads();
   const bool indexed = h->faces != nullptr;
@@ -358,7 +372,13 @@ __global__ void __launch_bounds__(PB_T, 4) k_pbwd_map(PBArgs a) {
       float tau[6];
       if (act) {
         SlotTerms t;
-        chain_terms(a, v, m0 + fe, sl, fdat + fe * PB_FS, views + v * VP, t);
+        if constexpr (STAGED) {
+          chain_terms(a, v, m0 + fe, sl, fdat + fe * PB_FS, views + v * VP, t);
+        } else {
+          float vp[16];
+          load_view(a, vp, v);
+          chain_terms(a, v, m0 + fe, sl, fdat + fe * PB_FS, vp, t);
+        }
         float* row = rows + lane * PB_RS;
 #pragma unroll
         for (int i = 0; i < 9; ++i) row[i] = t.out[i];
@@ -581,27 +601,29 @@ __global__ void __launch_bounds__(256) k_pose_reduce(const float* __restrict__ p
 constexpr long long MAP_BLOCKS = 608;    // 4 resident blocks on 152 SMs
 constexpr long long POSE_BLOCKS = 2432;  // most blocks per view of the form without map gradients
 int ts_pose_blocks(long long M) {        // the most either form uses
-  return (int)std::max<long long>(1, std::min<long long>((M + 31) / 32, POSE_BLOCKS));
+  return (int)std::max<long long>(1, std::min<long long>((M + 7) / 8, POSE_BLOCKS));
 }
 
 namespace {
 // Shared memory of a block of the form with map gradients, and whether four such blocks fit on a
-// multiprocessor (228 KB, of which each block takes 1 KB more): up to 23 views of 32 faces, 68 of 16.
+// multiprocessor (228 KB, of which each block takes 1 KB more): up to 23 views of 32 faces, 68 of 16, 110 of 8, all of
+// 2.  Four faces and fewer leave the views in global memory: a batch then holds many views of few faces.
+constexpr bool pbwd_staged(int faces) { return faces > 4; }
 constexpr int pbwd_smem(int V, int faces) {
-  return (PB_WARPS * pbwd_warp_floats(V, faces) + V * VP) * (int)sizeof(float);
+  return (PB_WARPS * pbwd_warp_floats(V, faces) + (pbwd_staged(faces) ? V * VP : 0)) * (int)sizeof(float);
 }
 constexpr bool pbwd_four_blocks(int V, int faces) { return 4 * (pbwd_smem(V, faces) + 1024) <= 228 * 1024; }
 static_assert(pbwd_four_blocks(23, 32) && !pbwd_four_blocks(65, 32) && pbwd_four_blocks(68, 16) &&
-                  !pbwd_four_blocks(129, 16) && TS_MAX_VIEWS <= 256,
+                  !pbwd_four_blocks(129, 16) && pbwd_four_blocks(TS_MAX_VIEWS, 2) && TS_MAX_VIEWS <= 256,
               "a lane looks up at most 64 views of its face, an entry holds its view in 8 bits");
 
 template <int FPW>
 cudaError_t launch_pbwd_map(const PBArgs& a, cudaStream_t s) {
-  const int smem = pbwd_smem(a.V, FPW);  // at most 90.6 KB (256 views)
-  const cudaError_t e = ts_smem_limit((const void*)k_pbwd_map<FPW>, smem);
+  const int smem = pbwd_smem(a.V, FPW);  // at most 56 KB
+  const cudaError_t e = ts_smem_limit((const void*)k_pbwd_map<FPW, pbwd_staged(FPW)>, smem);
   if (e != cudaSuccess) return e;
   const long long want = (a.M + PB_WARPS * FPW - 1) / (PB_WARPS * FPW);
-  k_pbwd_map<FPW><<<(unsigned)std::min(want, MAP_BLOCKS), PB_T, smem, s>>>(a);
+  k_pbwd_map<FPW, pbwd_staged(FPW)><<<(unsigned)std::min(want, MAP_BLOCKS), PB_T, smem, s>>>(a);
   return cudaGetLastError();
 }
 }  // namespace
@@ -641,14 +663,21 @@ cudaError_t ts_launch_project_bwd(const TsPlanImpl* p, const TsWs& w, const ts_m
     k_pbwd_pose<<<dim3((unsigned)nb, (unsigned)p->V), PB_T, smem, s>>>(a);
     return cudaGetLastError();
   }
-  // 32 faces a warp once every warp of the grid has some, fewer of smaller maps and where more views would
-  // leave room for three blocks on an SM instead of four (and the grid a second wave): 300k faces take 141 us at
-  // 23 views of 32 faces and 150 of 16, 332 at 64 views of 16 and 346 of 8.  Above 110 views even 8 faces leave three.
-  const int most = pbwd_four_blocks(p->V, 32) ? 32 : (pbwd_four_blocks(p->V, 16) ? 16 : 8);
-  const int faces = std::min(most, p->M > MAP_BLOCKS * PB_WARPS * 16 ? 32 : (p->M > MAP_BLOCKS * PB_WARPS * 8 ? 16 : 8));
-  if (faces == 32) return launch_pbwd_map<32>(a, s);
-  if (faces == 16) return launch_pbwd_map<16>(a, s);
-  return launch_pbwd_map<8>(a, s);
+  // As many faces a warp as leave every warp of the grid some, and four blocks room on a multiprocessor (fewer leave the
+  // grid a second wave); above 110 views two, which fill batches then.  300k faces take 141 us at 23 views of 32 faces
+  // and 150 of 16, 332 at 64 views of 16 and 346 of 8; 30k faces 101 us at 128 views of 8 faces, 81 of 4 and 83 of 2, 10k
+  // at 200 views 99, 68 and 59; 2000 faces of 64 views 25 us of 8, 18 of 4 and 13 of 2, 10k of 16 views 11 of 8 and 13
+  // of 4.
+  int faces = 32;
+  while (faces > 2 && (!pbwd_four_blocks(p->V, std::max(faces, 8)) || p->M <= MAP_BLOCKS * PB_WARPS * (faces / 2)))
+    faces /= 2;
+  switch (faces) {
+    case 32: return launch_pbwd_map<32>(a, s);
+    case 16: return launch_pbwd_map<16>(a, s);
+    case 8: return launch_pbwd_map<8>(a, s);
+    case 4: return launch_pbwd_map<4>(a, s);
+    default: return launch_pbwd_map<2>(a, s);
+  }
 }
 
 cudaError_t ts_launch_pose_reduce(const TsPlanImpl* p, const TsWs& w, float* dtau, cudaStream_t s) {
