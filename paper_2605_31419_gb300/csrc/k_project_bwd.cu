@@ -655,9 +655,12 @@ cudaError_t ts_launch_project_bwd(const TsPlanImpl* p, const TsWs& w, const ts_m
   bool map = a.dst_sigma != nullptr;
   for (int c = 0; c < 7; ++c) map = map || a.dst[c] != nullptr;
   if (!map) {
-    // faces per warp: enough that full batches dominate, once every SM has warps
+    // faces per warp: enough that full batches dominate, once every SM has warps.  One view is fastest with few (150k
+    // faces: 6.4 us at 128, 8.3 at 256, 12.5 at 512), many views with many (64: 191, 162 and 148); at 128, 256 and 512
+    // 7 views of 40k take 9.2, 10.6 and 14.2, 64 views 57, 51 and 53, 7 views of 65k 14.2, 11.7 and 15.1, 64 86, 77 and 74.
     const long long least = (p->M + PB_WARPS * POSE_BLOCKS - 1) / (PB_WARPS * POSE_BLOCKS);
-    a.unit = p->M >= (1 << 16) ? (int)std::max<long long>(512, (least + 31) / 32 * 32) : (p->M >= (1 << 14) ? 128 : 32);
+    a.unit = p->M >= (1 << 16) ? (int)std::max<long long>(512, (least + 31) / 32 * 32)
+                               : (p->M >= 3 << 14 ? 256 : (p->M >= 1 << 14 ? 128 : 32));
     const long long nb = (p->M + PB_WARPS * a.unit - 1) / (PB_WARPS * a.unit);
     const int smem = PB_T * (TS_GRAD_WORDS + PB_FS) * (int)sizeof(float);  // 26 KB
     k_pbwd_pose<<<dim3((unsigned)nb, (unsigned)p->V), PB_T, smem, s>>>(a);

@@ -219,6 +219,7 @@ def _padded(sc, n_faces, indexed):
     (12_002, 2, False), (12_002, 110, True), (9_729, 111, False),   # 8 up to 110 views
     (19_457, 2, False), (19_500, 68, True), (19_457, 69, False),    # 16 up to 68
     (38_913, 1, True), (38_950, 23, False), (38_913, 24, True),     # 32 up to 23
+    (49_152, 2, False),                                             # 256 faces a warp, pose only
     (65_601, 1, False), (65_600, 3, True), (140_003, 2, False),     # 65 and more face blocks; 512 faces a warp, pose only
 ])
 def test_padded_maps(n_faces, n_views, indexed):
