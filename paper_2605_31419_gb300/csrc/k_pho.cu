@@ -411,11 +411,11 @@ Taps gaussian_taps() {
 }
 
 // Output rows per strip, 16 k - 10 for k steps: long strips recompute less at their ends (k = 16: 4 %), but
-// a small batch is cut into at least four waves of two CTAs on 152 SMs, down to k = 2.
+// a small batch is cut into at least four waves of two CTAs on every SM, down to k = 2.
 int strip_rows(const TsView* views, int V) {
   long long total = 0;  // rows of all strips and channels
   for (int v = 0; v < V; ++v) total += 3ll * ((views[v].W + OW - 1) / OW) * views[v].H;
-  const long long k = (total / 1216 + 2 * RAD + RB - 1) / RB;
+  const long long k = (total / (8 * TS_SMS) + 2 * RAD + RB - 1) / RB;
   return RB * (int)std::max(2ll, std::min(16ll, k)) - 2 * RAD;
 }
 

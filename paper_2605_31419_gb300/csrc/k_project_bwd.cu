@@ -598,9 +598,9 @@ __global__ void __launch_bounds__(256) k_pose_reduce(const float* __restrict__ p
 // The faces per warp and block fix the partial sums of the pose gradient and so its summation order: without
 // map gradients they depend on the map's size alone, so that a tracked view's dtau is the same alone and
 // among others, and on every GPU.
-constexpr long long MAP_BLOCKS = 608;    // 4 resident blocks on 152 SMs
-constexpr long long POSE_BLOCKS = 2432;  // most blocks per view of the form without map gradients
-int ts_pose_blocks(long long M) {        // the most either form uses
+constexpr long long MAP_BLOCKS = 4 * TS_SMS;    // the resident blocks
+constexpr long long POSE_BLOCKS = 16 * TS_SMS;  // most blocks per view of the form without map gradients
+int ts_pose_blocks(long long M) {               // the most either form uses
   return (int)std::max<long long>(1, std::min<long long>((M + 7) / 8, POSE_BLOCKS));
 }
 

@@ -143,10 +143,19 @@ ts_status ts_plan_init(ts_plan* plan, const ts_camera* cams, int32_t n_views, in
   if (cap >= ((int64_t)1 << 32) - 4096) return TS_ERR_INVALID_ARG;
   p->cap = cap;
   p->max_view_tiles = max_tiles;
-  // faces per binning block: the fewest, from 1024 by powers of two, that leave at most 456 blocks (three on
-  // each of 152 multiprocessors); a larger problem takes the most, which keeps the count matrix small
-  p->bin_faces = 1024;
-  while (p->bin_faces < TS_BIN_FACES && n_views * ((n_faces + p->bin_faces - 1) / p->bin_faces) > 456) p->bin_faces *= 2;
+  // faces per binning block, 1024 to 8192: what the rounds of blocks cost (three blocks on each of 152 multiprocessors
+  // at a time; a block costs its faces, and its tiles and start some thousand faces more).  With 8192 wherever fewer
+  // leave more than one round, 200 views of 20k faces had two rounds, the second a third full: counts and places
+  // 65 -> 48 us with 4096 (and the counts' own walk of small rectangles).
+  int64_t least = INT64_MAX;
+  for (int64_t f = 1024; f <= TS_BIN_FACES; f *= 2) {
+    const int64_t blocks = n_views * ((n_faces + f - 1) / f), rounds = (blocks + 3 * TS_SMS - 1) / (3 * TS_SMS);
+    const int64_t cost = rounds * (f + 1024 + max_tiles);
+    if (cost <= least) {
+      least = cost;
+      p->bin_faces = f;
+    }
+  }
   p->bin_blocks = max_tiles <= TS_BIN_MAX_TILES ? std::max<int64_t>(1, (n_faces + p->bin_faces - 1) / p->bin_faces) : 0;
   p->bin_shift = p->bin_blocks <= TS_BIN_FEW && toff >= 16384 ? 8 : 5;
   const int64_t scan_items = p->bin_blocks ? int64_t(1) << p->bin_shift : TS_SCAN_ITEMS;

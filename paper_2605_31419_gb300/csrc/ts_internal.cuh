@@ -14,6 +14,8 @@
 #define TS_PLAN_MAGIC 0x54535031u  // "TSP1"
 #define TS_REC_WORDS 32            // 128-byte record, a multiple of 16 B for cp.async.bulk
 #define TS_GRAD_WORDS 32           // per-(view, face) gradient slot
+#define TS_SMS 152                 // multiprocessors the splits are laid out for: a plan, made on the host, and the
+                                   // order of its sums do not depend on the device in use
 #define TS_SCAN_ITEMS 4096         // items per scan block (1024 threads x 4)
 #define TS_BIN_FACES 8192          // most faces per block of the shared-memory tile counts
 #define TS_BIN_FEW 8               // rows of the count matrix up to which a thread sums a tile's column
