@@ -390,16 +390,21 @@ cudaError_t ts_launch_project(const TsPlanImpl* p, const TsWs& w, const ts_map* 
   a.count = w.count;
   a.hdr = w.hdr;
   a.ctr = w.ctr;
-  // views per block: up to PJ_VIEWS, so that a map is read once per block of views and full warps of faces
-  // collect, but fewer where that leaves over half of the GPU's places (six blocks per multiprocessor) empty: 8 against 4
-  // measured 147 against 161 us at 20 views of 300k faces, 280 against 294 at 9 of 2M, 10.9 against 9.3 at 7
-  // of 40k (one partly filled wave there beats a full one and a bit: 784 blocks 7.7 us, 1568 9.9).  Steps per warp likewise: up to PJ_STEPS once every place has eight blocks to run.
+  // views per block: up to PJ_VIEWS, so that a map is read once per block of views and full warps of faces collect, but
+  // fewer where that leaves over half of the GPU's places (six blocks per multiprocessor) empty: 8 against 4 measured
+  // 147 against 161 us at 20 views of 300k faces, 280 against 294 at 9 of 2M, 10.9 against 9.3 at 7 of 40k (one partly
+  // filled wave there beats a full one and a bit: 784 blocks 7.7 us, 1568 9.9).  Steps per warp: up to PJ_STEPS once
+  // every place has eight blocks to run.  One view leaves a step a quarter of a warp of faces to project, and takes up
+  // to three of them as soon as the places are full: 1, 2, 3 and 4 steps 12.0, 10.2, 9.5 and 9.3 us for 300k faces, 38,
+  // 29, 26 and 26 for 1M, 73, 53, 49 and 48 for 2M.
   const long long places = 6LL * ts_sm_count(), fg = (p->M + 31) / 32;
   int per = std::min(p->V, PJ_VIEWS);
   auto blocks_of = [&](int n) { return (fg + PJ_T / 32 - 1) / (PJ_T / 32) * ((p->V + n - 1) / n); };
   while (per > 1 && 2 * blocks_of(per) < places) per = (per + 1) / 2;
   const long long vb = (p->V + per - 1) / per;
-  const int groups = (int)std::max(1LL, std::min<long long>(PJ_STEPS / per, blocks_of(per) / (8 * places)));
+  const long long steps = p->V == 1 ? std::min(3LL, (blocks_of(1) + places - 1) / places)
+                                    : std::min<long long>(PJ_STEPS / per, blocks_of(per) / (8 * places));
+  const int groups = (int)std::max(1LL, steps);
   const long long face_blocks = (fg + (long long)groups * (PJ_T / 32) - 1) / ((long long)groups * (PJ_T / 32));
   k_project<<<dim3((unsigned)face_blocks, (unsigned)vb), PJ_T, 0, s>>>(a, per, groups);
   return cudaGetLastError();
