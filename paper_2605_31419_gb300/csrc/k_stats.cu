@@ -27,11 +27,12 @@ struct StatsArgs {
   uint32_t* n_visible;
 };
 
-// grid (ceil(M / 1024), V): 1024 faces of view v per block, 256 at a time; a warp covers 32 faces of one view,
+// grid (ceil(M / (256 ST_PER)), V): 256 ST_PER faces of view v per block, 256 at a time; a warp covers 32 faces of one view,
 // so its ballot is one word of the view's bitset.  Bound by its 12 to 20 bytes per (view, face) and the
 // visible records' sectors.  The visible counts are summed per block: one add per warp queued 9,375 adds on
-// each view's address (8 views of 300k faces: 58 -> 23 us).
-constexpr int ST_PER = 4;
+// each view's address (8 views of 300k faces: 58 -> 23 us).  Maps that leave most multiprocessors without a block
+// take a face per thread (ST_PER 1).
+template <int ST_PER>
 __global__ void __launch_bounds__(ST_T) k_face_stats(StatsArgs a) {
   __shared__ unsigned red[ST_T / 32];
   const int v = blockIdx.y;
@@ -137,7 +138,11 @@ cudaError_t ts_launch_face_stats(const TsPlanImpl* p, const TsWs& w, uint32_t* c
   a.area = area;
   a.visible = visible;
   a.n_visible = n_visible;
-  k_face_stats<<<dim3((unsigned)((p->M + ST_PER * ST_T - 1) / (ST_PER * ST_T)), (unsigned)p->V), ST_T, 0, s>>>(a);
+  const long long blocks = (p->M + 4 * ST_T - 1) / (4 * ST_T);
+  if (blocks * p->V >= TS_SMS)
+    k_face_stats<4><<<dim3((unsigned)blocks, (unsigned)p->V), ST_T, 0, s>>>(a);
+  else
+    k_face_stats<1><<<dim3((unsigned)((p->M + ST_T - 1) / ST_T), (unsigned)p->V), ST_T, 0, s>>>(a);
   return cudaGetLastError();
 }
 
