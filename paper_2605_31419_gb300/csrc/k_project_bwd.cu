@@ -53,6 +53,7 @@ struct PBArgs {
   bool min_opacity;  // o_F = min of the vertex opacities: dL/do_F to the first minimal vertex
   float* part;       // per (view, block): the pose sums
   int part_stride;   // blocks the workspace has room for
+  uint32_t* part_n;  // receives the blocks used
   int unit;          // without map gradients: consecutive faces per warp (a multiple of 32)
 };
 
@@ -492,7 +493,7 @@ __global__ void __launch_bounds__(PB_T, 4) k_pbwd_map(PBArgs a) {
     for (int w = 0; w < PB_WARPS; ++w) sum += pv[(size_t)w * per_warp + (my - slots) + v * PB_PS + i];
     a.part[((long long)v * a.part_stride + blockIdx.x) * 6 + i] = sum;
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) a.hdr->pose_blocks = gridDim.x;
+  if (blockIdx.x == 0 && threadIdx.x == 0) *a.part_n = gridDim.x;
 }
 
 // Without map gradients: blocks (part of the faces, view), a.unit consecutive faces per warp.
@@ -566,14 +567,14 @@ __global__ void __launch_bounds__(PB_T, 4) k_pbwd_pose(PBArgs a) {
     for (int w = 0; w < PB_WARPS; ++w) sum += red[w][threadIdx.x];
     a.part[((long long)v * a.part_stride + blockIdx.x) * 6 + threadIdx.x] = sum;
   }
-  if (blockIdx.x == 0 && v == 0 && threadIdx.x == 0) a.hdr->pose_blocks = gridDim.x;
+  if (blockIdx.x == 0 && v == 0 && threadIdx.x == 0) *a.part_n = gridDim.x;
 }
 
 __global__ void __launch_bounds__(256) k_pose_reduce(const float* __restrict__ part, int part_stride,
-                                                     const TsDevHeader* __restrict__ hdr, float* dtau) {
+                                                     const uint32_t* __restrict__ part_n, float* dtau) {
   __shared__ float red[256][6];
   const int v = blockIdx.x;
-  const int nblocks = min((int)hdr->pose_blocks, part_stride);  // written by the backward
+  const int nblocks = (int)min(*part_n, (uint32_t)part_stride);  // written by the backward
   float s[6] = {0, 0, 0, 0, 0, 0};
   for (int b = threadIdx.x; b < nblocks; b += 256) {
     const float* p = part + ((long long)v * part_stride + b) * 6;
@@ -630,7 +631,7 @@ cudaError_t launch_pbwd_map(const PBArgs& a, cudaStream_t s) {
 
 cudaError_t ts_launch_project_bwd(const TsPlanImpl* p, const TsWs& w, const ts_map_grad* g, cudaStream_t s) {
   if (p->M == 0) {
-    return cudaMemsetAsync(w.pose, 0, (size_t)p->V * p->n_pose_blocks * 6 * 4, s);
+    return cudaMemsetAsync(w.pose_n, 0, 4, s);  // no partials
   }
   PBArgs a;
   a.views = w.views;
@@ -651,6 +652,7 @@ cudaError_t ts_launch_project_bwd(const TsPlanImpl* p, const TsWs& w, const ts_m
   a.min_opacity = p->min_opacity;
   a.part = w.pose;
   a.part_stride = (int)p->n_pose_blocks;
+  a.part_n = w.pose_n;
   a.unit = 0;
   bool map = a.dst_sigma != nullptr;
   for (int c = 0; c < 7; ++c) map = map || a.dst[c] != nullptr;
@@ -684,6 +686,6 @@ cudaError_t ts_launch_project_bwd(const TsPlanImpl* p, const TsWs& w, const ts_m
 }
 
 cudaError_t ts_launch_pose_reduce(const TsPlanImpl* p, const TsWs& w, float* dtau, cudaStream_t s) {
-  k_pose_reduce<<<p->V, 256, 0, s>>>(w.pose, (int)p->n_pose_blocks, w.hdr, dtau);
+  k_pose_reduce<<<p->V, 256, 0, s>>>(w.pose, (int)p->n_pose_blocks, w.pose_n, dtau);
   return cudaGetLastError();
 }

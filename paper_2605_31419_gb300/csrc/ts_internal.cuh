@@ -83,9 +83,8 @@ struct TsDevHeader {
   long long n_vertices;
   unsigned int tile_counter;  // work counter of the persistent raster launches
   unsigned int n_large;       // tiles listed for the CTA-wide pair sort
-  unsigned int pose_blocks;   // per-view pose partials the last backward wrote
   unsigned int pair_wraps;    // binning: 2^32s of pairs that the 32-bit sums of groups of tiles dropped
-  unsigned int pad[10];
+  unsigned int pad[11];
 };
 
 struct TsPlanImpl {
@@ -136,6 +135,7 @@ struct TsWs {
   int32_t* nlast;
   float* grad;
   float* pose;
+  uint32_t* pose_n;  // the per-view pose partials the plan's last backward wrote
   float* loss;
   float* pho;  // per (view, channel, strip): L1, SSIM and depth partial sums of the photometric loss
   float* equi;  // per block of 256 faces: partial sums of the equilateral regulariser
@@ -170,6 +170,7 @@ inline TsWs ts_ws(const TsPlanImpl* p, void* ws) {
   w.nlast = (int32_t*)(b + p->o_nlast);
   w.grad = p->fwd_only ? nullptr : (float*)(b + p->o_grad);
   w.pose = (float*)(b + p->o_pose);
+  w.pose_n = (uint32_t*)(w.pose + (size_t)p->V * p->n_pose_blocks * 6);
   w.loss = (float*)(b + p->o_loss);
   w.pho = (float*)(b + p->o_pho);
   w.equi = (float*)(b + p->o_equi);

@@ -352,3 +352,30 @@ def test_losses_do_not_depend_on_the_batch():
         a, b = off[v], off[v + 1]
         parts = (whole[0][v:v + 1], whole[1][3 * a:3 * b], whole[2][a:b], whole[3][v:v + 1], whole[4][3 * a:3 * b])
         assert all(torch.equal(x, y) for x, y in zip(alone, parts)), v
+
+
+def test_pose_gradient_after_another_plans_step():
+    """The pose partials are the plan's own: a small plan's step on the same workspace, which ends before the large
+    plan's partials, leaves the large plan's pose gradient as it is."""
+    import torch
+    import paper_2605_31419_gb300 as ts
+    plans = []
+    for n, V in ((3000, 2), (40, 1)):
+        sc = random_triangles_scene(seed=n, n_faces=n, W=64, H=48, f=60.0)
+        poses = np.repeat(sc.poses[:1], V, axis=0).copy()
+        poses[:, 9] = 0.1 * np.arange(V)
+        r = ts.Rasterizer(np.repeat(sc.cams[:1], V, axis=0), n, pair_capacity=200 * n)
+        plans.append((r, ts.Map.from_numpy(sc.pos, sc.col, sc.opa), ts.poses_tensor(poses)))
+    large, small = plans
+    assert small[0].ws_bytes < 3000 * 2 * 128  # inside the large plan's records
+    small[0].ws = large[0].ws
+
+    def step(r, m, poses):
+        r.forward(m, poses)
+        r.backward(torch.ones_like(r.color), torch.ones_like(r.depth), None, m.zeros_like())
+
+    step(*large)
+    want = large[0].pose_grad().clone()
+    step(*small)
+    small[0].pose_grad()
+    assert float(want.abs().max()) > 0 and torch.equal(large[0].pose_grad(), want)
