@@ -24,9 +24,9 @@
 //
 // Backward: per pixel, back to front from that position: recover T_n = T_{n+1} / (1 - alpha_n),
 // keep the suffix sum S of later contributions (including the background term), form
-// dL/dalpha_n = T_n v_n - S / (1 - alpha_n) with v_n = gC . c_n + gD z_n + gA, and chain into 23
-// per-face sums (barycentric-weighted gradients of the edge, colour and depth interpolants, of
-// o_F, and the contribution count).  The forward stores, per sorted pair and warp, the 32-bit
+// dL/dalpha_n = T_n v_n - S / (1 - alpha_n) with v_n = gC . c_n + gD z_n + gA, and chain into 22
+// per-face sums (barycentric-weighted gradients of the edge, colour and depth interpolants, and of o_F;
+// 26 with the side array: the face's normal and sigma_F).  The forward stores, per sorted pair and warp, the 32-bit
 // mask of the warp's pixels that blended the face; the backward numbers those (face, pixel)
 // entries back to front (a warp-wide scan of the masks' bit counts) and processes them 32 at a
 // time, one per lane, so that no lane idles on a pixel the face does not cover.  Entries of
@@ -38,13 +38,17 @@
 // window), backward of 64 tracking views 780 -> 716.  Every
 // per-face sum is over products of two per-entry factors: one of seven weighted gradients times one of
 // three barycentrics (the gradient of o_F alone).  Each lane writes its entry's factors to a ring row in
-// shared memory; then the 8 lanes of each quarter warp walk 8 consecutive rows, lane a accumulating
-// factor a times the three barycentrics, and add them into the face's accumulator with one four-word
-// reduction per lane at the rows that end a face's entries or the quarter, which one ballot marks: 8
-// unrolled steps a batch.  The reductions themselves cost nothing measurable; the instructions do.  (A loop
-// over the faces' runs, one word per lane: the backward of 64 tracking views 1034 -> 918 us; testing every
-// row's sums for zero and the slot in 64 bits: fused step 1321 -> 1244 us for the 12-view window, backward
-// of 6 mapping views 172 -> 164.)
+// shared memory; then the 8 lanes of each quarter warp walk 8 rows, lane a accumulating factor a times the
+// three barycentrics, and add them into the face's accumulator with one four-word reduction per lane where a
+// face's run of rows ends: 8 unrolled steps a batch.  Odd quarters walk their rows the other way, so that a run
+// across two quarters is left over in both and added once, and so is one from the first quarter into the last.
+// (A reduction at every quarter's end gave the slot of a large face up to four times the additions, and its sums
+// twice the rounding error: the colour gradients of two views of large faces were 1.26 times as far from their
+// 64-bit values as those of a sum per batch, now 1.01.  Putting the quarters together costs 2 to 3 % of a step:
+// 1769 -> 1810 us for the 20-view room, 1846 -> 1892 for the 12-view window.)  The reductions themselves cost
+// nothing measurable; the instructions do.  (A loop over the faces' runs, one word per lane: the backward of 64
+// tracking views 1034 -> 918 us; testing every row's sums for zero and the slot in 64 bits: fused step 1321 ->
+// 1244 us for the 12-view window, backward of 6 mapping views 172 -> 164.)
 //
 // Launch forms: one CTA per tile, or persistent CTAs (as many as fit on the GPU) that take tiles
 // from a device counter.  The fused L1 step (ts_render_step_l1) runs a tile's forward, its loss
@@ -557,7 +561,8 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
     float2* pst = reinterpret_cast<float2*>(wbase + Ring<AUX>::WORDS * 4);  // per pixel lane: (T, S)
     pst[lane] = make_float2(T, Sacc);
     __syncwarp();  // read by other lanes; a stage that is still staged has no barrier before its first batch
-    float* row_here = ring + lane * EW + (lane >> 3) * 8;                      // this lane's entry's row
+    // this lane's entry's row (odd quarters' in falling order)
+    float* row_here = ring + (lane ^ ((lane & 8) ? 7 : 0)) * EW + (lane >> 3) * 8;
     const float* row_sum = ring + (lane >> 3) * (8 * EW + 8);                  // its quarter warp's first row
     const int fa = lane & 7;                                                   // the factor it sums
     const uint32_t vm32 = (uint32_t)min(a.VM, 0xffffffffll);                   // slots
@@ -735,12 +740,26 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
             row[0] = row[1] = row[2] = make_float4(0.f, 0.f, 0.f, 0.f);
             if constexpr (AUX) row[3] = make_float4(0.f, 0.f, 0.f, 0.f);
           }
-          // the batch's faces are runs of consecutive entries: rows that end one
+          // the batch's faces are runs of consecutive entries.  Even quarters take their rows upwards and add a run's
+          // sums at its last row, odd quarters downwards (their rows lie in that order) and at its first: a run that
+          // crosses from an even quarter into the next is then left in both, and put together
           const int jnext = __shfl_down_sync(FULL, j, 1);
-          // and, so that every quarter's sums are added, the last active row of each
-          const unsigned ends = __ballot_sync(FULL, act && (lane == ne - 1 || j != jnext || (lane & 7) == 7)) >> (lane & 24);
+          const unsigned ends = __ballot_sync(FULL, act && (lane == ne - 1 || j != jnext));
+          const unsigned rows = (2u << (ne - 1)) - 1u;  // the active ones
+          const unsigned firsts = ((ends << 1) | 1u) & rows;
+          const unsigned stop = (lane & 8) ? __brev(firsts) >> (24 - (lane & 24)) : ends >> (lane & 24);
+          const bool cross = ((~ends & (rows >> 1)) >> (lane & 16)) & 0x80u;  // into this lane's pair's odd quarter
           __syncwarp();
           float s0 = 0.f, s1 = 0.f, s2 = 0.f, s3 = 0.f;
+          uint32_t sl = 0u;
+          auto to_slot = [&]() {
+            if (fa == 7) s1 = s2 = 0.f;
+            if (sl < vm32) {
+              red_add_v4(a.grad + (size_t)sl * TS_GRAD_WORDS + 4 * fa, s0, s1, s2, s3);
+            } else {
+              atomicOr(&a.hdr->error_bits, TS_ERRBIT_BOUNDS);
+            }
+          };
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
             const float4 l = *reinterpret_cast<const float4*>(row_sum + i * EW);
@@ -749,17 +768,27 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
             s1 = fmaf(f, l.y, s1);
             s2 = fmaf(f, l.z, s2);
             if (AUX && fa < 4) s3 += row_sum[i * EW + 12 + fa];
-            if ((ends >> i) & 1u) {
-              if (fa == 7) s1 = s2 = 0.f;
-              const uint32_t sl = __float_as_uint(l.w);
-              if (sl < vm32) {
-                red_add_v4(a.grad + (size_t)sl * TS_GRAD_WORDS + 4 * fa, s0, s1, s2, s3);
-              } else {
-                atomicOr(&a.hdr->error_bits, TS_ERRBIT_BOUNDS);
-              }
+            sl = __float_as_uint(l.w);
+            if (i < 7 && ((stop >> i) & 1u)) {
+              to_slot();
               s0 = s1 = s2 = s3 = 0.f;
             }
           }
+          const float t0 = __shfl_xor_sync(FULL, s0, 8), t1 = __shfl_xor_sync(FULL, s1, 8);
+          const float t2 = __shfl_xor_sync(FULL, s2, 8), t3 = AUX ? __shfl_xor_sync(FULL, s3, 8) : 0.f;
+          s0 += cross ? t0 : 0.f;
+          s1 += cross ? t1 : 0.f;
+          s2 += cross ? t2 : 0.f;
+          if (AUX) s3 += cross ? t3 : 0.f;
+          bool whole = cross ? !(lane & 8) : ((stop >> 7) & 1u) != 0u;
+          if (ne > 24 && !(ends & 0x00ffff80u)) {  // uniform: one run from the first quarter into the last
+            s0 += __shfl_xor_sync(FULL, s0, 16);
+            s1 += __shfl_xor_sync(FULL, s1, 16);
+            s2 += __shfl_xor_sync(FULL, s2, 16);
+            if (AUX) s3 += __shfl_xor_sync(FULL, s3, 16);
+            whole = lane < 8;
+          }
+          if (whole) to_slot();
           __syncwarp();
         }
       }

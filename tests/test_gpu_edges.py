@@ -379,3 +379,38 @@ def test_pose_gradient_after_another_plans_step():
     step(*small)
     small[0].pose_grad()
     assert float(want.abs().max()) > 0 and torch.equal(large[0].pose_grad(), want)
+
+
+@pytest.mark.parametrize("normals", [False, True])
+def test_large_faces_are_summed_in_few_additions(oracle, normals):
+    """Eight faces that cover 2048 sub-blocks of 32 pixels in full: each sub-block adds a face's 32 terms to its
+    slot once.  n FP32 additions of like terms in any order leave a sum off by about sqrt(n / 3) roundings (each
+    2^-23 0.72 / sqrt(12) of it on average), 6.5e-7 for 2048 and 1.3e-6 for four times as many; the error over the
+    72 colour sums has to lie below what twice as many would leave."""
+    import torch
+    import paper_2605_31419_gb300 as ts
+    from oracle.oracle import SceneArrays
+    rng = np.random.default_rng(2)
+    W = H = 256
+    f, M = 200.0, 8
+    z = np.linspace(1.0, 2.0, M)
+    tri = np.array([[-300.0, -300.0], [1000.0, -300.0], [-300.0, 1000.0]]) + rng.uniform(-40, 40, (M, 3, 2))
+    pos = np.concatenate([(tri - [W / 2, H / 2]) * (z / f)[:, None, None], np.repeat(z[:, None, None], 3, 1)], 2)
+    sc = Scene(pos.reshape(-1, 3).astype(np.float32), rng.uniform(0.2, 0.8, (3 * M, 3)).astype(np.float32),
+               rng.uniform(0.1, 0.3, 3 * M).astype(np.float32), None, np.array([[f, f, W / 2, H / 2, W, H]]),
+               np.array([[1, 0, 0, 0, 1, 0, 0, 0, 1, 0, 0, 0]], np.float32))
+    p, po = params_pair(flags=ts.TS_FLAG_NORMALS if normals else 0)
+    r = ts.Rasterizer(sc.cams, M, p, pair_capacity=100_000)
+    m = ts.Map.from_numpy(sc.pos, sc.col, sc.opa)
+    r.forward(m, ts.poses_tensor(sc.poses))
+    assert r.counters()["fwd_contrib"] == M * W * H
+    dC = rng.uniform(0.5, 1.0, 3 * W * H).astype(np.float32)
+    want = oracle.backward(SceneArrays.of(sc), po, dC.astype(np.float64), np.zeros(W * H))["dcol"].T
+    err = []
+    for _ in range(4):
+        g = m.zeros_like()
+        r.forward(m, ts.poses_tensor(sc.poses))
+        r.backward(torch.as_tensor(dC, device="cuda"), torch.zeros_like(r.depth), None, g)
+        err.append(g.col.cpu().numpy().astype(np.float64) / want - 1)
+    rms = float(np.sqrt(np.mean(np.square(err))))
+    assert rms <= np.sqrt(2 * 2048 / 3) * 2.0 ** -23 * 0.72 / np.sqrt(12), rms
