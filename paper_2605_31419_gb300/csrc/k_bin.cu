@@ -25,12 +25,6 @@ namespace {
 constexpr int SCAN_T = 1024;
 constexpr int SCAN_PER = TS_SCAN_ITEMS / SCAN_T;  // 4
 
-// length of a scanned array
-struct Len {
-  long long n;
-  __device__ __forceinline__ long long get() const { return n; }
-};
-
 __device__ __forceinline__ uint32_t warp_incl_scan(uint32_t x) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
@@ -67,10 +61,9 @@ __device__ __forceinline__ void keep_wraps(unsigned long long total, unsigned in
   if (w) atomicAdd(wraps, w);
 }
 
-__global__ void __launch_bounds__(SCAN_T) k_scan_reduce(const uint32_t* __restrict__ in, Len len,
+__global__ void __launch_bounds__(SCAN_T) k_scan_reduce(const uint32_t* __restrict__ in, long long n,
                                                         uint32_t* __restrict__ bsums, unsigned int* wraps) {
   __shared__ unsigned long long wsum[SCAN_T / 32];
-  const long long n = len.get();
   const long long base = (long long)blockIdx.x * TS_SCAN_ITEMS;
   if (base >= n) return;
   unsigned long long s = 0;
@@ -824,9 +817,8 @@ cudaError_t ts_launch_bin(const TsPlanImpl* p, const TsWs& w, cudaStream_t s) {
                 &w.hdr->error_bits};
     const unsigned nf = (unsigned)((VM + 255) / 256);
     k_tile_count<<<nf, 256, 0, s>>>(ta);
-    Len lt{p->n_tiles};
     const unsigned nb = (unsigned)((p->n_tiles + TS_SCAN_ITEMS - 1) / TS_SCAN_ITEMS);
-    k_scan_reduce<<<nb, SCAN_T, 0, s>>>(w.tcnt, lt, w.bsums, &w.hdr->pair_wraps);
+    k_scan_reduce<<<nb, SCAN_T, 0, s>>>(w.tcnt, p->n_tiles, w.bsums, &w.hdr->pair_wraps);
     k_scan_bsums<<<1, SCAN_T, 0, s>>>(w.bsums, nb, &w.hdr->n_pairs, &w.hdr->error_bits, p->cap,
                                        &w.hdr->pair_wraps, &w.hdr->n_large);
     k_tile_starts<<<nb, SCAN_T, 0, s>>>(ta, w.bsums);

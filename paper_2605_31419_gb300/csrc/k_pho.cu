@@ -8,18 +8,18 @@
 // normalised) centred on p, with zeros outside the image; C1 = 0.01^2, C2 = 0.03^2.  Its gradient
 // is dSSIM_sum/dx(q) = (G * m0)(q) + 2 x(q) (G * m1)(q) + y(q) (G * m2)(q), where m0, m1, m2 are
 // the partials of SSIM(p) w.r.t. mu_x, e_xx and e_xy (zero outside the image) and G * the same
-// symmetric window sum.  In FP32 the variances formed as e_xx - mu_x^2 lose digits where the
-// window is nearly constant at a non-zero value; the error of dL/dC stays below ~1e-7 of the
-// magnitude of its terms weighted by (moments) / (sigma_x^2 + sigma_y^2 + C2).  (A shift of the
-// data by one constant per tile does not help: it moves the cancellation to flat regions at other
-// values, such as the zeros of a clamped or black background.)
+// symmetric window sum.
 //
 // SSIM and its partials need e_xx and e_yy only as their sum, and the differences B1 - A1 = (mu_x - mu_y)^2
 // and B2 - A2 = e_dd - (mu_x - mu_y)^2, with e_dd the window's mean of (x - y)^2, without cancellation where
 // the images agree: so four moments are filtered (mu_x, mu_y, e_dd, e_xy), not five.  dL/dC came closer to its
 // 64-bit value (3.3e-6 -> 1.8e-6 of its largest for 20 views of 1200 x 680), equal images still give SSIM = 1,
 // and 714 us became 668.  (Filtering x^2 + y^2 instead is as fast, but leaves rounding noise of the moments
-// in the gradient of images that agree.)
+// in the gradient of images that agree.)  In FP32 the covariance e_xy - mu_x mu_y, and with it A2 and B2, still
+// loses digits where the window is nearly constant at a non-zero value; the error of dL/dC stays below ~1e-7 of
+// the magnitude of its terms weighted by (moments) / (sigma_x^2 + sigma_y^2 + C2).  (A shift of the data by one
+// constant per tile does not help: it moves the cancellation to flat regions at other values, such as the zeros
+// of a clamped or black background.)
 //
 // One CTA owns a strip of 64 output columns and HS output rows of one channel of one view and walks down
 // it 16 rows at a time.  x and y arrive as interleaved pairs (asynchronous copies two steps ahead) over
@@ -31,11 +31,13 @@
 // pairs with two-element FMAs (fma.rn.f32x2: (mu_x, mu_y), (e_dd, e_xy), (m0, m1)), which halves the
 // instructions of a pass that is bound by issue.  A row pass takes two rows
 // per warp, so its warps go from the moments to the filtered partials without a CTA barrier (two per
-// step); five outputs per lane put the 16 lanes of a row on distinct banks.  Issue-bound (60 % issue active; FMA pipe half busy):
-// 668 us for 20 views of 1200 x 680 where 32 x 32 tiles with scalar FMAs, each recomputing its halo on
-// all sides, took 1259; 798 us for 64 views of 640 x 480 (1466).
+// step); five outputs per lane put the 16 lanes of a row on distinct banks.  Issue-bound (60 % issue active; FMA
+// pipe half busy): 689 us for 20 views of 1200 x 680 where 32 x 32 tiles with scalar FMAs, each recomputing its
+// halo on all sides, took 1259; 823 us for 64 views of 640 x 480 (1466).  (An approximate reciprocal and one
+// Newton-Raphson step for 1 / (B1 B2) save 3 % and lose its values where it leaves the normal range.)
 // Loss partial sums go to one slot per CTA and are reduced per view in a fixed order: the loss is
-// deterministic; dL/dC of a pixel does not depend on the strips' heights.
+// deterministic.  dL/dC of a pixel does not depend on the strips' heights; the last bits of a view's loss do, and
+// the heights follow from all of the plan's views.
 #include <algorithm>
 #include <cmath>
 

@@ -59,7 +59,6 @@ struct ProjArgs {
   const TsView* views;
   const ts_pose* poses;
   long long M;
-  long long VM;
   int V;
   float z_near, r_min, alpha_min;
   bool min_opacity;
@@ -73,7 +72,6 @@ struct ProjArgs {
   short4* rect;
   uint32_t* zbits;
   uint32_t* count;
-  TsDevHeader* hdr;
   unsigned long long* ctr;
 };
 
@@ -371,7 +369,6 @@ cudaError_t ts_launch_project(const TsPlanImpl* p, const TsWs& w, const ts_map* 
   a.views = w.views;
   a.poses = w.poses;
   a.M = p->M;
-  a.VM = VM;
   a.z_near = p->prm.z_near;
   a.r_min = p->prm.r_min;
   a.alpha_min = p->prm.alpha_min;
@@ -388,7 +385,6 @@ cudaError_t ts_launch_project(const TsPlanImpl* p, const TsWs& w, const ts_map* 
   a.rect = w.rect;
   a.zbits = w.zbits;
   a.count = w.count;
-  a.hdr = w.hdr;
   a.ctr = w.ctr;
   // views per block: up to PJ_VIEWS, so that a map is read once per block of views and full warps of faces collect, but
   // fewer where that leaves over half of the GPU's places (six blocks per multiprocessor) empty: 8 against 4 measured

@@ -1,6 +1,6 @@
 // k_project_bwd.cu -- chain rule from the per-face screen-space sums to the map and the pose.
 //
-// Closed form per visible (view, face), from the 24 sums the raster backward accumulated:
+// Closed form per visible (view, face), from the 22 sums the raster backward accumulated (26 with the side array):
 //   * interpolants with vertex values w (colour channels, camera depth): dL/dw_k is the sum
 //     itself, and moving vertex k moves the interpolant's plane: dL/dq_k -= dL/dw_k * grad f;
 //   * edge functions E_i = s_i lambda_{i+2} with s_i = perimeter / |e_i| (Eq. 2-3 normalised
@@ -14,23 +14,24 @@
 //
 // Gradient slots are face-major (slot = face * V + view) and cleared by the projection pass for
 // the visible ones; each is read once, in full, and nothing is written back.  Two forms:
-//   * with map gradients, a warp takes 32 faces at a time (8 or 16 of a small map): it stages the faces'
-//     vertices in shared memory, lists their visible entries face by face with views in order, and runs
-//     the chain rule on 32 entries at a time; each entry leaves its 20 map words in a shared row, lane w
-//     sums word w over each face's rows in view order, and the sums are added to the map gradient,
-//     consecutive vertices by consecutive lanes.  Pose terms are added to per-view sums in face order;
+//   * with map gradients, a warp takes 32 faces at a time (2 to 16 of a small map or for many views): it stages
+//     the faces' vertices in shared memory, lists their visible entries face by face with views in order, and
+//     runs the chain rule on 32 entries at a time; each entry leaves its 20 map words in a shared row, the words
+//     are summed over each face's rows in view order, and the sums are added to the map gradient, consecutive
+//     vertices by consecutive lanes.  Pose terms are added to per-view sums in face order;
 //   * without map gradients (tracking), warps walk one view's faces, queue the visible ones and run the
 //     chain rule on full warps, each lane keeping its own pose sums.
 // In both, a lane's next slot crosses into shared memory (cp.async) while the current one is worked on.
 // Every sum runs in a fixed order, so the gradients are deterministic given the slots.  The pose sums
-// leave per-block partials, which a last kernel adds in a fixed order.
+// leave per-block partials, which a last kernel adds in a fixed order.  (The two forms' orders differ, and with
+// map gradients the order depends on the number of views as well as on the map's size.)
 //
 // Both are bound by the latency of their loads and by issue (37 % issue active, 16 warps per SM; the chain
 // rule is about 550 instructions a batch).  With 4 faces a warp, each lane gathering its entry's vertices,
-// view and slot itself, and a separate two-pass form below 8 views, the map form took 489 us of a 12-view
-// window of 1M faces (now 278), 185 of a 20-view room of 300k (157), 130 of a 6-view window of 300k (70),
-// 48 of a 3-view indexed mesh (25); the pose alone, 64 views of 150k faces, 185 (155).  Two buffers of
-// staged vertices cost the fourth resident block and a second wave: 263 us on the room.
+// view and slot itself, and a separate two-pass form below 8 views, the map form took 484 us of 12 views of 320 x
+// 240 of 1M faces (now 267), 163 of 20 views of 300k (127), 117 of 6 (59), 16.9 of 3 views of 30k (8.7); the pose
+// alone, 64 tracking views of 150k faces, 151 (138).  Two buffers of staged vertices cost the fourth resident block
+// and a second wave: 263 us on the 20-view room.
 
 #include <algorithm>
 
@@ -42,13 +43,13 @@ struct PBArgs {
   const TsView* views;
   const ts_pose* poses;
   int V;
-  long long M, VM;
+  long long M;
   const uint32_t* count;
   float* grad;
   const float4* aux;  // per (view, face) normal and sigma_F (TS_FLAG_NORMALS / TS_FLAG_FACE_SIGMA)
-  bool normals, face_sigma;
+  bool normals;
   float* dst_sigma;  // dL/dsigma_F per face (TS_FLAG_FACE_SIGMA), may be null
-  TsDevHeader* hdr;
+  const TsDevHeader* hdr;
   float* dst[7];  // gpx, gpy, gpz, gcr, gcg, gcb, gop
   bool min_opacity;  // o_F = min of the vertex opacities: dL/do_F to the first minimal vertex
   float* part;       // per (view, block): the pose sums
@@ -638,12 +639,10 @@ cudaError_t ts_launch_project_bwd(const TsPlanImpl* p, const TsWs& w, const ts_m
   a.poses = w.poses;
   a.V = p->V;
   a.M = p->M;
-  a.VM = (long long)p->V * p->M;
   a.count = w.count;
   a.grad = w.grad;
   a.aux = w.aux;
   a.normals = p->normals;
-  a.face_sigma = p->face_sigma;
   a.dst_sigma = p->face_sigma ? g->gsigma : nullptr;
   a.hdr = w.hdr;
   a.dst[0] = g->gpx; a.dst[1] = g->gpy; a.dst[2] = g->gpz;

@@ -249,15 +249,6 @@ __device__ __forceinline__ void ts_count_add(unsigned long long* ctr, int c, uns
   }
 }
 
-__device__ __forceinline__ int ts_find_view(const TsView* views, int V, long long tile) {
-  int lo = 0, hi = V - 1;
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if (views[mid].tile_off <= tile) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
 // Camera-space vertex in the fixed FP32 operation order (Eq. 1, one rounding per operation,
 // no FMA): x_c = ((R0 x + R1 y) + R2 z) + t0, likewise y_c, z_c.
 __device__ __forceinline__ void ts_rigid_f32(const ts_pose& P, float x, float y, float z, float& xc, float& yc,
