@@ -37,7 +37,7 @@ FLOPS_PHO = 394.0
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per view of one k_render_step launch of
 # this workload, from a one-kernel, one-launch ncu capture of the same step cut to 4 views (tile
 # 16x8, 64 faces per stage), scaled by the views of the launch; reported only for that configuration
-STEP_TRAFFIC_PER_VIEW = (150.714112e6 + 77.189632e6) / 4
+STEP_TRAFFIC_PER_VIEW = (156.875776e6 + 75.447552e6) / 4
 W, H, F, N_FACES, N_VIEWS = 1200, 680, 600.0, 300_000, 20
 WORKLOAD = "room 1200x680 f=600, 300k faces, 20 poses, fwd+bwd (L1 colour+depth), batched"
 

@@ -271,15 +271,16 @@ ts_status ts_render_step_l1(const ts_plan* plan, void* ws, const float* tgt_colo
                            float* dD, const ts_map_grad* grad, ts_stream stream);
 
 /* Eq. 5-7: dL/dtau per view for the left perturbation Exp(tau) o T_CW, tau = (rho, theta), as
- * sum over the view's visible face vertices of [g_C ; v_C x g_C], reduced deterministically.
+ * sum over the view's visible face vertices of [g_C ; v_C x g_C], reduced deterministically (in an
+ * order that depends on the plan and on whether the backward had map gradients to add).
  *   dtau: device float [n_views][6], overwritten. */
 ts_status ts_pose_grad(const ts_plan* plan, void* ws, float* dtau, ts_stream stream);
 
 /* Mean-L1 colour + depth loss used by tracking and mapping (Eq. 8 L1 part, Eq. 9): per view,
  *   loss_v = sum |C - Cbar| / (3HW) + lambda_dep * sum_{Dbar > 0} |D - Dbar| / (HW),
  * with dC = dloss/dC and dD = dloss/dD (overwritten; sign(0) = 0).  All pointers device, packed
- * per view; loss: float [n_views], overwritten.  Deterministic.  Uses only the workspace's
- * partial-sum region: no earlier call on the workspace is needed.  A negative or non-finite
+ * per view; loss: float [n_views], overwritten.  Deterministic, and the same for a view alone and
+ * among others.  Uses only the workspace's partial-sum region: no earlier call on the workspace is needed.  A negative or non-finite
  * lambda_dep returns TS_ERR_INVALID_ARG. */
 ts_status ts_l1_loss(const ts_plan* plan, void* ws, const float* color, const float* depth,
                      const float* tgt_color, const float* tgt_depth, float lambda_dep, float* loss,
@@ -294,8 +295,9 @@ ts_status ts_l1_loss(const ts_plan* plan, void* ws, const float* color, const fl
  * dD = dloss/dD (overwritten; sign(0) = 0).  Pointers and packing as in ts_l1_loss; loss: device
  * float [n_views], overwritten.  lambda_ssim = 0 gives the ts_l1_loss value.  lambda_ssim outside
  * [0, 1] or a negative or non-finite lambda_dep returns TS_ERR_INVALID_ARG.  Deterministic: the
- * partial sums per image strip are reduced in a fixed order.  Like ts_l1_loss it needs no earlier
- * call on the workspace. */
+ * partial sums per image strip are reduced in a fixed order.  The strips' height follows from all of
+ * the plan's views, so the last bits of a view's loss may differ between plans; its dC and dD do not.
+ * Like ts_l1_loss it needs no earlier call on the workspace. */
 ts_status ts_pho_loss(const ts_plan* plan, void* ws, const float* color, const float* depth,
                       const float* tgt_color, const float* tgt_depth, float lambda_ssim, float lambda_dep,
                       float* loss, float* dC, float* dD, ts_stream stream);
