@@ -414,3 +414,28 @@ def test_large_faces_are_summed_in_few_additions(oracle, normals):
         err.append(g.col.cpu().numpy().astype(np.float64) / want - 1)
     rms = float(np.sqrt(np.mean(np.square(err))))
     assert rms <= np.sqrt(2 * 2048 / 3) * 2.0 ** -23 * 0.72 / np.sqrt(12), rms
+
+
+def test_photometric_loss_of_tall_strips():
+    """A batch of 80 views of 310 x 300 walks strips of 246 rows (and 54 below them) where one view alone takes
+    22: the images' gradients bit for bit, the losses to the rounding of their sums."""
+    import torch
+    import paper_2605_31419_gb300 as ts
+    W, H, V = 310, 300, 80
+    gen = torch.Generator(device="cuda").manual_seed(9)
+    C, tC = (torch.rand(V, 3 * W * H, generator=gen, device="cuda") for _ in range(2))
+    D, tD = (torch.rand(V, W * H, generator=gen, device="cuda") for _ in range(2))
+    tD[tD < 0.1] = 0.0
+
+    def run(views):
+        r = ts.Rasterizer(np.array([[50.0, 50.0, W / 2, H / 2, W, H]] * len(views)), 0)
+        r.color.copy_(C[views].reshape(-1)), r.depth.copy_(D[views].reshape(-1))
+        loss, dC, dD = r.pho_loss(tC[views].reshape(-1), tD[views].reshape(-1), 0.2)
+        return loss, dC.view(len(views), -1), dD.view(len(views), -1)
+
+    loss, dC, dD = run(list(range(V)))
+    for v in (0, 37, 79):
+        a, b, c = run([v])
+        assert torch.equal(b[0], dC[v]) and torch.equal(c[0], dD[v]), v
+        # sums of 90,000 x 3 terms: partial sums of at most 64 x 246 of them in 32 bits
+        assert abs(float(a[0]) - float(loss[v])) <= 2e-6 * abs(float(a[0]))
