@@ -44,8 +44,9 @@
 // across two quarters is left over in both and added once, and so is one from the first quarter into the last.
 // (A reduction at every quarter's end gave the slot of a large face up to four times the additions, and its sums
 // twice the rounding error: the colour gradients of two views of large faces were 1.26 times as far from their
-// 64-bit values as those of a sum per batch, now 1.01.  Putting the quarters together costs 2 to 3 % of a step:
-// 1769 -> 1810 us for the 20-view room, 1846 -> 1892 for the 12-view window.)  The reductions themselves cost
+// 64-bit values as those of a sum per batch, now 1.01.  Putting the quarters together cost 3 % of the fused pass,
+// 1438 -> 1484 us for the 20-view room; with an entry's slot checked once, where its row is written, instead of at
+// every reduction it takes 1433, the backward of 64 tracking views 709 for 688 before.)  The reductions themselves cost
 // nothing measurable; the instructions do.  (A loop over the faces' runs, one word per lane: the backward of 64
 // tracking views 1034 -> 918 us; testing every row's sums for zero and the slot in 64 bits: fused step 1321 ->
 // 1244 us for the 12-view window, backward of 6 mapping views 172 -> 164.)
@@ -730,16 +731,18 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
             }
           }
           float4* row = reinterpret_cast<float4*>(row_here);
-          if (act) {
+          // (never expected: record the fault, add nothing)
+          if (act && slot >= vm32) atomicOr(&a.hdr->error_bits, TS_ERRBIT_BOUNDS);
+          if (act && slot < vm32) {
             row[0] = make_float4(l0, l1, l2, __uint_as_float(slot));
             row[1] = make_float4(e.arg == 0 ? dm : 0.f, e.arg == 1 ? dm : 0.f, e.arg == 2 ? dm : 0.f, qC0 * w);
             row[2] = make_float4(qC1 * w, qC2 * w, qD * w, go);
             if constexpr (AUX) row[3] = make_float4(qN0 * w, qN1 * w, qN2 * w, gs);
-            ++contrib;
           } else {  // nothing to add
             row[0] = row[1] = row[2] = make_float4(0.f, 0.f, 0.f, 0.f);
             if constexpr (AUX) row[3] = make_float4(0.f, 0.f, 0.f, 0.f);
           }
+          contrib += act ? 1u : 0u;
           // the batch's faces are runs of consecutive entries.  Even quarters take their rows upwards and add a run's
           // sums at its last row, odd quarters downwards (their rows lie in that order) and at its first: a run that
           // crosses from an even quarter into the next is then left in both, and put together
@@ -754,11 +757,7 @@ __device__ __forceinline__ void bwd_tile(const RenderArgs& a, long long tile, fl
           uint32_t sl = 0u;
           auto to_slot = [&]() {
             if (fa == 7) s1 = s2 = 0.f;
-            if (sl < vm32) {
-              red_add_v4(a.grad + (size_t)sl * TS_GRAD_WORDS + 4 * fa, s0, s1, s2, s3);
-            } else {
-              atomicOr(&a.hdr->error_bits, TS_ERRBIT_BOUNDS);
-            }
+            red_add_v4(a.grad + (size_t)sl * TS_GRAD_WORDS + 4 * fa, s0, s1, s2, s3);
           };
 #pragma unroll
           for (int i = 0; i < 8; ++i) {
