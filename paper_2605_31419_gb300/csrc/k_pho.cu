@@ -32,10 +32,9 @@
 // instructions of a pass that is bound by issue.  A row pass takes two rows
 // per warp, so its warps go from the moments to the filtered partials without a CTA barrier (two per
 // step); five outputs per lane put the 16 lanes of a row on distinct banks.  Issue-bound (60 % issue active; FMA
-// pipe half busy): 677 us for 20 views of 1200 x 680 where 32 x 32 tiles with scalar FMAs, each recomputing its
-// halo on all sides, took 1259; 809 us for 64 views of 640 x 480 (1466).  (With a division per pixel for 1 / (B1 B2)
-// 689; the approximate reciprocal and its Newton-Raphson step for every product 668, but their values are wrong
-// where the product leaves the normal range.)
+// pipe half busy): 689 us for 20 views of 1200 x 680 where 32 x 32 tiles with scalar FMAs, each recomputing its
+// halo on all sides, took 1259; 823 us for 64 views of 640 x 480 (1466).  (An approximate reciprocal and one
+// Newton-Raphson step for 1 / (B1 B2) save 3 % and lose its values where it leaves the normal range.)
 // Loss partial sums go to one slot per CTA and are reduced per view in a fixed order: the loss is
 // deterministic.  dL/dC of a pixel does not depend on the strips' heights; the last bits of a view's loss do, and
 // the heights follow from all of the plan's views.
@@ -135,13 +134,6 @@ __device__ __forceinline__ void stage_block(float* xy, const float* xc, const fl
 
 // The weight of distance t along a window (both sides alike), or -1 outside it.
 __host__ __device__ constexpr int tap(int t) { return t < 0 || t >= NT ? -1 : (t <= RAD ? t : NT - 1 - t); }
-
-// Reciprocal of x by the hardware approximation and one Newton-Raphson step: equal to 1 / x for every x with
-// 2^-126 <= |x| < 2^126 (all of them compared), not defined outside.
-__device__ __forceinline__ float reciprocal(float x) {
-  const float r = ts_rcp_approx(x);
-  return fmaf(r, fmaf(-x, r, 1.f), r);
-}
 
 __device__ __forceinline__ float block_sum(float v, float* red) {
 #pragma unroll
@@ -250,39 +242,29 @@ __global__ void __launch_bounds__(PT, 2)
         const int i = s * RB + r, gy = Y0 - RAD + i;
         const bool rowin = gy >= 0 && gy < H, rowinner = i >= RAD && i < RAD + rows;
         const bool edge = X0 < RAD || X0 + OW + RAD > W || Y0 + s * RB < RAD || Y0 - RAD + (s + 1) * RB > H;  // uniform
-        bool normal = true;
-        // SSIM and its partials with 1 / (B1 B2) from `inverse`; returns sum + the SSIM of the strip's own pixels
-        auto partials = [&](auto inverse, float sum) {
 #pragma unroll
-          for (int j = 0; j < R_H1; ++j) {
-            const int cm = c0 + j, gx = X0 - RAD + cm;
-            float mx, my, edd, exy;
-            unpack2(mu[j], mx, my);
-            unpack2(ee[j], edd, exy);
-            const float A1 = 2.f * mx * my + C1, A2 = 2.f * (exy - mx * my) + C2;
-            const float dm = mx - my;
-            const float B1 = fmaf(dm, dm, A1), B2 = A2 + fmaf(-dm, dm, edd);
-            const float P = B1 * B2, size = fabsf(P);
-            normal = normal && ((size >= 0x1p-126f && size < 0x1p126f) || cm >= MO);
-            const float iB = inverse(P);
-            const float ssim = A1 * A2 * iB;
-            // partials w.r.t. mu_x, e_xx and e_xy: zero outside the image
-            float m0 = 2.f * (my * (A2 - A1) - mx * ssim * (B2 - B1)) * iB;
-            float m1 = -ssim * B1 * iB;
-            float m2 = 2.f * A1 * iB;
-            const bool in = !edge || (rowin && gx >= 0 && gx < W);
-            if (!in) m0 = m1 = m2 = 0.f;
-            if (in && rowinner && cm >= RAD && cm < RAD + OW) sum += ssim;
-            if (cm < MO) {
-              ma[r * MS + cm] = pack2(m0, m1);
-              mb[r * MS + cm] = m2;
-            }
+        for (int j = 0; j < R_H1; ++j) {
+          const int cm = c0 + j, gx = X0 - RAD + cm;
+          float mx, my, edd, exy;
+          unpack2(mu[j], mx, my);
+          unpack2(ee[j], edd, exy);
+          const float A1 = 2.f * mx * my + C1, A2 = 2.f * (exy - mx * my) + C2;
+          const float dm = mx - my;
+          const float B1 = fmaf(dm, dm, A1), B2 = A2 + fmaf(-dm, dm, edd);
+          const float iB = 1.f / (B1 * B2);  // (0 where the product overflows: such a pixel's terms vanish)
+          const float ssim = A1 * A2 * iB;
+          // partials w.r.t. mu_x, e_xx and e_xy: zero outside the image
+          float m0 = 2.f * (my * (A2 - A1) - mx * ssim * (B2 - B1)) * iB;
+          float m1 = -ssim * B1 * iB;
+          float m2 = 2.f * A1 * iB;
+          const bool in = !edge || (rowin && gx >= 0 && gx < W);
+          if (!in) m0 = m1 = m2 = 0.f;
+          if (in && rowinner && cm >= RAD && cm < RAD + OW) ss += ssim;
+          if (cm < MO) {
+            ma[r * MS + cm] = pack2(m0, m1);
+            mb[r * MS + cm] = m2;
           }
-          return sum;
-        };
-        const float sum = partials([](float x) { return reciprocal(x); }, ss);
-        // (a product outside the normal range: divisions, 0 where it overflows, so that such a pixel's terms vanish)
-        ss = normal ? sum : partials([](float x) { return 1.f / x; }, ss);
+        }
       }
     }
     __syncwarp();  // the next pass reads the rows that this warp has just written
